@@ -17,7 +17,7 @@
 
 namespace molt {
 
-struct BatchSweep {
+struct alignas(16) BatchSweep {
   SweepArgs a;       // geometry, coefficients and tile shape of one (problem, axis)
   int E;             // points per lane (4, 8 or 16)
   int first_item;    // first work item of this problem in the phase
@@ -25,7 +25,8 @@ struct BatchSweep {
 };
 
 struct BatchUpdate {
-  const float* acc;
+  const float* acc;  // S of x
+  const float* accy; // S of y
   double* u;         // u^n
   double* st1;       // stage states
   double* st2;
@@ -48,77 +49,25 @@ struct BatchParams {
   int* status;
   long long wait_limit;       // cycles
   int skip_arrive;            // test hook: CTA 0 never arrives at the first barrier
-  unsigned int stage_off;     // shared-memory offset of the tile staging buffer
+  unsigned int buf_bytes;     // shared bytes of one of the two tile buffers
 };
 
-// Staging buffer of one tile's raw input (W lines x n points, FP32): the
-// asynchronous copy of a CTA's next tile lands here while the current tile
-// is computed.
-constexpr int kStageFloats = 512 * 16;   // W * n = 512 * E <= 8192
+constexpr size_t kBatchHead = 128;   // shared bytes of the warps' totals (16 warps)
+static_assert(tile_head_bytes(1, 16, 4) <= kBatchHead, "totals of 16 warps");
 
-// 16-byte asynchronous copy through L2 only (.cg): the sweep inputs were
-// written earlier in the same launch by other CTAs, so no L1 line may serve
-// them.
-__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
+// 4-byte asynchronous copy: the tile's values land in the padded layout of
+// the compute core with no pass of their own.  (The inputs were written
+// earlier in the launch by other CTAs; the grid barrier's fences order them.)
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+  const unsigned int d = static_cast<unsigned int>(__cvta_generic_to_shared(dst));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   const unsigned int d = static_cast<unsigned int>(__cvta_generic_to_shared(dst));
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// Issues the copy of the tile starting at line0 into the staging buffer:
-// contiguous lines as [w][n], strided lines as [p][W].  Batch tiles are exact
-// fits (n a multiple of 128, the line count a multiple of W), so contiguous
-// rows and strided rows of W >= 4 floats move as asynchronous 16-byte
-// pieces; rows of one or two floats are loaded synchronously (through L2).
-// log2 of a power of two
-__device__ __forceinline__ int ilog2(int v) { return 31 - __clz(v); }
-
-__device__ __forceinline__ void stage_tile(const SweepArgs& a, float* stage, long long line0) {
-  const float* in = static_cast<const float*>(a.in);
-  const int n = a.g.n, W = a.W;          // powers of two in batch tiles
-  const int ln = ilog2(n), lW = ilog2(W);
-  if (a.contiguous) {
-    const int lc = ln - 2;               // 16-byte chunks per line
-    for (int t = threadIdx.x; t < W << lc; t += blockDim.x) {
-      const int w = t >> lc, c = t & ((1 << lc) - 1);
-      if (line0 + w < a.g.nlines) cp_async16(stage + (w << ln) + 4 * c, in + line_base(a.g, line0 + w) + 4 * c);
-    }
-  } else if (line0 < a.g.nlines) {
-    const long long b0 = line_base(a.g, line0);
-    if (W >= 4) {
-      const int lp = lW - 2;             // 16-byte pieces per row
-      for (int t = threadIdx.x; t < n << lp; t += blockDim.x) {
-        const int q = t >> lp, c = t & ((1 << lp) - 1);
-        cp_async16(stage + (q << lW) + 4 * c, in + b0 + q * a.g.stride + 4 * c);
-      }
-    } else {
-      for (int t = threadIdx.x; t < n << lW; t += blockDim.x) {
-        const int q = t >> lW, w = t & (W - 1);
-        stage[t] = __ldcg(in + b0 + q * a.g.stride + w);
-      }
-    }
-  }
-  cp_async_commit();
-}
-
-// Staging layout -> padded per-line layout of the compute core.
-template <int E>
-__device__ __forceinline__ void unstage_tile(const SweepArgs& a, const float* stage, float* lines) {
-  const int n = a.g.n, W = a.W;
-  const int ln = ilog2(n), lW = ilog2(W);
-  if (a.contiguous) {
-    for (int t = threadIdx.x; t < W << ln; t += blockDim.x) {
-      const int w = t >> ln, q = t & (n - 1);
-      lines[w * a.LS + phys<E>(q)] = stage[t];
-    }
-  } else {
-    for (int t = threadIdx.x; t < n << lW; t += blockDim.x) {
-      const int q = t >> lW, w = t & (W - 1);
-      lines[w * a.LS + phys<E>(q)] = stage[t];
-    }
-  }
-}
 
 #ifndef MOLT_BATCH_CHUNK
 #define MOLT_BATCH_CHUNK 4096
@@ -161,50 +110,42 @@ __device__ __forceinline__ bool grid_sync(const BatchParams& p, bool skip) {
   return ok != 0;
 }
 
-// One (problem, line tile) work item: the tile shape fills the CTA exactly
-// (32 * nwl * W == blockDim.x) and the lines are an exact fit (n = 32*nwl*E).
-// The tile's input is in the staging buffer (copy complete and visible); the
-// copy of the next tile (if any) is issued once the buffer has been read.
-template <int E>
-__device__ __forceinline__ void batch_tile(const SweepArgs& a, const TileSmem& sm, long long line0, int ax,
-                                           float* stage, const SweepArgs* next, long long next_line0) {
-  float* lines = static_cast<float*>(sm.lines);
+// Starts the copy of one (problem, line tile) work item into shared memory:
+// its arguments and its lines.  The tile shape fills the CTA exactly (32 * nwl
+// * W == blockDim.x) and the lines are an exact fit (n = 32*nwl*E).
+__device__ __forceinline__ void batch_fetch(const BatchSweep& bs, BatchSweep* args, float* lines, long long item) {
+  const SweepArgs& a = bs.a;
+  const char* src = reinterpret_cast<const char*>(&bs);
+  char* dst = reinterpret_cast<char*>(args);
+  for (int c = threadIdx.x; c < int(sizeof(BatchSweep) / 16); c += blockDim.x) cp_async16(dst + 16 * c, src + 16 * c);
+  const long long line0 = (item - bs.first_item) * a.W;
   const int warp = threadIdx.x >> 5, lw = warp / a.nwl;
-  unstage_tile<E>(a, stage, lines);
-  __syncthreads();
-  if (next) stage_tile(*next, stage, next_line0);
-  compute_lines_any<float, false, false, E>(a, sm, line0 + lw < a.g.nlines);
-  if (ax == 0) epilogue_tile<float, double, EPI_ACC_SET, E, true>(a, lines, line0, 0.0);
-  else epilogue_tile<float, double, EPI_ACC_ADD, E, true>(a, lines, line0, 0.0);
-  __syncthreads();
+  const int tl = (warp - lw * a.nwl) * 32 + (threadIdx.x & 31);
+  const float* in = static_cast<const float*>(a.in);
+  auto put = [](float* d, const float* g) { cp_async4(d, g); };
+  if (bs.E == 16) load_tile<float, float, 16>(a, in, lines, line0, lw, tl, put);
+  else if (bs.E == 8) load_tile<float, float, 8>(a, in, lines, line0, lw, tl, put);
+  else load_tile<float, float, 4>(a, in, lines, line0, lw, tl, put);
+  cp_async_commit();
 }
 
-// L2 prefetch of the accumulator a y-phase tile's epilogue reads, issued for
-// the CTA's next work item before the current one is computed.  One request
-// per 128-byte segment (contiguous lines) or per row (strided lines).
-__device__ __forceinline__ void prefetch_acc(const SweepArgs& a, long long line0) {
-  const LineGeom& g = a.g;
-  const int n = g.n, W = a.W;
-  const char* acc = static_cast<const char*>(a.acc);
-  if (a.contiguous) {
-    const int nseg = (n + 31) / 32;
-    for (int t = threadIdx.x; t < W * nseg; t += blockDim.x) {
-      const int w = t / nseg, sg = t - w * nseg;
-      if (line0 + w < g.nlines) prefetch_l2(acc + (line_base(g, line0 + w) + 32LL * sg) * 4);
-    }
-  } else if (line0 < g.nlines) {
-    const long long b0 = line_base(g, line0);
-    for (int q = threadIdx.x; q < n; q += blockDim.x) prefetch_l2(acc + (b0 + q * g.stride) * 4);
-  }
+template <int E>
+__device__ __forceinline__ void batch_tile(const SweepArgs& a, const TileSmem& sm, long long line0) {
+  const int lw = (threadIdx.x >> 5) / a.nwl;
+  compute_lines<float, JQ_D0, false, E>(a, sm, line0 + lw < a.g.nlines);
+  epilogue_tile<float, double, EPI_ACC_SET, E, true>(a, static_cast<const float*>(sm.lines), line0, 0.0);
 }
 
-__device__ __forceinline__ int find_problem(const BatchParams& p, long long item, int ax) {
-  int lo = 0, hi = p.nprob - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (p.sweeps[mid * 2 + ax].first_item <= item) lo = mid; else hi = mid - 1;
+// Problem of a work item, by one warp (the items of problem k start at
+// first_item): lanes compare 32 problems at a time.
+__device__ __forceinline__ int find_problem(const BatchParams& p, long long item, int ax, int lane) {
+  int count = 0;
+  for (int k0 = 0; k0 < p.nprob; k0 += 32) {
+    const int k = k0 + lane;
+    const bool le = k < p.nprob && p.sweeps[k * 2 + ax].first_item <= item;
+    count += __popc(__ballot_sync(0xffffffffu, le));
   }
-  return lo;
+  return count - 1;
 }
 
 __device__ __forceinline__ int find_update(const BatchParams& p, long long chunk) {
@@ -229,44 +170,50 @@ __global__ void batch_heat_kernel(const BatchParams p);
 #else
 __global__ void __launch_bounds__(512, MOLT_BATCH_MIN_BLOCKS) batch_heat_kernel(const BatchParams p) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ SweepArgs sa;
-  __shared__ int s_prob, s_tile, s_nprob, s_ntile;
+  __shared__ BatchSweep sa[2];
+  __shared__ int s_prob[3];   // problem of this item, the next and the one after (rotating)
   static const double rk[3][2] = {{0.0, 1.0}, {0.75, 0.25}, {1.0 / 3.0, 2.0 / 3.0}};
+  const int lane = threadIdx.x & 31;
+  float* buf[2] = {reinterpret_cast<float*>(smem_raw + kBatchHead),
+                   reinterpret_cast<float*>(smem_raw + kBatchHead + p.buf_bytes)};
   bool first = true;
   for (int s = 0; s < p.stages; ++s) {
     for (int ax = 0; ax < 2; ++ax) {
       if (p.phase_mask & (1 << ax)) {
-        float* stage = reinterpret_cast<float*>(smem_raw + p.stage_off);
-        if (blockIdx.x < p.items[ax]) {
-          const int p0 = find_problem(p, blockIdx.x, ax);
-          const SweepArgs& a0 = p.sweeps[p0 * 2 + ax].a;
-          stage_tile(a0, stage, (long long)(blockIdx.x - p.sweeps[p0 * 2 + ax].first_item) * a0.W);
-        }
-        for (long long item = blockIdx.x; item < p.items[ax]; item += gridDim.x) {
-          if (threadIdx.x == 0) {
-            s_prob = find_problem(p, item, ax);
-            s_tile = int(item - p.sweeps[s_prob * 2 + ax].first_item);
-            const long long nx = item + gridDim.x;
-            s_nprob = nx < p.items[ax] ? find_problem(p, nx, ax) : -1;
-            if (s_nprob >= 0) s_ntile = int(nx - p.sweeps[s_nprob * 2 + ax].first_item);
+        // the CTA's items: while one is computed, the next one's lines and
+        // arguments arrive in the other buffer and warp 0 looks up the
+        // problem of the one after
+        const long long step = gridDim.x;
+        if (threadIdx.x < 32) {
+          const int p0 = find_problem(p, blockIdx.x, ax, lane), p1 = find_problem(p, blockIdx.x + step, ax, lane);
+          if (lane == 0) {
+            s_prob[0] = p0;
+            s_prob[1] = p1;
           }
+        }
+        __syncthreads();
+        if (blockIdx.x < p.items[ax]) batch_fetch(p.sweeps[s_prob[0] * 2 + ax], &sa[0], buf[0], blockIdx.x);
+        int cur = 0, slot = 0;
+        for (long long item = blockIdx.x; item < p.items[ax]; item += step) {
           cp_async_wait_all();
-          __syncthreads();
-          const SweepArgs* na = s_nprob >= 0 ? &p.sweeps[s_nprob * 2 + ax].a : nullptr;
-          const long long nline0 = na ? (long long)s_ntile * na->W : 0;
-          if (na && ax == 1) prefetch_acc(*na, nline0);
-          const BatchSweep* bs = p.sweeps + s_prob * 2 + ax;
-          const int* src = reinterpret_cast<const int*>(&bs->a);
-          int* dst = reinterpret_cast<int*>(&sa);
-          for (int w = threadIdx.x; w < int(sizeof(SweepArgs) / 4); w += blockDim.x) dst[w] = src[w];
-          const int E = bs->E;
-          __syncthreads();
-          size_t used;
-          const TileSmem sm = carve<float>(smem_raw, sa, &used);
-          const long long line0 = (long long)s_tile * sa.W;
-          if (E == 16) batch_tile<16>(sa, sm, line0, ax, stage, na, nline0);
-          else if (E == 8) batch_tile<8>(sa, sm, line0, ax, stage, na, nline0);
-          else batch_tile<4>(sa, sm, line0, ax, stage, na, nline0);
+          __syncthreads();   // the item is in place; the other buffer's readers are done
+          const int s1 = slot == 2 ? 0 : slot + 1, s2 = s1 == 2 ? 0 : s1 + 1;
+          if (item + step < p.items[ax])
+            batch_fetch(p.sweeps[s_prob[s1] * 2 + ax], &sa[cur ^ 1], buf[cur ^ 1], item + step);
+          if (threadIdx.x < 32) {
+            const int p2 = find_problem(p, item + 2 * step, ax, lane);
+            if (lane == 0) s_prob[s2] = p2;
+          }
+          const BatchSweep& bs = sa[cur];
+          TileSmem sm{};
+          sm.totals = smem_raw;
+          sm.lines = buf[cur];
+          const long long line0 = (item - bs.first_item) * bs.a.W;
+          if (bs.E == 16) batch_tile<16>(bs.a, sm, line0);
+          else if (bs.E == 8) batch_tile<8>(bs.a, sm, line0);
+          else batch_tile<4>(bs.a, sm, line0);
+          cur ^= 1;
+          slot = s1;
         }
       }
       const bool skip = first && p.skip_arrive && blockIdx.x == 0;
@@ -298,6 +245,7 @@ __global__ void __launch_bounds__(512, MOLT_BATCH_MIN_BLOCKS) batch_heat_kernel(
                 prefetch_l2(j + 8 < j1 ? vs + j + 8 : vs + j);
               }
               prefetch_l2(V.acc + j);
+              prefetch_l2(V.accy + j);
             }
           }
         }
@@ -305,7 +253,7 @@ __global__ void __launch_bounds__(512, MOLT_BATCH_MIN_BLOCKS) batch_heat_kernel(
         // CTA is the SM's only one, so memory parallelism comes from here)
         constexpr int kPer = kChunk / 512;
         double uu[kPer], ss[kPer];
-        float aa[kPer];
+        float aa[kPer], ay[kPer];
 #pragma unroll
         for (int k = 0; k < kPer; ++k) {
           const long long i = i0 + threadIdx.x + (long long)k * blockDim.x;
@@ -313,13 +261,16 @@ __global__ void __launch_bounds__(512, MOLT_BATCH_MIN_BLOCKS) batch_heat_kernel(
             uu[k] = __ldcg(U.u + i);
             ss[k] = __ldcg(us + i);
             aa[k] = __ldcg(U.acc + i);
+            ay[k] = __ldcg(U.accy + i);
           }
         }
 #pragma unroll
         for (int k = 0; k < kPer; ++k) {
           const long long i = i0 + threadIdx.x + (long long)k * blockDim.x;
           if (i < i1) {
-            const double r = fma(a0, uu[k], a1 * fma(p.coefS, f2d(aa[k]), ss[k]));
+            // the axis sums meet in FP64: no FP32 rounding at their joint size
+            const double t = fma(p.coefS, f2d(aa[k]), fma(p.coefS, f2d(ay[k]), ss[k]));
+            const double r = s == 0 ? t : fma(a0, uu[k], a1 * t);
             dstp[i] = r;
             U.copy[i] = d2f(r);
             bad |= nonfinite(r);

@@ -10,75 +10,90 @@
 namespace molt {
 
 // Fills the weight and decay fields of `a` for lines of N intervals and E
-// points per lane.  FP64 sweeps take the table as it is.  FP32 sweeps run
-// their recurrences with q rounded to FP32 (q32); every constant they meet is
-// made consistent with that ratio:
-//   * the FP64 boundary constants use powers of q32 (mu = q32^N, ...), so the
-//     periodic image sum and the Dirichlet solve close the recurrences the
-//     kernel actually ran;
-//   * each rule's FP32 weights are rescaled to sum to 1 - q32 (the moment
-//     identity sum_l c_l = 1 - e^{-nu}, App. C), the last rounding residual
-//     moved onto the largest weight, so that D[const] = 0 holds in the FP32
-//     arithmetic.  Without this, the relative rounding of 1 - q32 (about
-//     1e-6 at nu = 0.03) shifts the symbol of D by that amount at every
-//     frequency, a systematic damping that a long run accumulates;
-//   * alpha in FP32 (one-sided derivatives alpha D) is alpha * nu32 / nu.
-#ifndef MOLT_FIT_F32_WEIGHTS
-#define MOLT_FIT_F32_WEIGHTS 1
-#endif
+// points per lane (a.g.n, a.bc and a.mode set).  FP32 sweeps run their scans
+// with q rounded to FP32 (q32): the powers and boundary constants they meet
+// are those of that ratio, so that the periodic image sum and the Dirichlet
+// solve close the recurrences the kernel actually runs.  Every form takes
+// differences of v, so D of a constant is exactly zero at any rounding.
+//   b[]     K_R(x_i) = sum_m b_m d_{i+m}, m = -2..2 (weights summing to 1 - q)
+//   f0, f1, kap   the residual form of D_0: with N(z) = (1-q/z)(1-qz) -
+//     [J(z)(1-qz) + J(1/z)(1-q/z)]/2 = delta^2 (a0 + a1 (z+1/z) + a2 (z^2+1/z^2))
+//     and x = delta^2 = z - 2 + 1/z, M(x) = M0 + M1 x + M2 x^2 is divided by
+//     (1-q)^2 - q x: M = (Q0 + Q1 x)((1-q)^2 - q x) + rho, and
+//     U + V = -(1+q) delta^2 v / ((1-q)^2 - q x) gives kap = -rho/(1+q),
+//     f0 = Q0 - 2 Q1, f1 = Q1.  Q0 and Q1 are small (below 0.03 up to nu = 1.2)
+//     and grow like e^{3 nu}; past kResidualMax their cancellation against
+//     kap (U + V) would show in the last digits, and the K filters run.
+constexpr double kResidualMax = 0.125;
 inline void set_line_constants(SweepArgs& a, const QuadTable& qt, int N, int E, bool f32_sweeps) {
-  const bool f32 = f32_sweeps && MOLT_FIT_F32_WEIGHTS;
-  for (int i = 0; i < 6; ++i) a.c[i] = qt.c[i];
-  for (int r = 0; r < 3; ++r) {
-    for (int j = 0; j < 4; ++j) a.sub[r][j] = qt.sub[r][j];
-    a.d[r] = qt.d[r];
+  const double nu = qt.nu, qx = qt.q;
+  const double* c = qt.c;
+  // difference taps
+  const double b[5] = {c[0], c[0] + c[1], c[0] + c[1] + c[2] + qx, -(c[4] + c[5]), -c[5]};
+  for (int i = 0; i < 5; ++i) a.b[i] = b[i];
+  // residual form of D_0
+  auto cc = [c](int m) { return m >= -3 && m <= 2 ? c[m + 3] : 0.0; };
+  double h[4];
+  for (int m = 0; m < 4; ++m) h[m] = 0.5 * (cc(m) - qx * cc(m - 1) + cc(-m) - qx * cc(-m - 1));
+  const double n1 = -qx - h[1], n2 = -h[2], n3 = -h[3];
+  const double a0 = n1 + 2.0 * n2 + 3.0 * n3, a1 = n2 + 2.0 * n3, a2 = n3;
+  const double M0 = a0 + 2.0 * a1 + 2.0 * a2, M1 = a1 + 4.0 * a2, M2 = a2;
+  const double p = -std::expm1(-nu), xs = p * p / qx;
+  const double Q1 = -M2 / qx, Q0 = (Q1 * p * p - M1) / qx;
+  a.f0 = Q0 - 2.0 * Q1;
+  a.f1 = Q1;
+  a.kap = -(M0 + xs * (M1 + xs * M2)) / (1.0 + qx);
+  a.d0 = std::fabs(Q0) + std::fabs(Q1) <= kResidualMax ? 1 : 0;   // NaN: the K filters
+  if (!a.d0) {
+    a.f0 = a.f1 = 0.0;
+    a.kap = 0.5;
   }
-  double q = qt.q, lq = -qt.nu;   // lq = log q
-  if (f32) {
-    q = double(float(qt.q));
-    lq = std::log(q);
+  // WENO-Z substencil rules on the differences (csrc/sweep.cuh, wenoz_defect)
+  a.wk[0] = qt.sub[0][0] + qt.sub[0][1];
+  a.wk[1] = qt.sub[0][0];
+  a.wk[2] = 1.0 - qt.sub[1][2];
+  a.wk[3] = qt.sub[1][0];
+  a.wk[4] = qt.sub[2][0] + qx;
+  a.wk[5] = -qt.sub[2][2];
+  for (int r = 0; r < 3; ++r) a.d[r] = qt.d[r];
+  // decays
+  // (clamped where q vanishes beside 1 in the arithmetic: 1/q stays finite)
+  double lq = std::fmax(f32_sweeps ? std::log(double(float(qx))) : -nu, f32_sweeps ? -40.0 : -300.0);
+  double pw = 1.0;
+  for (int k = 0; k < 13; ++k, pw *= 2.0) a.qp[k] = std::exp(lq * pw);
+  const int n = a.g.n, span = 32 * E;
+  a.qlast = std::exp(lq * double((n - 1) % E + 1));
+  a.qlw = std::exp(lq * double((n - 1) % span + 1));
+  // boundary constants (Sec. 2.3, 3.3), of scans whose first position adds
+  // its decay: periodic C = T/(1 - mu); D_0 between Dirichlet walls from the
+  // 2x2 system with determinant 1 - mu^2; one-sided Dirichlet D start from 0
+  a.kA = a.kB = 0.0;
+  a.close = 0;
+  if (a.bc == 0) {
+    a.kA = 1.0 / (-std::expm1(lq * double(N)));
+    a.close = 1;
+  } else if (a.mode == MODE_0) {
+    const double k = std::exp(-lq) / (-std::expm1(2.0 * lq * double(N)));
+    a.kA = std::exp(lq * double(N)) * k;
+    a.kB = -k;
+    a.close = 2;
   }
-  a.q = q;
-  a.qE = std::exp(lq * double(E));
-  a.invq = std::exp(-lq);
-  a.mu = std::exp(lq * double(N));
-  a.inv1mmu = 1.0 / (-std::expm1(lq * double(N)));
-  a.invdet = 1.0 / (-std::expm1(2.0 * lq * double(N)));
-  a.k2det = 2.0 * a.invdet;
-  a.k2detq = a.k2det * a.invq;
-  a.qf = float(q);
-  a.qEf = float(a.qE);
-  a.alphaf = float(f32 ? a.alpha * (-lq) / qt.nu : a.alpha);
-  // FP32 weights summing to 1 - q32 (exact in FP64: q32 is a float)
-  const double target = 1.0 - q;
-  auto fit = [target](const double* c, int n, float* out) {
-    double s = 0.0;
-    for (int i = 0; i < n; ++i) s += c[i];
-    int imax = 0;
-    for (int i = 0; i < n; ++i) {
-      out[i] = float(s != 0.0 ? c[i] * (target / s) : c[i]);
-      if (std::fabs(c[i]) > std::fabs(c[imax])) imax = i;
-    }
-    double got = 0.0;
-    for (int i = 0; i < n; ++i) got += double(out[i]);
-    out[imax] = float(double(out[imax]) + (target - got));
-  };
-  if (f32) {
-    fit(qt.c, 6, a.cf);
-    // the FP32 kernels read three substencil taps (the 5-point rule's)
-    for (int r = 0; r < 3; ++r) {
-      if (qt.npts == 5) {
-        fit(qt.sub[r], 3, a.subf[r]);
-      } else {
-        for (int j = 0; j < 3; ++j) a.subf[r][j] = float(qt.sub[r][j]);
-      }
-    }
-  } else {
-    for (int i = 0; i < 6; ++i) a.cf[i] = float(qt.c[i]);
-    for (int r = 0; r < 3; ++r)
-      for (int j = 0; j < 3; ++j) a.subf[r][j] = float(qt.sub[r][j]);
-  }
-  for (int r = 0; r < 3; ++r) a.df[r] = float(qt.d[r]);
+  a.kAh = float(a.kA);
+  a.kAl = float(a.kA - double(a.kAh));
+  a.kBh = float(a.kB);
+  a.kBl = float(a.kB - double(a.kBh));
+  // FP32 copies
+  for (int i = 0; i < 5; ++i) a.bf[i] = float(a.b[i]);
+  a.f0f = float(a.f0);
+  a.f1f = float(a.f1);
+  a.kapf = float(a.kap);
+  for (int i = 0; i < 6; ++i) a.wkf[i] = float(a.wk[i]);
+  for (int r = 0; r < 3; ++r) a.df[r] = float(a.d[r]);
+  for (int k = 0; k < 13; ++k) a.qpf[k] = float(a.qp[k]);
+  a.qlastf = float(a.qlast);
+  a.qlwf = float(a.qlw);
+  // one-sided derivatives alpha D: D carries the factor (1-q)/(1-q32)
+  a.alphaf = float(f32_sweeps ? a.alpha * std::expm1(lq) / std::expm1(-nu) : a.alpha);
 }
 
 }  // namespace molt

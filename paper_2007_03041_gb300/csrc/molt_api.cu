@@ -58,6 +58,7 @@ struct Problem {
   mutable NuCache nu[3];
   mutable void* nu_tmp[2] = {nullptr, nullptr};   // transposed copies for strided non-uniform 2-D sweeps
   mutable void* nu_sum = nullptr;                 // S of one axis in the compute type (molt_step)
+  void* accy = nullptr;     // batched heat: the y sums (FP32)
   void* acc2 = nullptr;     // heat with concurrent axes: the y (and z) sums (compute type)
   int64_t hj_steps = 0;     // HJ steps taken (rotates the speed slots)
   bool hj_lag_ready = false;
@@ -235,8 +236,8 @@ int device_sms() {
 }
 
 // Points per lane for a line of n points: the largest of 16, 8, 4 whose
-// tile fits the line exactly (n = 32 * E * nwl, nwl <= 16 warps), else 16
-// with masked (ragged) tiles.  FP64 sweeps of grids with few lines (fewer
+// tile fits the line exactly (n = 32 * E * nwl, nwl <= 16 warps), else
+// masked (ragged) tiles of the shape with the least work.  FP64 sweeps of grids with few lines (fewer
 // than 16 warps per SM at that E; nlines counts the lines of every sweep
 // running at the same time) are bound by the latency of their recurrences
 // on the FP64 pipe, not by bandwidth, and take a shorter chain per lane:
@@ -259,6 +260,7 @@ int device_sms() {
 #define MOLT_SMALL_TILE_THREADS 256
 #endif
 constexpr int kSmallTileThreads = MOLT_SMALL_TILE_THREADS;
+constexpr int kStridedRowBytes = 32;
 
 int choose_E(int n, bool f64, long long nlines) {
   auto fits = [n](int E) { return n % (32 * E) == 0 && n / (32 * E) <= kMaxThreads / 32; };
@@ -266,7 +268,19 @@ int choose_E(int n, bool f64, long long nlines) {
   int first = 0;
   for (int i = 0; i < 4 && !first; ++i)
     if (fits(kOrder[i])) first = kOrder[i];
-  if (!first) return kE;
+  if (!first) {
+    // ragged lines: the shape with the least work, nwl warps of E points a
+    // lane plus a scan worth 4 points (FP64: 2); 16 unless another saves 15%
+    // (lanes past the end of a line cost as much as the others: 201 points
+    // fill 39% of a 16-point tile and 79% of an 8-point one)
+    const int extra = f64 ? 2 : 4;
+    auto cost = [n, extra](int E) { return (n + 32 * E - 1) / (32 * E) * (E + extra); };
+    int best = kE;
+    for (int E : {8, 4})
+      if ((n + 32 * E - 1) / (32 * E) <= kMaxThreads / 32 && 100 * cost(E) < 85 * cost(kE) && cost(E) < cost(best))
+        best = E;
+    return best;
+  }
   const long long sms = device_sms();
   if (f64 && MOLT_F64_SMALL_E && nlines * (n / (32 * first)) < 16 * sms) {
     int smallest = 0;
@@ -318,12 +332,14 @@ molt_status plan_axis(molt_ctx* c, const Problem& p, int ax, int mode, int P, do
   // tile shape: nwl warps per line, W lines per CTA, <= kMaxThreads threads
   const int nwl = (n + 32 * E - 1) / (32 * E);
   if (nwl > kMaxThreads / 32) return fail(c, MOLT_EUNSUPPORTED, "line longer than 8192 points");
-  // contiguous lines: tiles of at most kSmallTileThreads threads where a line
-  // fits in them, so the register-heavy sweeps (128 per thread) keep two CTAs
-  // per SM and one computes while the other waits at a barrier (strided lines
-  // keep the wider tiles: their W lines are the width of every row they read)
-  const int tmax =
-      (auto_shape && a.contiguous && nwl * 32 <= kSmallTileThreads) ? kSmallTileThreads : kMaxThreads;
+  // tiles of at most kSmallTileThreads threads where a line fits in them, so
+  // the register-heavy sweeps (128 per thread) keep two CTAs per SM and one
+  // computes while the other waits at a barrier; strided lines (their W lines
+  // are the width of every row they read) as long as a row fills a 32-byte
+  // sector (201 x 151 x 101 wave steps: 0.91 -> 0.81 ms), else the wider tiles
+  const int row = kSmallTileThreads / 32 / nwl * int(compute_bytes(p.d));   // bytes of a strided tile's row
+  const int tmax = (auto_shape && nwl * 32 <= kSmallTileThreads && (a.contiguous || row >= kStridedRowBytes))
+                       ? kSmallTileThreads : kMaxThreads;
   int W = (tmax / 32) / nwl;
   int Wp = 1;
   while (Wp * 2 <= W) Wp *= 2;
@@ -338,8 +354,7 @@ molt_status plan_axis(molt_ctx* c, const Problem& p, int ax, int mode, int P, do
   a.nwl = nwl;
   a.LS = LS;
   const size_t tb = compute_bytes(p.d);
-  size_t off = (size_t(4 * W) * 8 + size_t(W * nwl * 4) * tb + 15) & ~size_t(15);
-  out->smem = off + size_t(W) * LS * tb;
+  out->smem = tile_head_bytes(W, nwl, tb) + size_t(W) * LS * tb;
   if (a.two_out) out->smem += 16 + size_t(W) * LS * tb;   // second line buffer (carve order)
   if (p.d.weights == MOLT_W_LEARNED) {
     if (!c->mlp_ready) return fail(c, MOLT_EINVAL, "learned weights: call molt_set_mlp first");
@@ -419,67 +434,91 @@ void plan_tma(const Problem& p, int ax, const void* in, size_t in_bytes, Plan* p
 
 #define TMA (pl.use_tma ? &pl.tma : nullptr)
 
+// Kind of the sweep kernel: D_0 with linear weights, one side alone, or both.
+int jquad(const molt_desc& d, int mode) {
+  if (d.weights == MOLT_W_LEARNED) return JQ_LEARNED;
+  const bool one = mode == MODE_R || mode == MODE_L, wz = d.weights == MOLT_W_WENOZ;
+  if (one) return wz ? JQ_WENOZ1 : JQ_LINEAR1;
+  return wz ? JQ_WENOZ : (mode == MODE_0 ? JQ_D0 : JQ_LINEAR);
+}
+
+#define SWEEP(JQ, EPI) return launch_sweep<T, TIN, TST, JQ, EPI>(pl.a, TMA, pl.grid, pl.block, pl.smem, s)
+
 template <typename T, typename TIN, typename TST>
-cudaError_t dispatch_lin(int epi, const Plan& pl, cudaStream_t s) {
-  const SweepArgs& a = pl.a;
+cudaError_t dispatch_d0(int epi, const Plan& pl, cudaStream_t s) {
   switch (epi) {
-    case EPI_STORE: return launch_sweep<T, TIN, TST, JQ_LINEAR, EPI_STORE>(a, TMA, pl.grid, pl.block, pl.smem, s);
-    case EPI_ACC_SET: return launch_sweep<T, TIN, TST, JQ_LINEAR, EPI_ACC_SET>(a, TMA, pl.grid, pl.block, pl.smem, s);
-    case EPI_ACC_ADD: return launch_sweep<T, TIN, TST, JQ_LINEAR, EPI_ACC_ADD>(a, TMA, pl.grid, pl.block, pl.smem, s);
-    case EPI_HEAT_FINAL: return launch_sweep<T, TIN, TST, JQ_LINEAR, EPI_HEAT_FINAL>(a, TMA, pl.grid, pl.block, pl.smem, s);
-    case EPI_WAVE_FINAL: return launch_sweep<T, TIN, TST, JQ_LINEAR, EPI_WAVE_FINAL>(a, TMA, pl.grid, pl.block, pl.smem, s);
-    case EPI_ACC_AXPY: return launch_sweep<T, TIN, TST, JQ_LINEAR, EPI_ACC_AXPY>(a, TMA, pl.grid, pl.block, pl.smem, s);
+    case EPI_STORE: SWEEP(JQ_D0, EPI_STORE);
+    case EPI_ACC_SET: SWEEP(JQ_D0, EPI_ACC_SET);
+    case EPI_ACC_ADD: SWEEP(JQ_D0, EPI_ACC_ADD);
+    case EPI_HEAT_FINAL: SWEEP(JQ_D0, EPI_HEAT_FINAL);
+    case EPI_WAVE_FINAL: SWEEP(JQ_D0, EPI_WAVE_FINAL);
+    case EPI_ACC_AXPY: SWEEP(JQ_D0, EPI_ACC_AXPY);
     default: return cudaErrorNotSupported;
   }
 }
 
 template <typename T>
 cudaError_t dispatch_same(int jq, int epi, const Plan& pl, cudaStream_t s) {
-  const SweepArgs& a = pl.a;
+  using TIN = T;
+  using TST = T;
+  if (jq == JQ_D0) return dispatch_d0<T, T, T>(epi, pl, s);
+  if (jq == JQ_LINEAR1) {
+    if (epi == EPI_STORE) SWEEP(JQ_LINEAR1, EPI_STORE);
+    if (epi == EPI_ACC_AXPY) SWEEP(JQ_LINEAR1, EPI_ACC_AXPY);
+    return cudaErrorNotSupported;
+  }
+  if (jq == JQ_WENOZ1) {
+    if (epi == EPI_STORE) SWEEP(JQ_WENOZ1, EPI_STORE);
+    if (epi == EPI_ACC_AXPY) SWEEP(JQ_WENOZ1, EPI_ACC_AXPY);
+    return cudaErrorNotSupported;
+  }
   if (jq == JQ_WENOZ) {
-    if (epi == EPI_STORE) return launch_sweep<T, T, T, JQ_WENOZ, EPI_STORE>(a, TMA, pl.grid, pl.block, pl.smem, s);
-    if (epi == EPI_HJ_X) return launch_sweep<T, T, T, JQ_WENOZ, EPI_HJ_X>(a, TMA, pl.grid, pl.block, pl.smem, s);
-    if (epi == EPI_HJ_Y) return launch_sweep<T, T, T, JQ_WENOZ, EPI_HJ_Y>(a, TMA, pl.grid, pl.block, pl.smem, s);
-    if (epi == EPI_HJ_XG) return launch_sweep<T, T, T, JQ_WENOZ, EPI_HJ_XG>(a, TMA, pl.grid, pl.block, pl.smem, s);
-    if (epi == EPI_HJ_YG) return launch_sweep<T, T, T, JQ_WENOZ, EPI_HJ_YG>(a, TMA, pl.grid, pl.block, pl.smem, s);
-    if (epi == EPI_ACC_AXPY) return launch_sweep<T, T, T, JQ_WENOZ, EPI_ACC_AXPY>(a, TMA, pl.grid, pl.block, pl.smem, s);
+    if (epi == EPI_STORE) SWEEP(JQ_WENOZ, EPI_STORE);
+    if (epi == EPI_HJ_X) SWEEP(JQ_WENOZ, EPI_HJ_X);
+    if (epi == EPI_HJ_Y) SWEEP(JQ_WENOZ, EPI_HJ_Y);
+    if (epi == EPI_HJ_XG) SWEEP(JQ_WENOZ, EPI_HJ_XG);
+    if (epi == EPI_HJ_YG) SWEEP(JQ_WENOZ, EPI_HJ_YG);
+    if (epi == EPI_ACC_AXPY) SWEEP(JQ_WENOZ, EPI_ACC_AXPY);
     return cudaErrorNotSupported;
   }
   if (jq == JQ_LEARNED) {
     if constexpr (sizeof(T) == 4) {
-      if (epi == EPI_STORE) return launch_sweep<T, T, T, JQ_LEARNED, EPI_STORE>(a, nullptr, pl.grid, pl.block, pl.smem, s);
-      if (epi == EPI_HJ_X) return launch_sweep<T, T, T, JQ_LEARNED, EPI_HJ_X>(a, nullptr, pl.grid, pl.block, pl.smem, s);
-      if (epi == EPI_HJ_Y) return launch_sweep<T, T, T, JQ_LEARNED, EPI_HJ_Y>(a, nullptr, pl.grid, pl.block, pl.smem, s);
+      if (epi == EPI_STORE) return launch_sweep<T, T, T, JQ_LEARNED, EPI_STORE>(pl.a, nullptr, pl.grid, pl.block, pl.smem, s);
+      if (epi == EPI_HJ_X) return launch_sweep<T, T, T, JQ_LEARNED, EPI_HJ_X>(pl.a, nullptr, pl.grid, pl.block, pl.smem, s);
+      if (epi == EPI_HJ_Y) return launch_sweep<T, T, T, JQ_LEARNED, EPI_HJ_Y>(pl.a, nullptr, pl.grid, pl.block, pl.smem, s);
     }
     return cudaErrorNotSupported;
   }
-  if (epi == EPI_HJ_X) return launch_sweep<T, T, T, JQ_LINEAR, EPI_HJ_X>(a, TMA, pl.grid, pl.block, pl.smem, s);
-  if (epi == EPI_HJ_Y) return launch_sweep<T, T, T, JQ_LINEAR, EPI_HJ_Y>(a, TMA, pl.grid, pl.block, pl.smem, s);
-  if (epi == EPI_HJ_XG) return launch_sweep<T, T, T, JQ_LINEAR, EPI_HJ_XG>(a, TMA, pl.grid, pl.block, pl.smem, s);
-  if (epi == EPI_HJ_YG) return launch_sweep<T, T, T, JQ_LINEAR, EPI_HJ_YG>(a, TMA, pl.grid, pl.block, pl.smem, s);
-  return dispatch_lin<T, T, T>(epi, pl, s);
-}
-
-int jquad(const molt_desc& d) {
-  return d.weights == MOLT_W_WENOZ ? JQ_WENOZ : (d.weights == MOLT_W_LEARNED ? JQ_LEARNED : JQ_LINEAR);
+  if (epi == EPI_HJ_X) SWEEP(JQ_LINEAR, EPI_HJ_X);
+  if (epi == EPI_HJ_Y) SWEEP(JQ_LINEAR, EPI_HJ_Y);
+  if (epi == EPI_HJ_XG) SWEEP(JQ_LINEAR, EPI_HJ_XG);
+  if (epi == EPI_HJ_YG) SWEEP(JQ_LINEAR, EPI_HJ_YG);
+  return cudaErrorNotSupported;
 }
 
 // apply_D in mixed precision reads the FP64 array directly; molt_step's
 // sweeps read the FP32 copy of the state.
 cudaError_t launch(const Problem& p, int epi, const Plan& pl, cudaStream_t s, bool from_state_copy) {
-  const int jq = jquad(p.d);
+  const int jq = jquad(p.d, pl.a.mode);
   if (is_f64_sweep(p.d)) return dispatch_same<double>(jq, epi, pl, s);
   if (is_f32_state(p.d)) return dispatch_same<float>(jq, epi, pl, s);
   if (jq == JQ_LEARNED) return cudaErrorNotSupported;
+  using T = float;
+  using TST = double;
   if (!from_state_copy) {
+    using TIN = double;
     if (epi != EPI_STORE) return cudaErrorNotSupported;
-    if (jq == JQ_WENOZ)
-      return launch_sweep<float, double, double, JQ_WENOZ, EPI_STORE>(pl.a, TMA, pl.grid, pl.block, pl.smem, s);
-    return launch_sweep<float, double, double, JQ_LINEAR, EPI_STORE>(pl.a, TMA, pl.grid, pl.block, pl.smem, s);
+    if (jq == JQ_WENOZ) SWEEP(JQ_WENOZ, EPI_STORE);
+    if (jq == JQ_WENOZ1) SWEEP(JQ_WENOZ1, EPI_STORE);
+    if (jq == JQ_LINEAR1) SWEEP(JQ_LINEAR1, EPI_STORE);
+    SWEEP(JQ_D0, EPI_STORE);
   }
-  if (jq == JQ_WENOZ) return cudaErrorNotSupported;
-  return dispatch_lin<float, float, double>(epi, pl, s);
+  using TIN = float;
+  if (jq == JQ_LINEAR1 && epi == EPI_ACC_AXPY) SWEEP(JQ_LINEAR1, EPI_ACC_AXPY);
+  if (jq != JQ_D0) return cudaErrorNotSupported;
+  return dispatch_d0<float, float, double>(epi, pl, s);
 }
+#undef SWEEP
 
 // Line-per-lane FP32 sweeps (csrc/sweep_lanes.cuh): FP32 input, linear rule,
 // D_0 / D_R / D_L with P <= 2, lines of 16..512 points (multiples of 16) in
@@ -2057,19 +2096,20 @@ molt_status batch_build(molt_ctx* c, void* const* u, const std::vector<int>& sel
       if (st != MOLT_OK) return st;
       if (pl.block != 512) return fail(c, MOLT_EUNSUPPORTED, "batch tile does not fill 512 threads");
       pl.a.in = p.shadow;
-      pl.a.acc = p.acc;
+      pl.a.acc = ax == 0 ? p.acc : p.accy;
       pl.a.status = c->status_dev;
-      BatchSweep bs;
+      BatchSweep bs{};
       bs.a = pl.a;
       bs.E = B.E[ax][i];
       bs.first_item = items[ax];
       bs.ntiles = int((pl.a.g.nlines + pl.a.W - 1) / pl.a.W);
       items[ax] += bs.ntiles;
       hs.push_back(bs);
-      if (pl.smem > sm) sm = pl.smem;
+      sm = std::max(sm, size_t(pl.a.W) * pl.a.LS * sizeof(float));
     }
     BatchUpdate bu;
     bu.acc = static_cast<const float*>(p.acc);
+    bu.accy = static_cast<const float*>(p.accy);
     bu.u = static_cast<double*>(u ? u[i] : nullptr);
     bu.st1 = static_cast<double*>(p.stage1);
     bu.st2 = static_cast<double*>(p.stage2);
@@ -2101,9 +2141,9 @@ molt_status batch_build(molt_ctx* c, void* const* u, const std::vector<int>& sel
   prm.status = c->status_dev;
   prm.wait_limit = c->wait_limit;
   prm.skip_arrive = c->test_skip_arrive ? 1 : 0;
-  prm.stage_off = unsigned((sm + 127) & ~size_t(127));
+  prm.buf_bytes = unsigned((sm + 127) & ~size_t(127));
   *out = prm;
-  *smem = prm.stage_off + size_t(kStageFloats) * sizeof(float);
+  *smem = kBatchHead + 2 * size_t(prm.buf_bytes);
   return MOLT_OK;
 }
 
@@ -2204,6 +2244,13 @@ molt_status batch_prepare(molt_ctx* c) {
       B.E[ax][i] = shape_ok(n, 16) ? 16 : (shape_ok(n, 8) ? 8 : 4);
     }
   }
+  for (auto& p : c->probs)
+    if (!p.accy && cudaMalloc(&p.accy, sizeof(float) * size_t(p.total)) != cudaSuccess) {
+      cudaGetLastError();
+      p.accy = nullptr;
+      B.supported = false;   // no room for the second sum: problem by problem
+      return MOLT_OK;
+    }
   if (cudaMalloc(&B.d_sweeps, sizeof(BatchSweep) * 2 * np) != cudaSuccess ||
       cudaMalloc(&B.d_updates, sizeof(BatchUpdate) * np) != cudaSuccess ||
       cudaMalloc(&B.d_bar, 2 * sizeof(unsigned int)) != cudaSuccess) {
@@ -2553,6 +2600,7 @@ molt_status molt_destroy(molt_ctx* c) {
     for (auto& cch : p.nu) cudaFree(cch.dev);
     for (void* t : p.nu_tmp) cudaFree(t);
     cudaFree(p.nu_sum);
+    cudaFree(p.accy);
     cudaFree(p.acc2);
     if (p.heat_graph) cudaGraphExecDestroy(p.heat_graph);
     for (void* v : p.hv) cudaFree(v);

@@ -142,8 +142,7 @@ bool plan(const molt_desc& d, int ax, double alpha, int* status, SweepArgs* a, i
   a->W = W;
   a->nwl = nwl;
   a->LS = LS;
-  const size_t off = (size_t(4 * W) * 8 + size_t(W * nwl * 4) * 4 + 15) & ~size_t(15);
-  *smem = off + size_t(W) * LS * 4;
+  *smem = tile_head_bytes(W, nwl, 4) + size_t(W) * LS * 4;
   if (*smem > kSmemTileBudget) return false;
   *block = 32 * nwl * W;
   *grid = int((g.nlines + W - 1) / W);
@@ -203,8 +202,8 @@ extern "C" molt_status molt_wave_step_noalloc(const molt_desc* d, const double* 
     a.acc = acc;
     cudaError_t e;
     if (ax + 1 < d->ndim) {
-      e = ax == 0 ? launch_sweep<float, float, double, false, EPI_ACC_SET>(a, nullptr, grid, block, smem, s)
-                  : launch_sweep<float, float, double, false, EPI_ACC_ADD>(a, nullptr, grid, block, smem, s);
+      e = ax == 0 ? launch_sweep<float, float, double, JQ_D0, EPI_ACC_SET>(a, nullptr, grid, block, smem, s)
+                  : launch_sweep<float, float, double, JQ_D0, EPI_ACC_ADD>(a, nullptr, grid, block, smem, s);
     } else {
       if (d->ndim == 1) a.acc = nullptr;
       a.un = u;
@@ -212,7 +211,7 @@ extern "C" molt_status molt_wave_step_noalloc(const molt_desc* d, const double* 
       a.dst = u_next;
       a.coefS = -d->beta * d->beta;
       a.from_rest = from_rest ? 1 : 0;
-      e = launch_sweep<float, float, double, false, EPI_WAVE_FINAL>(a, nullptr, grid, block, smem, s);
+      e = launch_sweep<float, float, double, JQ_D0, EPI_WAVE_FINAL>(a, nullptr, grid, block, smem, s);
     }
     if (e != cudaSuccess) return MOLT_ECUDA;
   }

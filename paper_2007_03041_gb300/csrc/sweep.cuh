@@ -45,10 +45,6 @@ constexpr int kG = 16;   // ghost slots per side in shared memory (3 used)
 #define MOLT_MAX_THREADS 512
 #endif
 constexpr int kMaxThreads = MOLT_MAX_THREADS;
-#ifndef MOLT_MIN_BLOCKS
-#define MOLT_MIN_BLOCKS 1
-#endif
-constexpr int kMinBlocks = MOLT_MIN_BLOCKS;   // resident CTAs per SM the register budget targets
 // Shared memory per CTA (the GPU allows 227 KB): a sweep tile's budget, and the
 // dynamic size the sweep kernels opt into (a TMA tile plus its staging buffer
 // must fit it).
@@ -100,20 +96,20 @@ struct SweepArgs {
   int mode;           // Mode
   int P;
   int contiguous;     // stride == 1
-  double c[6];        // J_R weights on offsets -3..2
-  double sub[3][4];   // WENO substencil weights (5-point rule)
-  double d[3];        // linear weights
-  double q;           // e^{-nu}
-  double qE;          // e^{-nu E}
-  double invq;        // e^{+nu}
-  double inv1mmu;     // 1/(1-mu)
-  double mu;          // e^{-alpha(b-a)}
-  double invdet;      // 1/(1-mu^2)
-  double k2det, k2detq;  // 2/(1-mu^2) and 2 e^{nu}/(1-mu^2) (Dirichlet L_0 carries)
+  // line constants (csrc/line_constants.h); the FP32 copies are rounded on
+  // the host (converting on the device would use the FP64 pipe)
+  int d0;             // JQ_D0: 1 residual form, 0 K filters
+  int close;          // boundary constants: 0 none, 1 kA, 2 kA and kB
+  double b[5];        // K_R taps on the differences d_{i-2} .. d_{i+2}
+  double f0, f1, kap; // residual form of D_0 (K form: kap = 1/2)
+  double wk[6];       // WENO-Z substencil rules in difference form
+  double d[3];        // WENO linear weights
+  double qp[13];      // q^(2^k), q = e^{-nu}
+  double qlast, qlw;  // q^(valid points of the last lane / of the last warp)
+  double kA, kB;      // boundary constants C = kA T_same + kB T_other
   double alpha;
-  // the same coefficients rounded to FP32 on the host (FP32 kernels read
-  // these; converting on the device would use the FP64 pipe)
-  float cf[6], subf[3][3], df[3], qf, qEf, alphaf;
+  float bf[5], f0f, f1f, kapf, wkf[6], df[3], qpf[13], qlastf, qlwf, alphaf;
+  float kAh, kAl, kBh, kBl;   // kA, kB as FP32 pairs
   // epilogue operands
   const void* in;     // sweep input (TIN)
   void* out;          // EPI_STORE destination / HJ: H^_x buffer (state type)
@@ -147,8 +143,24 @@ struct SweepArgs {
   unsigned long long* mlp_stats;    // [stencils evaluated, WENO-Z fallbacks]
 };
 
-// Local-quadrature kind of a sweep kernel (template parameter JQ).
-enum JQuad { JQ_LINEAR = 0, JQ_WENOZ = 1, JQ_LEARNED = 2 };
+// Kind of a sweep kernel (template parameter JQ): the local quadrature, and
+// whether both scans run (LINEAR, WENOZ, LEARNED: D_R and D_L, or their mean),
+// D_0 with linear weights (D0), or one side alone (LINEAR1, WENOZ1).
+enum JQuad { JQ_LINEAR = 0, JQ_WENOZ = 1, JQ_LEARNED = 2, JQ_D0 = 3, JQ_LINEAR1 = 4, JQ_WENOZ1 = 5 };
+
+// Registers per thread of the scan kernels: 128 (512 threads per SM), and 80
+// for the FP64 D_0 and one-sided linear sweeps, which are bound by the FP64
+// pipe: a spilled value costs them nothing, a second or third resident CTA
+// keeps the pipe busy while another loads or stores (5277^2 diffusion, 2
+// steps: 128 / 80 / 64 registers 5.11 / 3.87 / 3.97 ms; the two-sided
+// Hamilton-Jacobi sweeps of a 1759^2 FP64 run 2.05 / 2.29 / 2.36 ms).
+#ifndef MOLT_SWEEP_REGS_F64
+#define MOLT_SWEEP_REGS_F64 80
+#endif
+template <typename T, int JQ>
+__host__ __device__ constexpr int sweep_regs() {
+  return sizeof(T) == 8 && (JQ == JQ_D0 || JQ == JQ_LINEAR1) ? MOLT_SWEEP_REGS_F64 : 128;
+}
 
 // Shared-memory index of point e of a line whose lanes own E points each: one
 // pad word after every E words (kG is a multiple of E), so lane chunks start
@@ -249,49 +261,11 @@ __device__ __forceinline__ TO cvt(FROM x) {
   else return TO(x);
 }
 
-// ---------------------------------------------------------------- arithmetic
-// y <- a*y + b on y = hi + lo.  FP32: compensated (exact product error by FMA,
-// TwoSum for the addition).  FP64: plain FMA.
-#ifndef MOLT_SHARED_BETA
-#define MOLT_SHARED_BETA 1   // WENO-Z: smoothness indicators from per-triple products shared by neighbouring points
-#endif
-#ifndef MOLT_COMPENSATED
-#define MOLT_COMPENSATED 1
-#endif
-template <typename T>
-struct Acc {
-  T hi, lo;
-  __device__ __forceinline__ void step(T a, T b) {
-    if constexpr (sizeof(T) == 4 && MOLT_COMPENSATED) {
-      const T p = a * hi;
-      const T pe = fmaf(a, hi, -p);
-      const T s = p + b;
-      const T bb = s - p;
-      const T se = (p - (s - bb)) + (b - bb);
-      lo = fmaf(a, lo, pe + se);
-      hi = s;
-    } else {
-      hi = fma(a, hi, b);
-    }
-  }
-  __device__ __forceinline__ T value() const {
-    if constexpr (sizeof(T) == 4 && MOLT_COMPENSATED) return hi + lo; else return hi;
-  }
-};
-
 template <typename T>
 __device__ __forceinline__ T shfl_up(T v, int d) { return __shfl_up_sync(0xffffffffu, v, d); }
 template <typename T>
 __device__ __forceinline__ T shfl_down(T v, int d) { return __shfl_down_sync(0xffffffffu, v, d); }
 
-// WENO-Z weighted local integral from the 5 values w[0..4] = v at offsets
-// -3..1 relative to the target node, in the orientation of J_R (J_L passes
-// the mirrored values).  Smoothness indicators: beta_r = int_{-1}^0
-// (p_r')^2 + (p_r'')^2 dt for the quadratic through substencil r, worked out
-// in closed form with s1 = (c-a)/2, s2 = a-2b+c:
-//   beta_0 = s1^2 + 3 s1 s2 + 10/3 s2^2,  beta_1 = s1^2 + s1 s2 + 4/3 s2^2,
-//   beta_2 = s1^2 - s1 s2 + 4/3 s2^2.
-// WENO-Z (Sec. 2.4): w~_r = d_r (1 + tau/(eps+beta_r)), tau = |beta_0-beta_2|.
 // Reciprocal for the nonlinear weights: FP32 takes the hardware
 // approximation (at most 1 ulp; the arguments eps + beta_r and sum_r w~_r are
 // at least 1e-6 and about 1), FP64 the division.
@@ -302,11 +276,17 @@ __device__ __forceinline__ float weight_rcp(float x) {
 }
 __device__ __forceinline__ double weight_rcp(double x) { return 1.0 / x; }
 
+// WENO-Z forcing K(x_i) = v_i - q v_{i-1} - J(x_i) in the orientation of J_R
+// (J_L passes the mirrored differences): e0 = v_i - v_{i-1}, e1 = v_{i-1} -
+// v_{i-2}, e2 = v_{i-2} - v_{i-3}, f = v_{i+1} - v_i.  Every substencil rule
+// integrates the constant to 1 - q and the weights sum to one, so
+// K = sum_r w_r K_r with K_r = q e0 + sum_j c^{(r)}_j (v_i - v_j) a filter of
+// the differences (wk, csrc/line_constants.h; the e0 weight of K_0 is 1).
+// WENO-Z (Sec. 2.4): w~_r = d_r (1 + tau/(eps+beta_r)), tau = |beta_0-beta_2|.
 template <typename T>
-__device__ __forceinline__ T wenoz_from_beta(const T* w, const T (&beta)[3], const T (&sub)[3][3], const T (&d)[3]) {
-  T J[3];
-#pragma unroll
-  for (int r = 0; r < 3; ++r) J[r] = sub[r][0] * w[r] + sub[r][1] * w[r + 1] + sub[r][2] * w[r + 2];
+__device__ __forceinline__ T wenoz_defect(T e0, T e1, T e2, T f, const T (&beta)[3], const T (&wk)[6],
+                                          const T (&d)[3]) {
+  const T K[3] = {fma(wk[1], e2, fma(wk[0], e1, e0)), fma(wk[3], e1, wk[2] * e0), fma(wk[5], f, wk[4] * e0)};
   const T tau = fabs(beta[0] - beta[2]);
   const T eps = T(1e-6);
   T wt[3], sum = T(0);
@@ -315,18 +295,19 @@ __device__ __forceinline__ T wenoz_from_beta(const T* w, const T (&beta)[3], con
     wt[r] = fma(d[r] * tau, weight_rcp(eps + beta[r]), d[r]);   // d_r (1 + tau/(eps+beta_r))
     sum += wt[r];
   }
-  return (wt[0] * J[0] + wt[1] * J[1] + wt[2] * J[2]) * weight_rcp(sum);
+  return (wt[0] * K[0] + wt[1] * K[1] + wt[2] * K[2]) * weight_rcp(sum);
 }
 
-// The smoothness indicator of substencil r from the products of its node
-// triple (a, b, c): with s1 = (c - a)/2 and s2 = a - 2b + c, beta_r = s1^2 +
-// k_r s1 s2 + m_r s2^2 (k = 3, 1, -1; m = 10/3, 4/3, 4/3).  A triple serves
-// three points' J_R and, mirrored (s1 -> -s1), three points' J_L, so the
-// products are formed once per triple.
+// Smoothness indicators: beta_r = int_{-1}^0 (p_r')^2 + (p_r'')^2 dt for the
+// quadratic through the node triple (a, b, c) of substencil r; with s1 =
+// (c - a)/2 and s2 = a - 2b + c, beta_r = s1^2 + k_r s1 s2 + m_r s2^2 (k = 3,
+// 1, -1; m = 10/3, 4/3, 4/3).  A triple serves three points' J_R and,
+// mirrored (s1 -> -s1), three points' J_L, so the products are formed once
+// per triple, from its differences da = b - a, db = c - b.
 template <typename T>
-__device__ __forceinline__ void triple_products(T a, T b, T c, T* p11, T* p12, T* p22) {
-  const T s1 = T(0.5) * (c - a);
-  const T s2 = a - T(2) * b + c;
+__device__ __forceinline__ void triple_products(T da, T db, T* p11, T* p12, T* p22) {
+  const T s1 = T(0.5) * (da + db);
+  const T s2 = db - da;
   *p11 = s1 * s1;
   *p12 = s1 * s2;
   *p22 = s2 * s2;
@@ -338,37 +319,21 @@ __device__ __forceinline__ T beta_from_products(int r, T p11, T p12, T p22, bool
   return p11 + (mirrored ? -k : k) * p12 + m * p22;
 }
 
-template <typename T>
-__device__ __forceinline__ T wenoz_integral(const T* w, const T (&sub)[3][3], const T (&d)[3]) {
-  T J[3], beta[3];
-#pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    const T a = w[r], b = w[r + 1], c = w[r + 2];
-    J[r] = sub[r][0] * a + sub[r][1] * b + sub[r][2] * c;
-    const T s1 = T(0.5) * (c - a);
-    const T s2 = a - T(2) * b + c;
-    const T k = r == 0 ? T(3) : (r == 1 ? T(1) : T(-1));
-    const T m = r == 0 ? T(10.0 / 3.0) : T(4.0 / 3.0);
-    beta[r] = s1 * s1 + k * s1 * s2 + m * s2 * s2;
-  }
-  const T tau = fabs(beta[0] - beta[2]);
-  const T eps = T(1e-6);
-  T wt[3], sum = T(0);
-#pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    wt[r] = fma(d[r] * tau, weight_rcp(eps + beta[r]), d[r]);   // d_r (1 + tau/(eps+beta_r))
-    sum += wt[r];
-  }
-  return (wt[0] * J[0] + wt[1] * J[1] + wt[2] * J[2]) * weight_rcp(sum);
+// -------------------------------------------------------------- tile staging
+// Barrier of the warps that share line lw of a tile (named barrier 1 + lw;
+// tiles of several warps per line hold at most 8 lines).
+__device__ __forceinline__ void line_sync(int nwl, int lw) {
+  if (nwl == 1) __syncwarp();
+  else asm volatile("bar.sync %0, %1;" ::"r"(1 + lw), "r"(32 * nwl) : "memory");
 }
 
-// -------------------------------------------------------------- tile staging
 // Contiguous lines: the nwl warps of line lw read it with consecutive lanes.
 // Strided lines: thread (p, w) with w fastest, so a warp reads whole rows of
 // W neighbouring lines.
-template <typename T, typename TIN, int E = kE, bool CG = false>
-__device__ __forceinline__ void load_tile(const SweepArgs& a, const TIN* in, T* lines, long long line0,
-                                          int lw, int tl) {
+// put(shared destination, global source) moves one value.
+template <typename T, typename TIN, int E, typename Put>
+__device__ __forceinline__ void load_tile(const SweepArgs& a, const TIN* in, T* lines, long long line0, int lw, int tl,
+                                          Put put) {
   const int W = a.W, n = a.g.n;
   if (a.contiguous) {
     const long long gl = line0 + lw;
@@ -377,7 +342,7 @@ __device__ __forceinline__ void load_tile(const SweepArgs& a, const TIN* in, T* 
     T* dstl = lines + lw * a.LS;
     const int step = a.nwl * 32;
 #pragma unroll 4
-    for (int p = tl; p < n; p += step) dstl[phys<E>(p)] = cvt<T>(gload<CG>(src + p));
+    for (int p = tl; p < n; p += step) put(dstl + phys<E>(p), src + p);
   } else {
     // prow = blockDim/W is a multiple of 16, so phys<E>() advances by a constant
     const int w = threadIdx.x % W;
@@ -392,41 +357,9 @@ __device__ __forceinline__ void load_tile(const SweepArgs& a, const TIN* in, T* 
     const int dstep = prow + prow / E;
 #pragma unroll 8
     for (; p < n; p += prow) {
-      *dst = cvt<T>(gload<CG>(src));
+      put(dst, src);
       src += sstep;
       dst += dstep;
-    }
-  }
-}
-
-template <typename T, int E = kE>
-__device__ __forceinline__ void fill_ghosts(const SweepArgs& a, T* lines) {
-  const int n = a.g.n;
-  for (int t = threadIdx.x; t < a.W * 6; t += blockDim.x) {
-    const int w = t / 6, g = t - w * 6;
-    T* b = lines + w * a.LS;
-    if (g < 3) {
-      const int j = g + 1;  // ghost e = -j
-      T val;
-      if (a.bc == 0) {
-        int s = (-j) % n;
-        if (s < 0) s += n;
-        val = b[phys<E>(s)];
-      } else {
-        const int m = j < n - 1 ? j : n - 1;
-        val = T(2) * b[phys<E>(0)] - b[phys<E>(m)];
-      }
-      b[phys<E>(-j)] = val;
-    } else {
-      const int j = g - 2;  // ghost e = n-1+j
-      T val;
-      if (a.bc == 0) {
-        val = b[phys<E>((n - 1 + j) % n)];
-      } else {
-        const int m = n - 1 - j > 0 ? n - 1 - j : 0;
-        val = T(2) * b[phys<E>(n - 1)] - b[phys<E>(m)];
-      }
-      b[phys<E>(n - 1 + j)] = val;
     }
   }
 }
@@ -436,11 +369,10 @@ __device__ __forceinline__ void fill_ghosts(const SweepArgs& a, T* lines) {
 // epilogue operands.
 
 struct TileSmem {
-  double* carries;   // [W][4] compute-type (hi, lo) carry pairs (room for FP64)
-  void* totals;      // [W][nwl][4] of T
+  void* totals;      // [W][nwl][2] of T: end values of the warps' scans from zero (R, L)
   void* lines;       // [W][LS] of T
   void* lines2;      // two_out: [W][LS] of T (delta of AFFINE_SQ)
-  float* jloc;       // JQ_LEARNED: [W][2][LS] local integrals J_R, J_L
+  float* jloc;       // JQ_LEARNED: [W][2][LS] forcings K_R, K_L
   MlpNet* net;       // JQ_LEARNED: the network
 };
 
@@ -450,12 +382,16 @@ __host__ __device__ constexpr size_t learned_extra_bytes(int W, int LS) {
   return 16 + size_t(2) * W * LS * sizeof(float) + sizeof(MlpNet);
 }
 
+// Shared bytes before the lines: the warps' totals.
+__host__ __device__ constexpr size_t tile_head_bytes(int W, int nwl, size_t elem) {
+  return (size_t(W) * nwl * 2 * elem + 15) & ~size_t(15);
+}
+
 template <typename T, int JQ = JQ_LINEAR>
 __device__ __forceinline__ TileSmem carve(unsigned char* smem, const SweepArgs& a, size_t* used) {
   TileSmem t;
-  t.carries = reinterpret_cast<double*>(smem);
-  t.totals = reinterpret_cast<T*>(t.carries + 4 * a.W);
-  const size_t off = (size_t(4 * a.W) * sizeof(double) + size_t(a.W * a.nwl * 4) * sizeof(T) + 15) & ~size_t(15);
+  t.totals = smem;
+  const size_t off = tile_head_bytes(a.W, a.nwl, sizeof(T));
   t.lines = smem + off;
   *used = off + size_t(a.W) * a.LS * sizeof(T);
   t.lines2 = nullptr;
@@ -476,100 +412,50 @@ __device__ __forceinline__ TileSmem carve(unsigned char* smem, const SweepArgs& 
   return t;
 }
 
-// Fills the ghosts of the staged lines, applies D P times (the whole method
-// step of the header comment) and leaves S_P (or, for MODE_RL, the per-axis
-// Lax-Friedrichs Hamiltonian) in the line buffers.  Returns the thread's
-// largest one-sided derivative magnitude (MODE_RL).  Ends synchronised.
-// Pairs of compute-type values advanced together: FP32 pairs use the packed
-// FP32x2 instructions of sm_100+ (FFMA2/FADD2/FMUL2), FP64 pairs plain FMAs.
-template <typename T> struct Pair;
-template <> struct Pair<float> { using type = float2; };
-template <> struct Pair<double> { using type = double2; };
+// Packed FP32x2 arithmetic of sm_100+ (line-per-lane and x-line sweeps).
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 
+// ------------------------------------------------------------- line constants
 template <typename T>
-__device__ __forceinline__ typename Pair<T>::type pair2(T x, T y) {
-  typename Pair<T>::type r;
-  r.x = x;
-  r.y = y;
+__device__ __forceinline__ T qpow_bit(const SweepArgs& a, int k) { return pick<T>(a.qp[k], a.qpf[k]); }
+
+// q^e for 0 <= e < 2^COUNT, times 2^LO: the product of the stored powers
+// q^(2^(LO + k)) over the bits of e.
+template <typename T, int LO, int COUNT>
+__device__ __forceinline__ T qpow(const SweepArgs& a, int e) {
+  T r = T(1);
+#pragma unroll
+  for (int k = 0; k < COUNT; ++k)
+    if ((e >> k) & 1) r *= qpow_bit<T>(a, LO + k);
   return r;
 }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-// a - b exactly as an FMA with -1
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-__device__ __forceinline__ double2 fma2(double2 a, double2 b, double2 c) {
-  return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
-}
-__device__ __forceinline__ double2 add2(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ double2 mul2(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
-__device__ __forceinline__ double2 sub2(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 
-// Acc on a pair of independent recurrences (y <- a*y + b per component).
-template <typename T>
-struct Acc2 {
-  using V = typename Pair<T>::type;
-  V hi, lo;
-  __device__ __forceinline__ void step(V a, V b) {
-    if constexpr (sizeof(T) == 4 && MOLT_COMPENSATED) {
-      const V p = mul2(a, hi);
-      const V pe = fma2(a, hi, pair2<T>(-p.x, -p.y));
-      const V s = add2(p, b);
-      const V bb = sub2(s, p);
-      const V se = add2(sub2(p, sub2(s, bb)), sub2(b, bb));
-      lo = fma2(a, lo, add2(pe, se));
-      hi = s;
-    } else {
-      hi = fma2(a, hi, b);
-    }
-  }
-  __device__ __forceinline__ V value() const {
-    if constexpr (sizeof(T) == 4 && MOLT_COMPENSATED) return add2(hi, lo); else return hi;
-  }
-};
-
-// Line boundary constants (Sec. 2.3, Sec. 3.3) in FP64 from the line totals
-// I_R(b) = tbR and I_L(a) = tbL, returned as the initial values of the R and
-// L scans: periodic -> the cyclic values I(b)/(1-mu), I(a)/(1-mu);
-// Dirichlet L_0 -> 2A and 2B from the 2x2 system with determinant 1-mu^2;
-// Dirichlet L_R / L_L -> v(a) / v(b).  Exact-fit kernels divide Dirichlet
-// values by q (their end nodes keep the map (q, 0)).
-template <typename T, bool RAGGED, int E = kE>
-__device__ __forceinline__ void boundary_carries(const SweepArgs& a, const T* bw, int n, T tbR, T tbL, double* CR,
-                                                 double* CL) {
-  const double IRb = cvt<double>(tbR);
-  const double ILa = cvt<double>(tbL);
-  if (a.bc == 0) {
-    *CR = IRb * a.inv1mmu;
-    *CL = ILa * a.inv1mmu;
-    return;
-  }
-  const double v0 = cvt<double>(bw[phys<E>(0)]), vN = cvt<double>(bw[phys<E>(n - 1)]);
-  double cr, cl;
-  if (a.mode == MODE_0) {
-    // 2A, 2B (the 1/q of exact-fit kernels folded into the constant)
-    const double r0 = fma(-0.5, ILa, v0), r1 = fma(-0.5, IRb, vN);
-    const double k = RAGGED ? a.k2det : a.k2detq;
-    cr = fma(-a.mu, r1, r0) * k;
-    cl = fma(-a.mu, r0, r1) * k;
+// Line boundary constants (Sec. 2.3, Sec. 3.3): the value C = kA T_same +
+// kB T_other that enters the line before its first scan position, from the
+// end values T of the scans started from zero.  FP64 sweeps compute it in
+// FP64.  FP32 sweeps compute it in pairs of FP32 numbers (kA, kB as hi + lo;
+// exact product errors by FMA, TwoSum for the addition: 48 bits, rounded once
+// to the FP32 that enters the scan), so that every warp solves its own line:
+// the FP64 pipe, two FMAs per clock and SM here, held a barrier of the whole
+// CTA per application of D.
+template <typename T, typename Args>
+__device__ __forceinline__ T line_constant(const Args& a, T same, T other) {
+  if constexpr (sizeof(T) == 8) {
+    const T c = a.kA * same;
+    return a.close == 2 ? fma(a.kB, other, c) : c;
   } else {
-    cr = v0;   // L_R^{-1}(a) = v(a)
-    cl = vN;   // L_L^{-1}(b) = v(b)
-    if (!RAGGED) {
-      cr *= a.invq;
-      cl *= a.invq;
+    T p = a.kAh * same;
+    T e = fmaf(a.kAl, same, fmaf(a.kAh, same, -p));
+    if (a.close == 2) {
+      const T p2 = a.kBh * other;
+      e += fmaf(a.kBl, other, fmaf(a.kBh, other, -p2));
+      const T s = p + p2, bb = s - p;
+      e += (p - (s - bb)) + (p2 - bb);
+      p = s;
     }
+    return p + e;
   }
-  *CR = cr;
-  *CL = cl;
-}
-
-// Compute-type (hi, lo) pair of an FP64 carry.
-template <typename T>
-__device__ __forceinline__ void split_carry(double c, T* hi, T* lo) {
-  const T h = cvt<T>(c);
-  *hi = h;
-  *lo = cvt<T>(c - cvt<double>(h));
 }
 
 // Ghost cells of one line by the lanes of the warp that owns it.
@@ -606,20 +492,18 @@ __device__ __forceinline__ void warp_fill_ghosts(const SweepArgs& a, T* b, int l
 // gather the 5-value stencils (J_R: v_{e-3..e+1}; J_L mirrored: v_{e+3..e-1})
 // from the staged line, the warp evaluates the network on the tensor cores,
 // and lanes t = 0, 1 of each row group finish rows g, g+8: WENO-Z fallback
-// check, then J = sum_r w_r J^{(r)} into jr / jl (shared, line layout).
+// check, then K = v - q v_prev - sum_r w_r J^{(r)} into jr / jl (shared, line layout).
 template <int E>
 __device__ __forceinline__ void learned_local_integrals(const SweepArgs& a, const MlpNet& net, const float* buf,
                                                         float* jr, float* jl, int first, int n, int lane) {
   const int g = lane >> 2, t = lane & 3;
   MlpRegs R;
   mlp_load_regs(net, lane, R);
-  float sub[3][3], d[3];
+  float wk[6], d[3];
 #pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    d[r] = a.df[r];
+  for (int r = 0; r < 3; ++r) d[r] = a.df[r];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) sub[r][j] = a.subf[r][j];
-  }
+  for (int i = 0; i < 6; ++i) wk[i] = a.wkf[i];
   unsigned evaluated = 0, fallbacks = 0;
   for (int b = 0; b < 32 * E; b += 16) {
     if (first + b >= n) break;   // warp-uniform
@@ -651,10 +535,11 @@ __device__ __forceinline__ void learned_local_integrals(const SweepArgs& a, cons
         for (int r = 0; r < 3; ++r) p[r] = t == 0 ? p0[r] : p1[r];
         fallbacks += mlp_final_weights(v, p, d, w) ? 1u : 0u;
         ++evaluated;
-        float J = 0.f;
-#pragma unroll
-        for (int r = 0; r < 3; ++r) J = fmaf(w[r], fmaf(sub[r][0], v[r], fmaf(sub[r][1], v[r + 1], sub[r][2] * v[r + 2])), J);
-        (side == 0 ? jr : jl)[phys<E>(e)] = J;
+        // K = sum_r w_r K_r in difference form (wenoz_defect)
+        const float f0 = v[3] - v[2], f1 = v[2] - v[1], f2 = v[1] - v[0], f = v[4] - v[3];
+        const float K0 = fmaf(wk[1], f2, fmaf(wk[0], f1, f0));
+        const float K1 = fmaf(wk[3], f1, wk[2] * f0), K2 = fmaf(wk[5], f, wk[4] * f0);
+        (side == 0 ? jr : jl)[phys<E>(e)] = fmaf(w[0], K0, fmaf(w[1], K1, w[2] * K2));
       }
     }
   }
@@ -669,353 +554,437 @@ __device__ __forceinline__ void learned_local_integrals(const SweepArgs& a, cons
   }
 }
 
-// WL (warp-local): every line is owned by a single warp (nwl == 1), so a D
-// application needs no CTA-wide barrier: ghosts, line totals and the FP64
-// boundary solve stay inside the warp (the solve runs on lane 0 and its
-// result is broadcast by shuffles).
+// Value of ghost point e (-3 <= e < 0 or n <= e < n + 3) of an exact-fit
+// line (n >= 128): the periodic image, or the odd reflection about the end
+// value (Sec. 2.3).
+template <typename T, int E>
+__device__ __forceinline__ T ghost_value(const T* b, int e, int n, int bc) {
+  if (bc == 0) return b[phys<E>(e < 0 ? e + n : e - n)];
+  if (e < 0) return T(2) * b[phys<E>(0)] - b[phys<E>(-e)];
+  return T(2) * b[phys<E>(n - 1)] - b[phys<E>(2 * (n - 1) - e)];
+}
+
+// Applies D P times to the staged lines and leaves S_P (or, for MODE_RL, the
+// per-axis Lax-Friedrichs Hamiltonian) in the line buffers.  Returns the
+// thread's largest one-sided derivative magnitude (MODE_RL).  Ends
+// synchronised (contiguous lines: the line's warps, strided: the CTA).
+//
+// All scans run in difference form: with W_R = v - L_R^{-1}[v], W_L = v -
+// L_L^{-1}[v] and d_i = v_i - v_{i-1} the recurrences of Sec. 2.4 give
+//   W_R(x_i) = q W_R(x_{i-1}) + K_R(x_i),  K_R(x_i) = v_i - q v_{i-1} - J_R(x_i),
+//   W_L(x_i) = q W_L(x_{i+1}) + K_L(x_i),  K_L(x_i) = v_i - q v_{i+1} - J_L(x_i),
+// with K a 5-tap filter of the differences d (the weights of J sum to 1 - q,
+// App. C): no value of the size of v is subtracted from another, so FP32
+// needs no compensated arithmetic and D of a constant is exactly zero.
+//
+// D_0 with linear weights (JQ_D0).  D_0 = (W_R + W_L)/2 is a symmetric filter
+// delta^2 M(delta^2) / ((1-q)^2 - q delta^2) of v (delta^2 the second
+// difference, M a quadratic from the weights).  Dividing M by the denominator
+// leaves
+//   D_0 v_i = kap (U_i + V_i) + f0 s_i + f1 (s_{i-1} + s_{i+1}),
+//   U_i = q U_{i-1} + d_i,  V_i = q V_{i+1} - d_{i+1},  s = delta^2 v:
+// the scans take the bare differences, and the whole quadrature enters as
+// three constants (the 3-point rule has f1 = 0).  Per point: 11 operations
+// (9 with the 3-point rule) where the two 6-tap integrals, folds, fix-ups and
+// D = v - (I_R + I_L)/2 took 20.  f0, f1 grow like e^{3 nu}: a.d0 chooses
+// this form while they stay small (set_line_constants), else the K filters.
+//
+// JQ_LINEAR1 / JQ_WENOZ1 (MODE_R or MODE_L alone): the one side that is
+// asked for, the L side as the R scan of the mirrored line.
+//
+// Constants of the scans come from the host as powers q^(2^k): the lane maps
+// all have the multiplier q^E, so a warp scan moves one value per lane, and a
+// line of several warps scans its warps' totals 16 lanes at a time (R in
+// lanes 0-15, L in lanes 16-31), each warp for itself: one barrier of the
+// line's warps per application of D and one per write-back, none for a line
+// owned by one warp.
 // GEN: MODE_RL supports every HamKind (else |grad u|^2/2 only).
-template <typename T, int JQ, bool RAGGED, bool WL, int E = kE, bool GEN = false>
+template <typename T, int JQ, bool RAGGED, int E = kE, bool GEN = false>
 __device__ __forceinline__ double compute_lines(const SweepArgs& a, const TileSmem& sm, bool line_ok) {
   static_assert(JQ != JQ_LEARNED || sizeof(T) == 4, "learned weights run in FP32");
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr bool ONE = JQ == JQ_LINEAR1 || JQ == JQ_WENOZ1;
+  constexpr bool WENO = JQ == JQ_WENOZ || JQ == JQ_WENOZ1;
+  constexpr int LE = log2i<E>();
   const int nwl = a.nwl, n = a.g.n;
-  double* carries = sm.carries;
   T* totals = static_cast<T*>(sm.totals);
   T* lines = static_cast<T*>(sm.lines);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int lw = warp / nwl, part = warp - lw * nwl;
   const int tl = part * 32 + lane;
   T* buf = lines + lw * a.LS;
-  const int e0 = tl * E;
-  T* cbase = buf + (E + 1) * tl;   // phys<E>(e0 + j) = (E+1)*tl + chunk_off<E>(j)
+  // the lane's chunk: points e0 .. e0+E-1 (one-sided L scans run the line mirrored)
+  const bool mir = ONE && a.mode == MODE_L;
+  const int ch = mir ? nwl * 32 - 1 - tl : tl;
+  const int e0 = ch * E;
+  T* cbase = buf + (E + 1) * ch;   // phys<E>(e0 + j) = (E+1)*ch + chunk_off<E>(j)
   static_assert(phys<E>(E * 3 + 2) == (E + 1) * 3 + chunk_off<E>(2), "lane base / chunk offset mismatch");
-
-  const T q = pick<T>(a.q, a.qf);
-  const T qE = pick<T>(a.qE, a.qEf);
-  T c[6];
-#pragma unroll
-  for (int i = 0; i < 6; ++i) c[i] = pick<T>(a.c[i], a.cf[i]);
-  T sub[3][3], dw[3];
-  if constexpr (JQ == JQ_WENOZ) {
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      dw[r] = pick<T>(a.d[r], a.df[r]);
-#pragma unroll
-      for (int j = 0; j < 3; ++j) sub[r][j] = pick<T>(a.sub[r][j], a.subf[r][j]);
-    }
-  }
-  // lines owned by one warp (nwl == 1) need CTA barriers only around the
-  // vectorised boundary solve: ghosts, write-backs and the final store of a
-  // line are warp-local
+  const bool dir = a.bc == 1;
+  const T q = qpow_bit<T>(a, 0);
   const bool own = nwl == 1;
-  if (WL || own) {
-    warp_fill_ghosts<T, E>(a, buf, lane);
-    __syncwarp();
-  } else {
-    fill_ghosts<T, E>(a, lines);
-    __syncthreads();
-  }
 
-  // element maps: (q, J) for points with a local integral, identity for
-  // points past the end of the line and for the Dirichlet end nodes where the
-  // recurrences start (I_R(x_0) = 0, I_L(x_N) = 0).  RAGGED kernels mask per
-  // point.  Exact-fit kernels (n = nwl*32*E) have no points past the end;
-  // their Dirichlet end nodes keep the map (q, 0) and the line's initial
-  // value is divided by q, which yields the same values (x_0: q*(C/q) + 0 = C).
-  const int eR0 = (a.bc == 1) ? 1 : 0;          // first R point with a J
-  const int eL1 = (a.bc == 1) ? n - 2 : n - 1;  // last L point with a J
-  const bool zeroR0 = !RAGGED && a.bc == 1 && e0 == 0;
-  const bool zeroLN = !RAGGED && a.bc == 1 && e0 + E == n;
+  // powers of q: up to this lane inside its warp, up to this warp (R: from
+  // the left end, L: from the right end; one-sided: in scan order)
+  T pwR = T(1), pwL = T(1), qwR = T(1), qwL = T(1);
+  auto lane_powers = [&]() {
+    const bool ragged_first = RAGGED && (ONE ? mir && part == 0 : part == nwl - 1);
+    pwR = qpow<T, LE, 5>(a, lane);
+    if (!ONE || mir) {
+      T pl = ONE ? pwR : __shfl_sync(FULL, pwR, 31 - lane);
+      if (ragged_first) {
+        const int before = n - e0 - E;
+        pl = before > 0 ? qpow<T, 0, LE + 5>(a, before) : T(1);
+      }
+      if (ONE) pwR = pl; else pwL = pl;
+    }
+    if (!own) {
+      const T qlw = pick<T>(a.qlw, a.qlwf);
+      if (!mir) qwR = qpow<T, LE + 5, 4>(a, part);
+      else if (part > 0) qwR = qlw * qpow<T, LE + 5, 4>(a, part - 1);
+      if (!ONE && part < nwl - 1) qwL = qlw * qpow<T, LE + 5, 4>(a, nwl - 2 - part);
+    }
+  };
+  if constexpr (JQ != JQ_LEARNED) lane_powers();   // (not live across the network)
+  // the lane whose last point closes the R scan of its warp
+  const int lastR = (RAGGED && !mir && part == nwl - 1) ? ((n - 1) / E) & 31 : 31;
+  const T mulR = (RAGGED && !mir && part == nwl - 1) ? pick<T>(a.qlast, a.qlastf) : qpow_bit<T>(a, LE);
+  // Dirichlet: the scans start from zero at the end nodes
+  const bool end0 = dir && e0 == 0;
+  const bool endN = dir && n - 1 >= e0 && n - 1 < e0 + E;
 
-  // J_R(e0+k) and J_L(e0+E-1-k) share the pair Y[k] so that the R chain
-  // (ascending) and the L chain (descending) of the recurrences advance
-  // together in packed FP32x2 instructions.
-  using T2 = typename Pair<T>::type;
-  T v[E], S[E];
-  T2 Y[E];
-#pragma unroll
-  for (int k = 0; k < E; ++k) S[k] = T(0);
+  T S[E];
   T rmax = T(0);
 
   for (int p = 0; p < a.P; ++p) {
-    // ---- 1. local integrals from a window of E + 6 points
-    float* jrl = nullptr;
+    // ---- 1. forcings of the scans
+    // JQ_D0: X the differences d, F the FIR part; else (and in D_0's K form)
+    // X = K_R, F = K_L.  Scalar arithmetic: in packed FP32x2 form (R ascending
+    // with L descending) the moves that build the pairs cost more than the
+    // halved FMA count saved (64 heat problems 11.4 against 12.4 ms a pass).
+    T X[E + 1], F[E];
     if constexpr (JQ == JQ_LEARNED) {
-      jrl = sm.jloc + lw * 2 * a.LS;
-      if (line_ok) learned_local_integrals<E>(a, *sm.net, buf, jrl, jrl + a.LS, part * 32 * E, n, lane);
+      if (part == 0) warp_fill_ghosts<T, E>(a, buf, lane);
+      line_sync(nwl, lw);
+      float* jrl = sm.jloc + lw * 2 * a.LS;
+      if (line_ok)
+        learned_local_integrals<E>(a, *sm.net, buf, jrl, jrl + a.LS, part * 32 * E, n, lane);
       __syncwarp();
-    }
-    {
-      T win[E + 6];
-#pragma unroll
-      for (int k = 0; k < E + 6; ++k) win[k] = cbase[chunk_off<E>(k - 3)];
-#if MOLT_SHARED_BETA
-      T p11[E + 4], p12[E + 4], p22[E + 4];   // products of the node triples win[t..t+2]
-      if constexpr (JQ == JQ_WENOZ) {
-#pragma unroll
-        for (int t = 0; t < E + 4; ++t) triple_products<T>(win[t], win[t + 1], win[t + 2], &p11[t], &p12[t], &p22[t]);
-      }
-#endif
+      lane_powers();
 #pragma unroll
       for (int k = 0; k < E; ++k) {
-        v[k] = win[k + 3];
-        if constexpr (JQ == JQ_LEARNED) {
-          Y[k].x = jrl[(E + 1) * tl + chunk_off<E>(k)];
-          Y[E - 1 - (k)].y = jrl[a.LS + (E + 1) * tl + chunk_off<E>(k)];
-        } else if constexpr (JQ == JQ_WENOZ) {
-          T wr[5], wl[5];
+        X[k] = jrl[(E + 1) * tl + chunk_off<E>(k)];
+        F[k] = jrl[a.LS + (E + 1) * tl + chunk_off<E>(k)];
+      }
+    } else {
+      if constexpr (RAGGED) {
+        if (part == 0) warp_fill_ghosts<T, E>(a, buf, lane);
+        line_sync(nwl, lw);
+      }
+      // window of the chunk in scan orientation: win[j] = v at offset j - 3
+      // from the chunk's first point
+      T win[E + 6];
+      if (!mir) {
 #pragma unroll
-          for (int j = 0; j < 5; ++j) {
-            wr[j] = win[k + j];        // offsets -3..1
-            wl[j] = win[k + 6 - j];    // mirrored: v_{e+3} .. v_{e-1}
-          }
-#if MOLT_SHARED_BETA
-          // substencil r of J_R is the triple at k + r; of J_L the triple at
-          // k + 4 - r, reversed
-          T bR[3], bL[3];
+        for (int j = 0; j < E + 6; ++j) win[j] = cbase[chunk_off<E>(j - 3)];
+      } else {
 #pragma unroll
-          for (int r = 0; r < 3; ++r) {
-            bR[r] = beta_from_products<T>(r, p11[k + r], p12[k + r], p22[k + r], false);
-            bL[r] = beta_from_products<T>(r, p11[k + 4 - r], p12[k + 4 - r], p22[k + 4 - r], true);
+        for (int j = 0; j < E + 6; ++j) win[j] = cbase[chunk_off<E>(E + 2 - j)];
+      }
+      if constexpr (!RAGGED) {
+        // ghosts of an exact-fit line: only the end lanes need them
+        if (e0 == 0 || e0 + E == n) {
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            const int el = mir ? e0 + E + 2 - j : e0 + j - 3;
+            const int er = mir ? e0 - 1 - j : e0 + E + j;
+            if (el < 0 || el >= n) win[j] = ghost_value<T, E>(buf, el, n, a.bc);
+            if (er < 0 || er >= n) win[E + 3 + j] = ghost_value<T, E>(buf, er, n, a.bc);
           }
-          Y[k].x = wenoz_from_beta<T>(wr, bR, sub, dw);
-          Y[E - 1 - (k)].y = wenoz_from_beta<T>(wl, bL, sub, dw);
-#else
-          Y[k].x = wenoz_integral<T>(wr, sub, dw);
-          Y[E - 1 - (k)].y = wenoz_integral<T>(wl, sub, dw);
-#endif
+        }
+      }
+      T dd[E + 5];   // dd[j] = win[j+1] - win[j]
+#pragma unroll
+      for (int j = 0; j < E + 5; ++j) dd[j] = win[j + 1] - win[j];
+      if (JQ == JQ_D0 && a.d0) {
+        const T f0 = pick<T>(a.f0, a.f0f), f1 = pick<T>(a.f1, a.f1f);
+        if (f1 != T(0)) {
+#pragma unroll
+          for (int k = 0; k < E; ++k) {
+            const T s0 = dd[k + 2] - dd[k + 1], s1 = dd[k + 3] - dd[k + 2], s2 = dd[k + 4] - dd[k + 3];
+            F[k] = fma(f1, s0 + s2, f0 * s1);
+          }
         } else {
+#pragma unroll
+          for (int k = 0; k < E; ++k) F[k] = f0 * (dd[k + 3] - dd[k + 2]);
+        }
+#pragma unroll
+        for (int k = 0; k <= E; ++k) X[k] = dd[k + 2];
+      } else if constexpr (!WENO) {
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
           T r = T(0), l = T(0);
 #pragma unroll
-          for (int j = 0; j < 6; ++j) {
-            r = fma(c[j], win[k + j], r);       // v_{e + (j-3)}
-            l = fma(c[j], win[k + 6 - j], l);   // v_{e - (j-3)}
+          for (int i = 0; i < 5; ++i) {
+            r = fma(pick<T>(a.b[i], a.bf[i]), dd[k + i], r);
+            if constexpr (!ONE) l = fma(-pick<T>(a.b[i], a.bf[i]), dd[k + 5 - i], l);
           }
-          Y[k].x = r;
-          Y[E - 1 - (k)].y = l;
-        }
-      }
-    }
-    if (zeroR0) Y[0].x = T(0);
-    if (zeroLN) Y[E - 1 - (E - 1)].y = T(0);
-    // ---- 2a. lane folds (R ascending, L descending, interleaved)
-    T aR, aL, bR, bL;
-    if constexpr (!RAGGED) {
-      const T2 q2 = pair2<T>(q, q);
-      T2 y = pair2<T>(T(0), T(0));
-#pragma unroll
-      for (int k = 0; k < E; ++k) y = fma2(q2, y, Y[k]);
-      aR = qE;
-      aL = qE;
-      bR = y.x;
-      bL = y.y;
-    } else {
-      T r = T(0), l = T(0);
-      aR = T(1);
-      aL = T(1);
-#pragma unroll
-      for (int k = 0; k < E; ++k) {
-        const int e = e0 + k;
-        if (e >= eR0 && e < n) { r = fma(q, r, Y[k].x); aR *= q; }
-        const int eL = e0 + E - 1 - k;
-        if (eL <= eL1) { l = fma(q, l, Y[E - 1 - (E - 1 - k)].y); aL *= q; }
-      }
-      bR = r;
-      bL = l;
-    }
-    // ---- 2b. warp scans (R ascending, L descending)
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const T ap = shfl_up(aR, o), bp = shfl_up(bR, o);
-      const T an = shfl_down(aL, o), bn = shfl_down(bL, o);
-      if (lane >= o) { bR = fma(aR, bp, bR); aR *= ap; }
-      if (lane + o < 32) { bL = fma(aL, bn, bL); aL *= an; }
-    }
-    T exaR = shfl_up(aR, 1), exbR = shfl_up(bR, 1);
-    T exaL = shfl_down(aL, 1), exbL = shfl_down(bL, 1);
-    if (lane == 0) { exaR = T(1); exbR = T(0); }
-    if (lane == 31) { exaL = T(1); exbL = T(0); }
-    T* tot = totals + (lw * nwl) * 4;
-    if constexpr (!WL) {
-      if (lane == 31) { tot[part * 4 + 0] = aR; tot[part * 4 + 1] = bR; }
-      if (lane == 0) { tot[part * 4 + 2] = aL; tot[part * 4 + 3] = bL; }
-      __syncthreads();
-    }
-    // ---- 2c. across the warps of the line
-    T paR = T(1), pbR = T(0), paL = T(1), pbL = T(0);
-    for (int j = 0; j < part; ++j) {
-      const T A = tot[j * 4 + 0], B = tot[j * 4 + 1];
-      pbR = fma(A, pbR, B);
-      paR *= A;
-    }
-    for (int j = nwl - 1; j > part; --j) {
-      const T A = tot[j * 4 + 2], B = tot[j * 4 + 3];
-      pbL = fma(A, pbL, B);
-      paL *= A;
-    }
-    // ---- 3. boundary constants in FP64
-    T cRh, cRl, cLh, cLl;
-    if constexpr (WL) {
-      // lane 31 holds the R line total, lane 0 the L line total
-      const T tbR = __shfl_sync(0xffffffffu, bR, 31);
-      const T tbL = __shfl_sync(0xffffffffu, bL, 0);
-      T c4[4] = {T(0), T(0), T(0), T(0)};
-      if (lane == 0) {
-        double CR, CL;
-        boundary_carries<T, RAGGED, E>(a, buf, n, tbR, tbL, &CR, &CL);
-        split_carry<T>(CR, &c4[0], &c4[1]);
-        split_carry<T>(CL, &c4[2], &c4[3]);
-      }
-      cRh = __shfl_sync(0xffffffffu, c4[0], 0);
-      cRl = __shfl_sync(0xffffffffu, c4[1], 0);
-      cLh = __shfl_sync(0xffffffffu, c4[2], 0);
-      cLl = __shfl_sync(0xffffffffu, c4[3], 0);
-    } else {
-      // vectorised over the CTA's lines: lane w of warp 0 solves line w
-      // (GB300's FP64 pipe is narrow: one warp instruction for all lines)
-      if (warp == 0 && lane < a.W) {
-        const T* tw = totals + (lane * nwl) * 4;
-        T tbR = T(0), tbL = T(0);
-        for (int j = 0; j < nwl; ++j) tbR = fma(tw[j * 4 + 0], tbR, tw[j * 4 + 1]);
-        for (int j = nwl - 1; j >= 0; --j) tbL = fma(tw[j * 4 + 2], tbL, tw[j * 4 + 3]);
-        double CR, CL;
-        boundary_carries<T, RAGGED, E>(a, lines + lane * a.LS, n, tbR, tbL, &CR, &CL);
-        T* cw = reinterpret_cast<T*>(carries) + lane * 4;
-        split_carry<T>(CR, &cw[0], &cw[1]);
-        split_carry<T>(CL, &cw[2], &cw[3]);
-      }
-      __syncthreads();
-      const T* cw = reinterpret_cast<const T*>(carries) + lw * 4;
-      cRh = cw[0];
-      cRl = cw[1];
-      cLh = cw[2];
-      cLl = cw[3];
-    }
-    // ---- 4. carries into the lane and the fix-up passes.  The first power
-    // accumulates I = L^{-1}[v] with |I| ~ |v| and D = v - L^{-1}[v] cancels,
-    // so its recurrences are compensated; later powers act on D^p[v], whose
-    // rounding errors enter S_P scaled by |D^p v| / |v| (already below the
-    // first power's error from the local integrals), so they run plain.
-    {
-      const T laR = exaR * paR, lbR = fma(exaR, pbR, exbR);
-      const T laL = exaL * paL, lbL = fma(exaL, pbL, exbL);
-      if constexpr (!RAGGED) {
-        const T2 q2 = pair2<T>(q, q);
-        if (p == 0 || sizeof(T) == 8) {
-          Acc2<T> y{pair2<T>(fma(laR, cRh, lbR), fma(laL, cLh, lbL)), pair2<T>(laR * cRl, laL * cLl)};
-#pragma unroll
-          for (int k = 0; k < E; ++k) {
-            y.step(q2, Y[k]);
-            Y[k] = y.value();
-          }
-        } else {
-          T2 y = pair2<T>(fma(laR, cRh, lbR) + laR * cRl, fma(laL, cLh, lbL) + laL * cLl);
-#pragma unroll
-          for (int k = 0; k < E; ++k) {
-            y = fma2(q2, y, Y[k]);
-            Y[k] = y;
-          }
+          X[k] = r;
+          if (!ONE) F[k] = l;
         }
       } else {
-        Acc<T> yR{fma(laR, cRh, lbR), laR * cRl};
-        Acc<T> yL{fma(laL, cLh, lbL), laL * cLl};
+        // WENO-Z: indicators from per-triple products; J_R of point k uses
+        // the triples k, k+1, k+2, J_L the triples k+4, k+3, k+2 mirrored
+        T wc[6], dw[3];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) wc[i] = pick<T>(a.wk[i], a.wkf[i]);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) dw[r] = pick<T>(a.d[r], a.df[r]);
+        constexpr int NT = ONE ? E + 2 : E + 4;
+        T p11[NT], p12[NT], p22[NT];
+#pragma unroll
+        for (int t = 0; t < NT; ++t) triple_products<T>(dd[t], dd[t + 1], &p11[t], &p12[t], &p22[t]);
 #pragma unroll
         for (int k = 0; k < E; ++k) {
-          const int e = e0 + k;
-          if (e >= eR0 && e < n) yR.step(q, Y[k].x);
-          Y[k].x = yR.value();
-          const int kl = E - 1 - k;
-          if (e0 + kl <= eL1) yL.step(q, Y[E - 1 - (kl)].y);
-          Y[E - 1 - (kl)].y = yL.value();
-        }
-      }
-    }
-    // ---- 5. D = v - L^{-1}, accumulate, write back for the next power
-    if (a.mode == MODE_RL) {
-      // one-sided derivatives v^- = alpha D_R, v^+ = -alpha D_L and the
-      // per-axis part of the Lax-Friedrichs Hamiltonian (Sec. 2.5)
-      const T al = pick<T>(a.alpha, a.alphaf);
-      if (!GEN || a.ham == HAM_HALF_SQ) {
+          T be[3];
 #pragma unroll
-        for (int k = 0; k < E; ++k) {
-          const T vm = al * (v[k] - Y[k].x);
-          const T vp = -al * (v[k] - Y[E - 1 - (k)].y);
-          const T r = fmax(fabs(vm), fabs(vp));
-          const T mean = T(0.5) * (vm + vp);
-          S[k] = T(0.5) * mean * mean + r * T(0.5) * (vm - vp);
-          if (line_ok && e0 + k < n) rmax = fmax(rmax, r);
-        }
-      } else if constexpr (GEN) {
-        // H_d' = a_d (LINEAR) has |H_d'| = |a_d| everywhere; AFFINE_SQ
-        // leaves (sigma, delta) and the last pass takes the box maximum
-        const T av = pick<T>(a.vel, a.velf), aa = fabs(av);
-        T* cbase2 = static_cast<T*>(sm.lines2) + (cbase - lines);
-#pragma unroll
-        for (int k = 0; k < E; ++k) {
-          const T vm = al * (v[k] - Y[k].x);
-          const T vp = -al * (v[k] - Y[E - 1 - (k)].y);
-          const T mean = T(0.5) * (vm + vp);
-          if (a.ham == HAM_LINEAR) {
-            S[k] = av * mean + aa * T(0.5) * (vm - vp);
+          for (int r = 0; r < 3; ++r) be[r] = beta_from_products<T>(r, p11[k + r], p12[k + r], p22[k + r], false);
+          const T r = wenoz_defect<T>(dd[k + 2], dd[k + 1], dd[k], dd[k + 3], be, wc, dw);
+          if constexpr (ONE) {
+            X[k] = r;
           } else {
-            S[k] = av * mean;
-            if (RAGGED ? e0 + k < n : true) cbase2[chunk_off<E>(k)] = aa * T(0.5) * (vp - vm);
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+              be[j] = beta_from_products<T>(j, p11[k + 4 - j], p12[k + 4 - j], p22[k + 4 - j], true);
+            const T l = wenoz_defect<T>(-dd[k + 3], -dd[k + 4], -dd[k + 5], -dd[k + 2], be, wc, dw);
+            X[k] = r;
+            F[k] = l;
           }
         }
-        if (a.ham == HAM_LINEAR && line_ok) rmax = aa;
+      }
+    }
+    // Dirichlet ends: no forcing at the node where a scan starts
+    const bool resid = JQ == JQ_D0 && a.d0;
+    if (ONE) {
+      if (dir) {
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+          const int e = mir ? e0 + E - 1 - k : e0 + k;
+          if (e == (mir ? n - 1 : 0)) X[k] = T(0);
+        }
+      }
+    } else {
+      if (end0) X[0] = T(0);
+      if (endN) {
+#pragma unroll
+        for (int k = 0; k < E; ++k)
+          if (RAGGED ? e0 + k == n - 1 : k == E - 1) {
+            if (resid) X[k + 1] = T(0); else F[k] = T(0);
+          }
+      }
+    }
+
+    // ---- 2. scans from zero: lane folds, warp scan, warps of the line
+    auto valid = [&](int k) { return !RAGGED || (mir ? e0 + E - 1 - k : e0 + k) < n; };
+    T bR = T(0), bL = T(0);
+#pragma unroll
+    for (int k = 0; k < E; ++k)
+      if (valid(k)) bR = fma(q, bR, X[k]);
+    if constexpr (!ONE) {
+      if (JQ == JQ_D0 && a.d0) {
+#pragma unroll
+        for (int k = E - 1; k >= 0; --k)
+          if (valid(k)) bL = fma(q, bL, -X[k + 1]);
+      } else {
+#pragma unroll
+        for (int k = E - 1; k >= 0; --k)
+          if (valid(k)) bL = fma(q, bL, F[k]);
+      }
+    }
+    const T ownR = bR;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      const int o = 1 << k;
+      const T m = qpow_bit<T>(a, LE + k);
+      const T bp = shfl_up(bR, o);
+      const T sR = fma(m, bp, bR);
+      bR = lane >= o ? sR : bR;
+      if constexpr (!ONE) {
+        const T bn = shfl_down(bL, o);
+        const T sL = fma(m, bn, bL);
+        bL = lane + o < 32 ? sL : bL;
+      }
+    }
+    T cR = shfl_up(bR, 1), cL = T(0);     // value entering the lane from zero before the warp
+    if (lane == 0) cR = T(0);
+    if constexpr (!ONE) {
+      cL = shfl_down(bL, 1);
+      if (lane == 31) cL = T(0);
+    }
+    const T endR = fma(mulR, cR, ownR);   // at lane lastR: the warp's R end value
+    T inR = T(0), inL = T(0), tR, tL = T(0);
+    if (own) {
+      tR = __shfl_sync(FULL, endR, lastR);
+      if constexpr (!ONE) tL = __shfl_sync(FULL, bL, 0);
+    } else {
+      T* tot = totals + lw * nwl * 2;
+      if (lane == lastR) tot[2 * part] = endR;
+      if (!ONE && lane == 0) tot[2 * part + 1] = bL;
+      line_sync(nwl, lw);
+      const int j = lane & 15;
+      const bool left = lane >= 16;
+      T x = T(0);
+      if (j < nwl && !(ONE && left)) x = left ? tot[2 * (nwl - 1 - j) + 1] : tot[2 * j];
+      const T x0 = x;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if ((1 << k) < nwl) {
+          const T xp = __shfl_up_sync(FULL, x, 1 << k, 16);
+          const T sx = fma(qpow_bit<T>(a, LE + 5 + k), xp, x);
+          x = j >= (1 << k) ? sx : x;
+        }
+      }
+      T ex = __shfl_up_sync(FULL, x, 1, 16);   // value entering warp j
+      if (j == 0) ex = T(0);
+      const T lastw = (left || mir) ? qpow_bit<T>(a, LE + 5) : pick<T>(a.qlw, a.qlwf);
+      const T te = fma(lastw, ex, x0);
+      tR = __shfl_sync(FULL, te, nwl - 1);
+      inR = __shfl_sync(FULL, ex, part);
+      if constexpr (!ONE) {
+        tL = __shfl_sync(FULL, te, 15 + nwl);
+        inL = __shfl_sync(FULL, ex, 15 + nwl - part);
+      }
+    }
+    // ---- 3. boundary constants, carried to the lane
+    if (a.close) {
+      inR = fma(qwR, line_constant<T>(a, tR, tL), inR);
+      if constexpr (!ONE) inL = fma(qwL, line_constant<T>(a, tL, tR), inL);
+    }
+    if (a.close || !own) {
+      cR = fma(pwR, inR, cR);
+      if constexpr (!ONE) cL = fma(pwL, inL, cL);
+    }
+    // ---- 4. the scans from their carries -> D of the power (in F; two-sided
+    // forms keep W_R, W_L)
+    T y = cR;
+    if (resid) {
+#pragma unroll
+      for (int k = 0; k < E; ++k) {
+        if (valid(k)) y = fma(q, y, X[k]);
+        F[k] = fma(pick<T>(a.kap, a.kapf), y, F[k]);
+      }
+      y = cL;
+#pragma unroll
+      for (int k = E - 1; k >= 0; --k) {
+        if (valid(k)) y = fma(q, y, -X[k + 1]);
+        F[k] = fma(pick<T>(a.kap, a.kapf), y, F[k]);
       }
     } else {
 #pragma unroll
       for (int k = 0; k < E; ++k) {
-        T linv;
-        if (a.mode == MODE_0) linv = T(0.5) * (Y[k].x + Y[E - 1 - (k)].y);
-        else if (a.mode == MODE_R) linv = Y[k].x;
-        else linv = Y[E - 1 - (k)].y;
-        v[k] = v[k] - linv;
-        S[k] += v[k];
+        if (valid(k)) y = fma(q, y, X[k]);
+        X[k] = y;
+      }
+      if constexpr (ONE) {
+#pragma unroll
+        for (int k = 0; k < E; ++k) F[k] = X[k];
+      } else {
+        y = cL;
+#pragma unroll
+        for (int k = E - 1; k >= 0; --k) {
+          if (valid(k)) y = fma(q, y, F[k]);
+          F[k] = JQ == JQ_D0 ? T(0.5) * (X[k] + y) : y;
+        }
       }
     }
-    if (p + 1 < a.P) {
-      if (WL || own) {
-        __syncwarp();
+    if constexpr (JQ == JQ_D0) {
+      // D_0 vanishes at Dirichlet ends
+      if (end0) F[0] = T(0);
+      if (endN) {
 #pragma unroll
         for (int k = 0; k < E; ++k)
-          if (RAGGED ? e0 + k < n : true) cbase[chunk_off<E>(k)] = v[k];
-        __syncwarp();
-        warp_fill_ghosts<T, E>(a, buf, lane);
-        __syncwarp();
+          if (RAGGED ? e0 + k == n - 1 : k == E - 1) F[k] = T(0);
+      }
+    }
+    // ---- 5. sum over the powers, write back for the next one
+    if constexpr (JQ != JQ_D0 && !ONE) {
+      if (a.mode == MODE_RL) {
+        // one-sided derivatives v^- = alpha D_R, v^+ = -alpha D_L and the
+        // per-axis part of the Lax-Friedrichs Hamiltonian (Sec. 2.5)
+        const T al = pick<T>(a.alpha, a.alphaf);
+        if (!GEN || a.ham == HAM_HALF_SQ) {
+#pragma unroll
+          for (int k = 0; k < E; ++k) {
+            const T vm = al * X[k];
+            const T vp = -al * F[k];
+            const T r = fmax(fabs(vm), fabs(vp));
+            const T mean = T(0.5) * (vm + vp);
+            S[k] = T(0.5) * mean * mean + r * T(0.5) * (vm - vp);
+            if (line_ok && (!RAGGED || e0 + k < n)) rmax = fmax(rmax, r);
+          }
+        } else if constexpr (GEN) {
+          // H_d' = a_d (LINEAR) has |H_d'| = |a_d| everywhere; AFFINE_SQ
+          // leaves (sigma, delta) and the last pass takes the box maximum
+          const T av = pick<T>(a.vel, a.velf), aa = fabs(av);
+          T* cbase2 = static_cast<T*>(sm.lines2) + (cbase - lines);
+#pragma unroll
+          for (int k = 0; k < E; ++k) {
+            const T vm = al * X[k];
+            const T vp = -al * F[k];
+            const T mean = T(0.5) * (vm + vp);
+            if (a.ham == HAM_LINEAR) {
+              S[k] = av * mean + aa * T(0.5) * (vm - vp);
+            } else {
+              S[k] = av * mean;
+              if (RAGGED ? e0 + k < n : true) cbase2[chunk_off<E>(k)] = aa * T(0.5) * (vp - vm);
+            }
+          }
+          if (a.ham == HAM_LINEAR && line_ok) rmax = aa;
+        }
       } else {
-        __syncthreads();
 #pragma unroll
-        for (int k = 0; k < E; ++k)
-          if (RAGGED ? e0 + k < n : true) cbase[chunk_off<E>(k)] = v[k];
-        __syncthreads();
-        fill_ghosts<T, E>(a, lines);
-        __syncthreads();
+        for (int k = 0; k < E; ++k) {
+          T D;
+          if (a.mode == MODE_0) D = T(0.5) * (X[k] + F[k]);
+          else if (a.mode == MODE_R) D = X[k];
+          else D = F[k];
+          F[k] = D;
+        }
+      }
+    }
+    if (JQ == JQ_D0 || ONE || a.mode != MODE_RL) {
+#pragma unroll
+      for (int k = 0; k < E; ++k) S[k] = p == 0 ? F[k] : S[k] + F[k];
+      if (p + 1 < a.P) {
+        // every lane of the line has read its window: of a line of several
+        // warps, before the totals' barrier
+        if (own) __syncwarp();
+        if (!mir) {
+#pragma unroll
+          for (int k = 0; k < E; ++k)
+            if (RAGGED ? e0 + k < n : true) cbase[chunk_off<E>(k)] = F[k];
+        } else {
+#pragma unroll
+          for (int k = 0; k < E; ++k)
+            if (RAGGED ? e0 + E - 1 - k < n : true) cbase[chunk_off<E>(E - 1 - k)] = F[k];
+        }
+        line_sync(nwl, lw);
       }
     }
   }
 
-  if (WL || own) __syncwarp(); else __syncthreads();
+  if (own) __syncwarp();
+  if (!mir) {
 #pragma unroll
-  for (int k = 0; k < E; ++k)
-    if (RAGGED ? e0 + k < n : true) cbase[chunk_off<E>(k)] = S[k];
-  __syncthreads();
+    for (int k = 0; k < E; ++k)
+      if (RAGGED ? e0 + k < n : true) cbase[chunk_off<E>(k)] = S[k];
+  } else {
+#pragma unroll
+    for (int k = 0; k < E; ++k)
+      if (RAGGED ? e0 + E - 1 - k < n : true) cbase[chunk_off<E>(E - 1 - k)] = S[k];
+  }
+  // the epilogue reads contiguous lines by their own warps, strided ones by rows
+  if (a.contiguous) line_sync(nwl, lw); else __syncthreads();
   return cvt<double>(rmax);
-}
-
-#ifndef MOLT_WL_MODE
-#define MOLT_WL_MODE 0
-#endif
-template <typename T, int JQ, bool RAGGED, int E = kE, bool GEN = false>
-__device__ __forceinline__ double compute_lines_any(const SweepArgs& a, const TileSmem& sm, bool line_ok) {
-#if MOLT_WL_MODE == 0
-  return compute_lines<T, JQ, RAGGED, false, E, GEN>(a, sm, line_ok);
-#elif MOLT_WL_MODE == 2
-  return compute_lines<T, JQ, RAGGED, true, E, GEN>(a, sm, line_ok);
-#else
-  if (a.nwl == 1) return compute_lines<T, JQ, RAGGED, true, E, GEN>(a, sm, line_ok);
-  return compute_lines<T, JQ, RAGGED, false, E, GEN>(a, sm, line_ok);
-#endif
 }
 
 // Epilogue operands of one point, loaded ahead of the stores so that the
@@ -1260,7 +1229,7 @@ __device__ __forceinline__ void publish_speed(const SweepArgs& a, double rmax) {
 
 // One tile per CTA, plain coalesced loads (any size / alignment).
 template <typename T, typename TIN, typename TST, int JQ, int EPI, bool RAGGED, int E = kE>
-__global__ void __launch_bounds__(kMaxThreads, kMinBlocks) sweep_kernel(const SweepArgs a) {
+__global__ void __maxnreg__((sweep_regs<T, JQ>())) sweep_kernel(const SweepArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   size_t used;
   const TileSmem sm = carve<T, JQ>(smem_raw, a, &used);
@@ -1269,11 +1238,12 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) sweep_kernel(const Sw
   const long long line0 = (long long)blockIdx.x * a.W;
   const int warp = threadIdx.x >> 5, lw = warp / a.nwl;
   const int tl = (warp - lw * a.nwl) * 32 + (threadIdx.x & 31);
-  load_tile<T, TIN, E>(a, static_cast<const TIN*>(a.in), lines, line0, lw, tl);
-  __syncthreads();
+  load_tile<T, TIN, E>(a, static_cast<const TIN*>(a.in), lines, line0, lw, tl,
+                       [](T* d, const TIN* g) { *d = cvt<T>(*g); });
+  if (a.contiguous && JQ != JQ_LEARNED) line_sync(a.nwl, lw); else __syncthreads();
   if constexpr (epi_hj_x(EPI) || epi_hj_y(EPI)) {
     const double rmax =
-        compute_lines_any<T, JQ, RAGGED, E, epi_hj_gen(EPI)>(a, sm, line0 + lw < a.g.nlines) * a.inv_h;
+        compute_lines<T, JQ, RAGGED, E, epi_hj_gen(EPI)>(a, sm, line0 + lw < a.g.nlines) * a.inv_h;
     // the general last pass finds its speeds in the epilogue
     if constexpr (!epi_hj_gen(EPI)) publish_speed<EPI>(a, rmax);
     const double dt = hj_dt<EPI>(a);
@@ -1281,7 +1251,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) sweep_kernel(const Sw
     const double re = epilogue_tile<T, TST, EPI, E>(a, lines, line0, dt, static_cast<const T*>(sm.lines2));
     if constexpr (epi_hj_gen(EPI)) publish_speed<EPI>(a, fmax(rmax, re));
   } else {
-    compute_lines_any<T, JQ, RAGGED, E>(a, sm, line0 + lw < a.g.nlines);
+    compute_lines<T, JQ, RAGGED, E>(a, sm, line0 + lw < a.g.nlines);
     epilogue_tile<T, TST, EPI, E>(a, lines, line0, 0.0);
   }
 }

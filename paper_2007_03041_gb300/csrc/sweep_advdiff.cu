@@ -4,9 +4,14 @@
 
 namespace molt {
 MOLT_DEFINE_LAUNCH
-MOLT_INST(double, double, double, JQ_LINEAR, EPI_ACC_AXPY)
+MOLT_INST(double, double, double, JQ_D0, EPI_ACC_AXPY)
+MOLT_INST(double, double, double, JQ_LINEAR1, EPI_ACC_AXPY)
 MOLT_INST(double, double, double, JQ_WENOZ, EPI_ACC_AXPY)
-MOLT_INST(float, float, float, JQ_LINEAR, EPI_ACC_AXPY)
+MOLT_INST(double, double, double, JQ_WENOZ1, EPI_ACC_AXPY)
+MOLT_INST(float, float, float, JQ_D0, EPI_ACC_AXPY)
+MOLT_INST(float, float, float, JQ_LINEAR1, EPI_ACC_AXPY)
 MOLT_INST(float, float, float, JQ_WENOZ, EPI_ACC_AXPY)
-MOLT_INST(float, float, double, JQ_LINEAR, EPI_ACC_AXPY)
+MOLT_INST(float, float, float, JQ_WENOZ1, EPI_ACC_AXPY)
+MOLT_INST(float, float, double, JQ_D0, EPI_ACC_AXPY)
+MOLT_INST(float, float, double, JQ_LINEAR1, EPI_ACC_AXPY)
 }  // namespace molt

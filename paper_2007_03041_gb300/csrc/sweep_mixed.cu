@@ -4,11 +4,13 @@
 
 namespace molt {
 MOLT_DEFINE_LAUNCH
-MOLT_INST(float, float, double, JQ_LINEAR, EPI_STORE)
-MOLT_INST(float, float, double, JQ_LINEAR, EPI_ACC_SET)
-MOLT_INST(float, float, double, JQ_LINEAR, EPI_ACC_ADD)
-MOLT_INST(float, float, double, JQ_LINEAR, EPI_HEAT_FINAL)
-MOLT_INST(float, float, double, JQ_LINEAR, EPI_WAVE_FINAL)
-MOLT_INST(float, double, double, JQ_LINEAR, EPI_STORE)
+MOLT_INST(float, float, double, JQ_D0, EPI_STORE)
+MOLT_INST(float, float, double, JQ_D0, EPI_ACC_SET)
+MOLT_INST(float, float, double, JQ_D0, EPI_ACC_ADD)
+MOLT_INST(float, float, double, JQ_D0, EPI_HEAT_FINAL)
+MOLT_INST(float, float, double, JQ_D0, EPI_WAVE_FINAL)
+MOLT_INST(float, double, double, JQ_D0, EPI_STORE)
+MOLT_INST(float, double, double, JQ_LINEAR1, EPI_STORE)
 MOLT_INST(float, double, double, JQ_WENOZ, EPI_STORE)
+MOLT_INST(float, double, double, JQ_WENOZ1, EPI_STORE)
 }  // namespace molt

@@ -203,7 +203,7 @@ __device__ __forceinline__ void transpose_tile(const SweepArgs& a, const TmaGeom
 }
 
 template <typename T, typename TIN, typename TST, int JQ, int EPI>
-__global__ void __launch_bounds__(kMaxThreads, kMinBlocks)
+__global__ void __maxnreg__((sweep_regs<T, JQ>()))
     sweep_tma_kernel(const SweepArgs a, const TmaGeom tg, const __grid_constant__ CUtensorMap map) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   size_t used;
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks)
       }
       prefetch_operands<T, TST, EPI>(a, next * a.W);
     }
-    rmax = fmax(rmax, compute_lines_any<T, JQ, false, kE, epi_hj_gen(EPI)>(a, sm, line0 + lw < a.g.nlines) *
+    rmax = fmax(rmax, compute_lines<T, JQ, false, kE, epi_hj_gen(EPI)>(a, sm, line0 + lw < a.g.nlines) *
                           a.inv_h);
     rmax = fmax(rmax, epilogue_tile<T, TST, EPI>(a, lines, line0, dt, static_cast<const T*>(sm.lines2)));
     __syncthreads();
