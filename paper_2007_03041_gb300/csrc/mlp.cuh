@@ -70,6 +70,20 @@ __device__ __forceinline__ void mlp_load_net(MlpNet& s, const MlpBlob* g) {
   }
 }
 
+// The network with the hidden layers' weights and biases halved (exact): the
+// pre-activations arrive as z/2, the form gelu_half2_pack takes.
+__device__ __forceinline__ void mlp_load_net_half(MlpNet& s, const MlpBlob* g) {
+  mlp_load_net(s, g);
+  __syncthreads();
+  const __nv_bfloat16 half = __float2bfloat16(0.5f);
+  for (int i = threadIdx.x; i < 32 * kLd1; i += blockDim.x) (&s.W1[0][0])[i] = __hmul((&s.W1[0][0])[i], half);
+  for (int i = threadIdx.x; i < 32 * kLd2; i += blockDim.x) (&s.W2[0][0])[i] = __hmul((&s.W2[0][0])[i], half);
+  for (int i = threadIdx.x; i < 32; i += blockDim.x) {
+    s.b1[i] *= 0.5f;
+    s.b2[i] *= 0.5f;
+  }
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&v);
@@ -197,6 +211,93 @@ __device__ __forceinline__ void softmax3(float l0, float l1, float l2, float (&p
   p[0] = e0 * inv;
   p[1] = e1 * inv;
   p[2] = e2 * inv;
+}
+
+// GELU of a pair of pre-activations given as h = z/2: GELU(z) = h + h tanh(v),
+// v = sqrt(2/pi)(z + a z^3) = h (2 c + 8 a c h^2), c = sqrt(2/pi): four
+// packed operations a pair beside the two hardware tanh.
+__device__ __forceinline__ uint32_t gelu_half2_pack(float h0, float h1) {
+  constexpr float kA = 2.f * kGeluC, kB = 8.f * kGeluA * kGeluC;
+  const float2 h = make_float2(h0, h1);
+  const float2 v = __fmul2_rn(h, __ffma2_rn(make_float2(kB, kB), __fmul2_rn(h, h), make_float2(kA, kA)));
+  const float2 g = __ffma2_rn(h, make_float2(tanh_approx(v.x), tanh_approx(v.y)), h);
+  return pack_bf16(g.x, g.y);
+}
+
+// Four 8x8 BF16 tiles from shared memory: lane l gives the address of row l
+// (16 bytes), tile i = rows 8i..8i+7.
+__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], const void* row) {
+  const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(row));
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(a)
+               : "memory");
+}
+
+// Logits of 16 stencils (accumulator layout) from the halved network; a0, a1:
+// the A fragment's column pairs 0..7 of rows g and g+8.
+__device__ __forceinline__ void mlp_logits16_half(const MlpRegs& R, uint32_t a0, uint32_t a1, float (&c3)[4]) {
+  const uint32_t xa[4] = {a0, a1, 0u, 0u};
+  uint32_t h1[2][4], h2[2][4];
+#pragma unroll
+  for (int nt = 0; nt < 4; ++nt) {
+    float c[4] = {R.b1[nt][0], R.b1[nt][1], R.b1[nt][0], R.b1[nt][1]};
+    mma16816(c, xa, R.w1[nt], 0u);
+    h1[nt >> 1][2 * (nt & 1)] = gelu_half2_pack(c[0], c[1]);
+    h1[nt >> 1][2 * (nt & 1) + 1] = gelu_half2_pack(c[2], c[3]);
+  }
+#pragma unroll
+  for (int nt = 0; nt < 4; ++nt) {
+    float c[4] = {R.b2[nt][0], R.b2[nt][1], R.b2[nt][0], R.b2[nt][1]};
+#pragma unroll
+    for (int kk = 0; kk < 2; ++kk) mma16816(c, h1[kk], R.w2[nt][kk][0], R.w2[nt][kk][1]);
+    h2[nt >> 1][2 * (nt & 1)] = gelu_half2_pack(c[0], c[1]);
+    h2[nt >> 1][2 * (nt & 1) + 1] = gelu_half2_pack(c[2], c[3]);
+  }
+  c3[0] = R.b3[0];
+  c3[1] = R.b3[1];
+  c3[2] = R.b3[0];
+  c3[3] = R.b3[1];
+#pragma unroll
+  for (int kk = 0; kk < 2; ++kk) mma16816(c3, h2[kk], R.w3[kk][0], R.w3[kk][1]);
+}
+
+// Warp scratch of a batch of 32 stencils: the BF16 inputs (16 bytes a
+// stencil), then the logits (16 bytes a stencil).
+constexpr int kMlpScratchBytes = 2 * 32 * 16;
+
+// Network outputs of the warp's 32 stencils, one a lane (v: its values).
+// Every lane normalises, and finishes the softmax of, its own stencil; the
+// fragments of the two 16-row products come from shared memory (one 16-byte
+// store a lane, one ldmatrix), the logits go back the same way.
+__device__ __forceinline__ void mlp_eval32(const MlpRegs& R, unsigned char* scratch, int lane, const float (&v)[5],
+                                           float (&p)[3]) {
+  const int g = lane >> 2, t = lane & 3;
+  float x[5];
+  mlp_normalise(v, x);
+  uint4* in = reinterpret_cast<uint4*>(scratch);
+  float4* lg = reinterpret_cast<float4*>(scratch + 32 * 16);
+  in[lane] = make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], 0.f), 0u);
+  __syncwarp();
+  uint32_t a[4];
+  ldmatrix_x4(a, in + lane);
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    float c[4];
+    mlp_logits16_half(R, a[2 * s], a[2 * s + 1], c);
+    // logits 0 and 1 sit in lane t = 0 of the row group, logit 2 in t = 1
+    float4* r0 = lg + 16 * s + g;
+    if (t == 0) {
+      *reinterpret_cast<float2*>(r0) = make_float2(c[0], c[1]);
+      *reinterpret_cast<float2*>(r0 + 8) = make_float2(c[2], c[3]);
+    } else if (t == 1) {
+      r0->z = c[0];
+      (r0 + 8)->z = c[2];
+    }
+  }
+  __syncwarp();
+  const float4 l = lg[lane];
+  softmax3(l.x, l.y, l.z, p);
 }
 
 // Forward pass of 16 stencils: rows g and g+8 of the warp's group.  On return

@@ -358,7 +358,7 @@ molt_status plan_axis(molt_ctx* c, const Problem& p, int ax, int mode, int P, do
   if (a.two_out) out->smem += 16 + size_t(W) * LS * tb;   // second line buffer (carve order)
   if (p.d.weights == MOLT_W_LEARNED) {
     if (!c->mlp_ready) return fail(c, MOLT_EINVAL, "learned weights: call molt_set_mlp first");
-    out->smem += learned_extra_bytes(W, LS);
+    out->smem += learned_extra_bytes(W, LS, nwl);
     a.mlp = static_cast<const MlpBlob*>(c->mlp_blob);
     a.mlp_stats = c->mlp_stats;
   }

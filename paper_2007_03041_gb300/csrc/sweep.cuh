@@ -374,12 +374,13 @@ struct TileSmem {
   void* lines2;      // two_out: [W][LS] of T (delta of AFFINE_SQ)
   float* jloc;       // JQ_LEARNED: [W][2][LS] forcings K_R, K_L
   MlpNet* net;       // JQ_LEARNED: the network
+  unsigned char* mlp_scratch;   // JQ_LEARNED: kMlpScratchBytes per warp
 };
 
 // Shared bytes of a tile beyond the lines for learned weights (the host
 // planner adds the same amount).
-__host__ __device__ constexpr size_t learned_extra_bytes(int W, int LS) {
-  return 16 + size_t(2) * W * LS * sizeof(float) + sizeof(MlpNet);
+__host__ __device__ constexpr size_t learned_extra_bytes(int W, int LS, int nwl) {
+  return 32 + size_t(2) * W * LS * sizeof(float) + sizeof(MlpNet) + size_t(W) * nwl * kMlpScratchBytes;
 }
 
 // Shared bytes before the lines: the warps' totals.
@@ -402,12 +403,15 @@ __device__ __forceinline__ TileSmem carve(unsigned char* smem, const SweepArgs& 
   }
   t.jloc = nullptr;
   t.net = nullptr;
+  t.mlp_scratch = nullptr;
   if constexpr (JQ == JQ_LEARNED) {
     const size_t j0 = (*used + 15) & ~size_t(15);
     t.jloc = reinterpret_cast<float*>(smem + j0);
     const size_t n0 = j0 + size_t(2) * a.W * a.LS * sizeof(float);
     t.net = reinterpret_cast<MlpNet*>(smem + n0);
-    *used = n0 + sizeof(MlpNet);
+    const size_t c0 = (n0 + sizeof(MlpNet) + 15) & ~size_t(15);
+    t.mlp_scratch = smem + c0;
+    *used = c0 + size_t(a.W) * a.nwl * kMlpScratchBytes;
   }
   return t;
 }
@@ -488,15 +492,15 @@ __device__ __forceinline__ void warp_fill_ghosts(const SweepArgs& a, T* b, int l
 }
 
 // Learned local integrals of the points a warp owns (32*E consecutive points
-// of its line from `first`): for 16 points at a time and each side, the lanes
-// gather the 5-value stencils (J_R: v_{e-3..e+1}; J_L mirrored: v_{e+3..e-1})
-// from the staged line, the warp evaluates the network on the tensor cores,
-// and lanes t = 0, 1 of each row group finish rows g, g+8: WENO-Z fallback
-// check, then K = v - q v_prev - sum_r w_r J^{(r)} into jr / jl (shared, line layout).
+// of its line from `first`): 16 points at a time, lanes 0-15 take their J_R
+// stencils (v_{e-3..e+1}), lanes 16-31 the J_L ones (mirrored: v_{e+3..e-1}),
+// the warp evaluates the network on the tensor cores, and every lane finishes
+// its stencil: WENO-Z fallback check, then K = v - q v_prev - sum_r w_r
+// J^{(r)} into jr / jl (shared, line layout).
 template <int E>
 __device__ __forceinline__ void learned_local_integrals(const SweepArgs& a, const MlpNet& net, const float* buf,
-                                                        float* jr, float* jl, int first, int n, int lane) {
-  const int g = lane >> 2, t = lane & 3;
+                                                        float* jr, float* jl, unsigned char* scratch, int first,
+                                                        int n, int lane) {
   MlpRegs R;
   mlp_load_regs(net, lane, R);
   float wk[6], d[3];
@@ -505,42 +509,24 @@ __device__ __forceinline__ void learned_local_integrals(const SweepArgs& a, cons
 #pragma unroll
   for (int i = 0; i < 6; ++i) wk[i] = a.wkf[i];
   unsigned evaluated = 0, fallbacks = 0;
+  const bool left = lane >= 16;
+  float* jk = left ? jl : jr;
   for (int b = 0; b < 32 * E; b += 16) {
     if (first + b >= n) break;   // warp-uniform
-    const int e0 = first + b + g, e1 = e0 + 8;
-    const int c0 = e0 < n ? e0 : n - 1, c1 = e1 < n ? e1 : n - 1;
+    const int e = first + b + (lane & 15), ec = e < n ? e : n - 1;
+    float v[5], p[3];
 #pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      float v0[5], v1[5];
-#pragma unroll
-      for (int j = 0; j < 5; ++j) {
-        const int o = side == 0 ? j - 3 : 3 - j;
-        v0[j] = buf[phys<E>(c0 + o)];
-        v1[j] = buf[phys<E>(c1 + o)];
-      }
-      float x0[5], x1[5];
-      mlp_normalise(v0, x0);
-      mlp_normalise(v1, x1);
-      uint32_t xa[4];
-      mlp_input_frag(x0, x1, t, xa);
-      MlpCache f;
-      float p0[3], p1[3];
-      mlp_forward16(R, xa, f, p0, p1);
-      const int e = t == 0 ? e0 : e1;
-      if (t < 2 && e < n) {
-        float v[5], p[3], w[3];
-#pragma unroll
-        for (int j = 0; j < 5; ++j) v[j] = t == 0 ? v0[j] : v1[j];
-#pragma unroll
-        for (int r = 0; r < 3; ++r) p[r] = t == 0 ? p0[r] : p1[r];
-        fallbacks += mlp_final_weights(v, p, d, w) ? 1u : 0u;
-        ++evaluated;
-        // K = sum_r w_r K_r in difference form (wenoz_defect)
-        const float f0 = v[3] - v[2], f1 = v[2] - v[1], f2 = v[1] - v[0], f = v[4] - v[3];
-        const float K0 = fmaf(wk[1], f2, fmaf(wk[0], f1, f0));
-        const float K1 = fmaf(wk[3], f1, wk[2] * f0), K2 = fmaf(wk[5], f, wk[4] * f0);
-        (side == 0 ? jr : jl)[phys<E>(e)] = fmaf(w[0], K0, fmaf(w[1], K1, w[2] * K2));
-      }
+    for (int j = 0; j < 5; ++j) v[j] = buf[phys<E>(ec + (left ? 3 - j : j - 3))];
+    mlp_eval32(R, scratch, lane, v, p);
+    if (e < n) {
+      float w[3];
+      fallbacks += mlp_final_weights(v, p, d, w) ? 1u : 0u;
+      ++evaluated;
+      // K = sum_r w_r K_r in difference form (wenoz_defect)
+      const float f0 = v[3] - v[2], f1 = v[2] - v[1], f2 = v[1] - v[0], f = v[4] - v[3];
+      const float K0 = fmaf(wk[1], f2, fmaf(wk[0], f1, f0));
+      const float K1 = fmaf(wk[3], f1, wk[2] * f0), K2 = fmaf(wk[5], f, wk[4] * f0);
+      jk[phys<E>(e)] = fmaf(w[0], K0, fmaf(w[1], K1, w[2] * K2));
     }
   }
 #pragma unroll
@@ -667,7 +653,8 @@ __device__ __forceinline__ double compute_lines(const SweepArgs& a, const TileSm
       line_sync(nwl, lw);
       float* jrl = sm.jloc + lw * 2 * a.LS;
       if (line_ok)
-        learned_local_integrals<E>(a, *sm.net, buf, jrl, jrl + a.LS, part * 32 * E, n, lane);
+        learned_local_integrals<E>(a, *sm.net, buf, jrl, jrl + a.LS, sm.mlp_scratch + warp * kMlpScratchBytes,
+                                   part * 32 * E, n, lane);
       __syncwarp();
       lane_powers();
 #pragma unroll
@@ -1233,7 +1220,7 @@ __global__ void __maxnreg__((sweep_regs<T, JQ>())) sweep_kernel(const SweepArgs 
   extern __shared__ __align__(128) unsigned char smem_raw[];
   size_t used;
   const TileSmem sm = carve<T, JQ>(smem_raw, a, &used);
-  if constexpr (JQ == JQ_LEARNED) mlp_load_net(*sm.net, a.mlp);
+  if constexpr (JQ == JQ_LEARNED) mlp_load_net_half(*sm.net, a.mlp);
   T* lines = static_cast<T*>(sm.lines);
   const long long line0 = (long long)blockIdx.x * a.W;
   const int warp = threadIdx.x >> 5, lw = warp / a.nwl;
