@@ -52,7 +52,7 @@ struct Problem {
     double alpha = 0.0;
     int npts = 0;
     int weights = -1;
-    void* dev = nullptr;         // cR[K n], cL[K n], q[n] of the compute type (K = 6, WENO-Z 30)
+    void* dev = nullptr;         // pack_nonuniform tables of the compute type
     size_t count = 0;            // values allocated
   };
   mutable NuCache nu[3];
@@ -1150,7 +1150,8 @@ molt_status apply_D_nonuniform(molt_ctx* c, const Problem& p, int axis, int mode
   const double L = dir ? 0.0 : p.d.hi[axis] - p.d.lo[axis];   // 0: the tables of a Dirichlet line
   const bool f64 = is_f64_sweep(p.d);
   const bool weno = p.d.weights == MOLT_W_WENOZ;
-  const size_t slots = weno ? size_t(kNuWeno) : 6;
+  const int E = nu_points_per_lane(n, f64), nw = std::max(1, (n + 32 * E - 1) / (32 * E));
+  if (nw > kNuMaxWarps) return fail(c, MOLT_EUNSUPPORTED, "non-uniform line longer than 8192 points");
   const size_t tb = f64 ? 8 : 4;
   Problem::NuCache& cch = p.nu[axis];
   const size_t io_bytes = io_compute ? compute_bytes(p.d) : state_bytes(p.d);
@@ -1159,10 +1160,7 @@ molt_status apply_D_nonuniform(molt_ctx* c, const Problem& p, int axis, int mode
     std::vector<double> cR, cL, q;
     build_nonuniform_tables(x, L, alpha, p.d.quad_points, &cR, &cL, &q);
     if (weno) build_nonuniform_weno_tables(x, L, alpha, &cR, &cL);
-    std::vector<double> all(cR);
-    all.insert(all.end(), cL.begin(), cL.end());
-    all.insert(all.end(), q.begin(), q.end());
-    if (all.size() != (2 * slots + 1) * size_t(n)) return fail(c, MOLT_EINVAL, "non-uniform table size");
+    const std::vector<double> all = pack_nonuniform(cR, cL, q, weno, dir, E, int((weno ? 8 : 16) / tb), nw);
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cuda_fail(c, e, "table sync");
     if (cch.dev && cch.count < all.size()) {
       cudaFree(cch.dev);
@@ -1214,45 +1212,58 @@ molt_status apply_D_nonuniform(molt_ctx* c, const Problem& p, int axis, int mode
   a.bc = dir ? 1 : 0;
   if (dir) {
     const double w = x[size_t(n - 1)] - x[0];
-    a.mu = std::exp(-alpha * w);
-    a.kdir = 2.0 / (-std::expm1(-2.0 * alpha * w));
+    // one-sided D starts from W = 0 (L_R^{-1}(a) = v(a)); L_0: W_R(a) =
+    // (mu W_R^0(b) - W_L^0(a)) / (1 - mu^2) and its mirror (Sec. 3.3)
+    if (mode == MODE_0) {
+      const double k = 1.0 / (-std::expm1(-2.0 * alpha * w));
+      a.kA = std::exp(-alpha * w) * k;
+      a.kB = -k;
+      a.close = 2;
+    }
   } else {
-    a.inv1mmu = 1.0 / (-std::expm1(-alpha * L));
+    a.kA = 1.0 / (-std::expm1(-alpha * L));
+    a.close = 1;
   }
+  a.kAh = float(a.kA);
+  a.kAl = float(a.kA - double(a.kAh));
+  a.kBh = float(a.kB);
+  a.kBl = float(a.kB - double(a.kBh));
+  a.tab = cch.dev;
   a.in = kin;
   a.out = kout;
-  a.status = c->status_dev;
-  // one CTA per line, its scan positions split between up to 16 warps (at
-  // most 512 each: the kernel keeps a segment's local integrals in registers)
-  const int nw = std::max(1, (n + 511) / 512);
-  if (nw > 16) return fail(c, MOLT_EUNSUPPORTED, "non-uniform line longer than 8192 points");
-  const size_t smem = (size_t(2 * n + 6) + size_t(2 * nw)) * tb;
-  if (smem > kSmemTileBudget) return fail(c, MOLT_EUNSUPPORTED, "non-uniform line too long for shared memory");
   if (a.g.nlines >= (1LL << 31)) return fail(c, MOLT_EUNSUPPORTED, "more than 2^31 lines along an axis");
-  const long long blocks = a.g.nlines;
-  const int warps = nw;
+  // lines per CTA: two FP32 lines of 8 points a lane share the table reads
+  const int G = E == 8 && !f64 && a.g.nlines >= 4LL * device_sms() ? 2 : 1;
+  const int cap = 32 * E * nw + 3;
+  a.nw = nw;
+  a.LS = (E == 16 ? phys<16>(cap) : (E == 8 ? phys<8>(cap) : phys<4>(cap))) + 1;
+  const size_t smem = (size_t(G + 1) * kNuMaxWarps * 2 + size_t(G) * a.LS) * tb;
+  const long long blocks = (a.g.nlines + G - 1) / G;
   molt_ctx::Rec rec;
   record_begin(c, &rec, MOLT_KERNEL_STORE);
-  auto launch = [&](auto kernel, auto tables) {
+  auto launch = [&](auto kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemOptIn));
-    kernel<<<unsigned(blocks), 32 * warps, smem, c->stream>>>(a, tables);
+    kernel<<<unsigned(blocks), 32 * nw, smem, c->stream>>>(a);
   };
+#define MOLT_NU(T, TIO, E, G)                                  \
+  do {                                                         \
+    if (weno) launch(nonuniform_kernel<T, TIO, true, E, G>);   \
+    else launch(nonuniform_kernel<T, TIO, false, E, G>);       \
+  } while (0)
   if (f64) {
-    const double* d = static_cast<const double*>(cch.dev);
-    NuTables<double> t{d, d + slots * n, d + 2 * slots * n};
-    if (weno) launch(nonuniform_kernel<double, double, true>, t);
-    else launch(nonuniform_kernel<double, double, false>, t);
+    if (E == 4) MOLT_NU(double, double, 4, 1);
+    else if (E == 8) MOLT_NU(double, double, 8, 1);
+    else MOLT_NU(double, double, 16, 1);
+  } else if (io_bytes == 4) {
+    if (E == 16) MOLT_NU(float, float, 16, 1);
+    else if (G == 2) MOLT_NU(float, float, 8, 2);
+    else MOLT_NU(float, float, 8, 1);
   } else {
-    const float* d = static_cast<const float*>(cch.dev);
-    NuTables<float> t{d, d + slots * n, d + 2 * slots * n};
-    if (io_bytes == 4) {
-      if (weno) launch(nonuniform_kernel<float, float, true>, t);
-      else launch(nonuniform_kernel<float, float, false>, t);
-    } else {
-      if (weno) launch(nonuniform_kernel<float, double, true>, t);
-      else launch(nonuniform_kernel<float, double, false>, t);
-    }
+    if (E == 16) MOLT_NU(float, double, 16, 1);
+    else if (G == 2) MOLT_NU(float, double, 8, 2);
+    else MOLT_NU(float, double, 8, 1);
   }
+#undef MOLT_NU
   record_end(c, &rec);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "non-uniform sweep");

@@ -8,12 +8,10 @@
 //
 // Host side: build_nonuniform_tables() integrates the Lagrange basis of each
 // point's stencil against the exponential by 16-point Gauss-Legendre
-// quadrature (FP64).  Device side: one CTA per line, the line staged in
-// shared memory and its scan positions split between the CTA's warps; per D
-// application and direction each warp computes its segment's local integrals
-// once (chunks of 32 x 4 points: per-lane affine maps (q, J), a warp scan of
-// their compositions), the segment maps and the periodic closure give every
-// segment its start value, and the warp replays its chunks from there.
+// quadrature (FP64); pack_nonuniform() brings them into difference form and
+// into the order the kernel's lanes read them.  Device side: the scan of
+// csrc/sweep.cuh (E consecutive points per lane, both directions at once, one
+// CTA barrier per application of D) with a multiplier per point.
 #pragma once
 
 #include <cmath>
@@ -23,26 +21,17 @@
 
 namespace molt {
 
-// Device tables of one (axis, alpha, rule): structure of arrays.  Linear
-// weights: slot m belongs to offset m - 3 (offsets -3..2; unused slots are
-// 0).  WENO-Z: cR, cL hold the kNuWeno-slot tables of
-// build_nonuniform_weno_tables.
-template <typename T>
-struct NuTables {
-  const T* cR;   // [6][n]: J_R(x_i) = sum_m cR[m][i] v_{i + m - 3}   (WENO-Z: [30][n])
-  const T* cL;   // [6][n]: J_L(x_i) = sum_m cL[m][i] v_{i - (m - 3)} (WENO-Z: [30][n])
-  const T* q;    // [n]: q_i = e^{-alpha (x_i - x_{i-1})}
-};
-
 struct NuArgs {
   LineGeom g;
   int mode, P;
   int bc;               // 0 periodic, 1 Dirichlet (nodes x_0 = a .. x_{n-1} = b)
-  double inv1mmu;       // periodic: 1/(1 - mu), mu = e^{-alpha L}
-  double mu, kdir;      // Dirichlet: mu = e^{-alpha (b - a)}, kdir = 2/(1 - mu^2)
+  int nw, LS;           // warps per line, shared line stride (elements)
+  int close;            // boundary constants C = kA T_same + kB T_other: 0 none, 1 kA, 2 both
+  double kA, kB;
+  float kAh, kAl, kBh, kBl;   // kA, kB as FP32 pairs
+  const void* tab;      // device tables (pack_nonuniform) in the compute type
   const void* in;
   void* out;
-  int* status;
 };
 
 // Roots and weights of the n-point Gauss-Legendre rule on [-1, 1] (Newton on
@@ -214,36 +203,118 @@ inline void build_nonuniform_weno_tables(const std::vector<double>& x, double L,
   }
 }
 
-// WENO-Z local integral of point i from its point tables tw ([30][n], layout
-// of build_nonuniform_weno_tables), in difference form: returns
-// (1 - q) v_i - J(x_i) = sum_r w_r sum_j c^{(r)}_j (v_i - v_j), exact since
-// every substencil rule integrates the constant to 1 - q and the normalised
-// weights sum to one.  The five stencil values are taken in the orientation
-// of the direction (J_L reads the mirrored nodes); per substencil r its
-// rule, a = p_t(0) and b = p_tt, beta_r = a^2 - a b + 4/3 b^2, and the
-// WENO-Z map w~_r = d_r (1 + tau/(eps + beta_r)), tau = |beta_0 - beta_2|,
+// Slots of the device tables: decays qR, qL, then per direction the forcing's
+// filter.  Linear rule: b_m, m = -2..2, K_R(x_i) = sum_m b_m d_{i+m}, K_L(x_i)
+// = -sum_m b_m d_{i+1-m} (d_i = v_i - v_{i-1}).  WENO-Z: per direction 21
+// values, in the differences e0 = v_i - v_{i-1}, e1, e2 (further back), f =
+// v_{i+1} - v_i (mirrored for L): the substencil rules K_0 = e0 + k0 e1 + k1
+// e2, K_1 = k2 e0 + k3 e1, K_2 = k4 e0 + k5 f (sum_j c^{(r)}_j = 1 - q makes
+// K_r = v_i - q v_{i-1} - J^{(r)} a filter of the differences), d_r, and per r
+// the two weights each of a = p_t(0) and b = p_tt on the substencil's two
+// differences (their rows sum to zero).
+constexpr int kNuLinSlots = 5, kNuWenoSlots = 21;
+constexpr int kNuMaxWarps = 16;
+inline int nu_slots(bool weno) { return 2 + 2 * (weno ? kNuWenoSlots : kNuLinSlots); }
+
+// Points per lane: the fewest that let 16 warps cover the line (FP32 from 8
+// on: two lines share a CTA's table reads).
+inline int nu_points_per_lane(int n, bool f64) {
+  if (f64 && n <= 4 * 32 * kNuMaxWarps) return 4;
+  return n <= 8 * 32 * kNuMaxWarps ? 8 : 16;
+}
+
+// Index of slot s of point e (lane e / E of the line) in the device tables:
+// groups of V points (nu_group), those of a line's lanes side by side, so that a
+// warp's reads are contiguous.
+inline size_t nu_index(int s, int e, int E, int V, int lanes) {
+  const int lane = e / E, k = e % E;
+  return (size_t(s) * (E / V) + k / V) * lanes * V + size_t(lane) * V + k % V;
+}
+
+// Device tables from the point rules (linear: cR, cL of
+// build_nonuniform_tables; WENO-Z: wR, wL of build_nonuniform_weno_tables),
+// padded with pass-through points (decay 1, no forcing).  Dirichlet lines
+// (L == 0): the scans' start nodes have decay 1, so the start value passes on
+// unchanged (the kernel sets no forcing there).
+inline std::vector<double> pack_nonuniform(const std::vector<double>& cR, const std::vector<double>& cL,
+                                           const std::vector<double>& q, bool weno, bool dirichlet, int E, int V,
+                                           int nw) {
+  const int n = int(q.size()), lanes = 32 * nw, cap = lanes * E, ns = nu_slots(weno);
+  std::vector<double> t(size_t(ns) * cap, 0.0);
+  auto put = [&](int s, int i, double v) { t[nu_index(s, i, E, V, lanes)] = v; };
+  for (int i = 0; i < cap; ++i) {
+    put(0, i, 1.0);
+    put(1, i, 1.0);
+  }
+  for (int i = 0; i < n; ++i) {
+    const double qr = q[size_t(i)], ql = q[size_t(i + 1 < n ? i + 1 : 0)];
+    put(0, i, dirichlet && i == 0 ? 1.0 : qr);
+    put(1, i, dirichlet && i == n - 1 ? 1.0 : ql);
+    for (int side = 0; side < 2; ++side) {
+      const std::vector<double>& c = side == 0 ? cR : cL;
+      const double qd = side == 0 ? qr : ql;
+      auto at = [&](int slot) { return c[size_t(slot) * n + i]; };
+      if (!weno) {
+        const int s0 = 2 + side * kNuLinSlots;
+        put(s0 + 0, i, at(0));
+        put(s0 + 1, i, at(0) + at(1));
+        put(s0 + 2, i, at(0) + at(1) + at(2) + qd);
+        put(s0 + 3, i, -(at(4) + at(5)));
+        put(s0 + 4, i, -at(5));
+      } else {
+        const int s0 = 2 + side * kNuWenoSlots;
+        put(s0 + 0, i, at(0) + at(1));
+        put(s0 + 1, i, at(0));
+        put(s0 + 2, i, 1.0 - at(5));
+        put(s0 + 3, i, at(3));
+        put(s0 + 4, i, at(6) + qd);
+        put(s0 + 5, i, -at(8));
+        for (int r = 0; r < 3; ++r) {
+          put(s0 + 6 + r, i, at(9 + r));
+          put(s0 + 9 + 4 * r, i, -at(12 + 3 * r));
+          put(s0 + 10 + 4 * r, i, at(14 + 3 * r));
+          put(s0 + 11 + 4 * r, i, -at(21 + 3 * r));
+          put(s0 + 12 + 4 * r, i, at(23 + 3 * r));
+        }
+      }
+    }
+  }
+  return t;
+}
+
+// One group of V values of a table.  The loads are volatile: left free, the
+// compiler gathers a whole chunk's tables ahead of the arithmetic and spills
+// them (2 KB a thread with WENO-Z weights).
+template <typename T, int V> struct NuVec { T v[V]; };
+__device__ __forceinline__ void nu_load(NuVec<float, 4>& x, const float* p) {
+  asm volatile("ld.global.nc.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x.v[0]), "=f"(x.v[1]), "=f"(x.v[2]), "=f"(x.v[3]) : "l"(p));
+}
+__device__ __forceinline__ void nu_load(NuVec<float, 2>& x, const float* p) {
+  asm volatile("ld.global.nc.v2.f32 {%0,%1}, [%2];" : "=f"(x.v[0]), "=f"(x.v[1]) : "l"(p));
+}
+__device__ __forceinline__ void nu_load(NuVec<double, 2>& x, const double* p) {
+  asm volatile("ld.global.nc.v2.f64 {%0,%1}, [%2];" : "=d"(x.v[0]), "=d"(x.v[1]) : "l"(p));
+}
+__device__ __forceinline__ void nu_load(NuVec<double, 1>& x, const double* p) {
+  asm volatile("ld.global.nc.f64 %0, [%1];" : "=d"(x.v[0]) : "l"(p));
+}
+// Values per group: 16 bytes, with WENO-Z weights (44 values a point) 8.
+template <typename T, bool WENO>
+__host__ __device__ constexpr int nu_group() { return (WENO ? 8 : 16) / int(sizeof(T)); }
+
+// WENO-Z forcing from the point's 21 table values w (kNuWenoSlots) and its
+// differences in the orientation of the direction: beta_r = a^2 - a b +
+// 4/3 b^2, w~_r = d_r (1 + tau/(eps + beta_r)), tau = |beta_0 - beta_2|,
 // eps = 1e-6 (Sec. 2.4).
-template <typename T, bool LEFT>
-__device__ __forceinline__ T nu_wenoz_defect(const T* tw, const T* v, int n, int i) {
-  T w[5];
-#pragma unroll
-  for (int k = 0; k < 5; ++k) w[k] = LEFT ? v[3 + i - (k - 3)] : v[3 + i + (k - 3)];
-  T Jr[3], beta[3];
+template <typename T>
+__device__ __forceinline__ T nu_wenoz_defect(const T (&w)[kNuWenoSlots], T e0, T e1, T e2, T f) {
+  const T K[3] = {fma(w[1], e2, fma(w[0], e1, e0)), fma(w[3], e1, w[2] * e0), fma(w[5], f, w[4] * e0)};
+  const T lo[3] = {e2, e1, e0}, hi[3] = {e1, e0, f};
+  T beta[3];
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
-    T J = T(0), a = T(0), b = T(0);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      // differences from the centre: the derivative rows sum to zero, so a
-      // and b change sign only (beta is even in (a, b)), and the centre's
-      // term drops
-      if (r + j == 3) continue;
-      const T dj = w[3] - w[r + j];
-      J = fma(tw[(3 * r + j) * n + i], dj, J);
-      a = fma(tw[(12 + 3 * r + j) * n + i], dj, a);
-      b = fma(tw[(21 + 3 * r + j) * n + i], dj, b);
-    }
-    Jr[r] = J;
+    const T a = fma(w[9 + 4 * r], lo[r], w[10 + 4 * r] * hi[r]);
+    const T b = fma(w[11 + 4 * r], lo[r], w[12 + 4 * r] * hi[r]);
     beta[r] = fma(a, a - b, T(4.0 / 3.0) * b * b);
   }
   const T tau = fabs(beta[0] - beta[2]);
@@ -251,205 +322,238 @@ __device__ __forceinline__ T nu_wenoz_defect(const T* tw, const T* v, int n, int
   T num = T(0), sum = T(0);
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
-    const T d = tw[(9 + r) * n + i];
-    const T wt = fma(d * tau, weight_rcp(eps + beta[r]), d);
-    num = fma(wt, Jr[r], num);
+    const T wt = fma(w[6 + r] * tau, weight_rcp(eps + beta[r]), w[6 + r]);
+    num = fma(wt, K[r], num);
     sum += wt;
   }
   return num * weight_rcp(sum);
 }
 
-// One direction, split over the `nw` warps of the line (segment `seg` <= 512
-// scan positions each, R ascending, L descending), in difference form: the
-// scan carries W = v - I, which obeys the recurrence of I with the forcing
-// K_i = v_i - q_i v_{i-1} - J_R(x_i) = sum_l c_{i,l} (v_i - v_{i+l}) +
-// q_i (v_i - v_{i-1}) (mirrored for L; the rules integrate constants to
-// 1 - q_i), so W of constant data is exactly zero and on smooth data its
-// rounding error scales with the differences, not with v.  Each warp
-// computes K and the decays of its segment once (chunks of 32 x 4 points,
-// kept in registers), the per-lane affine maps x -> q x + K composed by a
-// warp scan per chunk; the segments' maps meet in shared memory
-// (maps[2 * nw]) and give the line's end value from W = 0, `all`.  The value
-// entering the line is then k1 * all + start0: the periodic closure (k1 =
-// 1/(1 - mu), start0 = 0) or a Dirichlet line's boundary value of W (the
-// recurrence starts at the end node, whose decay is taken as 1 so that the
-// scan passes the start value on unchanged; K there is zero).  Each warp
-// replays its chunks from its start value and stores by OUT: 0 nothing (the
-// total only), 1 W in w (D_R or D_L, or W_R of L_0), 3 D_0 = (w + W)/2 in w
-// (w holding W_R: the L pass of L_0).  Returns `all`.
-template <typename T, bool LEFT, int OUT, bool WENO>
-__device__ __forceinline__ T nu_direction(const NuTables<T>& tb, const T* v, T* w, int n, int nw, int part, int seg,
-                                          double k1, double start0, bool dirichlet, T* maps, int lane) {
-  constexpr int kPer = 4, kChunks = 4;          // seg <= kChunks * 32 * kPer
-  const int s0 = min(n, part * seg), s1 = min(n, s0 + seg);
-  T jk[kChunks][kPer], qk[kChunks][kPer];
-  T Ae[kChunks], Be[kChunks], At[kChunks], Bt[kChunks];
-  T sA = T(1), sB = T(0);                        // the segment's map
-#pragma unroll
-  for (int c = 0; c < kChunks; ++c) {
-    const int c0 = s0 + c * 32 * kPer;
-    T A = T(1), B = T(0);
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      const int step = c0 + lane * kPer + k;
-      qk[c][k] = T(1);
-      jk[c][k] = T(0);
-      if (step < s1) {
-        const int i = LEFT ? n - 1 - step : step;
-        const T vc = v[3 + i];
-        T K = T(0);
-        if constexpr (WENO) {
-          K = nu_wenoz_defect<T, LEFT>(LEFT ? tb.cL : tb.cR, v, n, i);
-        } else {
-#pragma unroll
-          for (int m = 0; m < 6; ++m) {
-            const int off = m - 3;
-            if (off == 0) continue;          // the centre's difference is 0
-            if (LEFT) K = fma(tb.cL[m * n + i], vc - v[3 + i - off], K);
-            else K = fma(tb.cR[m * n + i], vc - v[3 + i + off], K);
-          }
-        }
-        const T qi = LEFT ? tb.q[i + 1 < n ? i + 1 : 0] : tb.q[i];
-        K = fma(qi, vc - v[3 + i + (LEFT ? 1 : -1)], K);
-        qk[c][k] = (dirichlet && step == 0) ? T(1) : qi;
-        jk[c][k] = K;
-        B = fma(qk[c][k], B, K);
-        A *= qk[c][k];
-      }
-    }
-    // inclusive scan of the lane maps (later lanes apply after)
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const T Ap = __shfl_up_sync(0xffffffffu, A, o), Bp = __shfl_up_sync(0xffffffffu, B, o);
-      if (lane >= o) {
-        B = fma(A, Bp, B);
-        A *= Ap;
-      }
-    }
-    Ae[c] = __shfl_up_sync(0xffffffffu, A, 1);
-    Be[c] = __shfl_up_sync(0xffffffffu, B, 1);
-    if (lane == 0) {
-      Ae[c] = T(1);
-      Be[c] = T(0);
-    }
-    At[c] = __shfl_sync(0xffffffffu, A, 31);
-    Bt[c] = __shfl_sync(0xffffffffu, B, 31);
-    sB = fma(At[c], sB, Bt[c]);
-    sA *= At[c];
-  }
-  if (lane == 0) {
-    maps[2 * part] = sA;
-    maps[2 * part + 1] = sB;
-  }
-  __syncthreads();
-  // value before this segment from W = 0 before the line, and the line's end value
-  T pre = T(0), all = T(0), gA = T(1);
-  for (int j = 0; j < nw; ++j) {
-    if (j == part) pre = all;
-    if (j < part) gA *= maps[2 * j];
-    all = fma(maps[2 * j], all, maps[2 * j + 1]);
-  }
-  if constexpr (OUT == 0) {
-    __syncthreads();   // maps[] is reused by the next pass
-    return all;
-  }
-  // the start value carried through the earlier segments
-  // (the boundary algebra in FP64: 1/(1 - mu) and 2/(1 - mu^2) grow large as
-  // alpha times the line length shrinks)
-  T carry = fma(gA, T(fma(double(all), k1, start0)), pre);
-#pragma unroll
-  for (int c = 0; c < kChunks; ++c) {
-    const int c0 = s0 + c * 32 * kPer;
-    T y = fma(Ae[c], carry, Be[c]);
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      const int step = c0 + lane * kPer + k;
-      if (step < s1) {
-        y = fma(qk[c][k], y, jk[c][k]);
-        const int i = LEFT ? n - 1 - step : step;
-        if constexpr (OUT == 1) w[i] = y;
-        if constexpr (OUT == 3) w[i] = T(0.5) * (w[i] + y);
-      }
-    }
-    carry = fma(At[c], carry, Bt[c]);
-  }
-  __syncthreads();
-  return all;
-}
-
-// S_P along non-uniform lines, periodic or Dirichlet: one CTA of `nw` warps per line (the
-// scan positions split into nw segments of at most 512); shared memory: v
-// (n + 6) and w (n) of T plus the segment maps.  WENO: local integrals by
-// WENO-Z with the point-local tables, else the linear point weights.
-template <typename T, typename TIO, bool WENO>
-// FP32 lines take at most 64 registers (two 512-thread or four 256-thread
-// CTAs per SM: the scans' shuffle chains wait on latency, so more resident
-// warps keep the SM issuing; 4096^2: 1.14 -> 0.94 ms per S_2 step with the
-// linear rule, 2.39 -> 2.20 with WENO-Z); FP64 keeps 128 (it would spill).
-#ifndef MOLT_NU_MIN_BLOCKS_F32
-#define MOLT_NU_MIN_BLOCKS_F32 2
-#endif
-__global__ void __launch_bounds__(512, sizeof(T) == 4 ? MOLT_NU_MIN_BLOCKS_F32 : 1)
-    nonuniform_kernel(const NuArgs a, const NuTables<T> tb) {
+// S_P along non-uniform lines, periodic or Dirichlet, G lines per CTA of `nw`
+// warps: lane tl owns points E tl .. E tl + E - 1 of every line, staged in
+// the padded layout of csrc/sweep.cuh.  W_R = v - L_R^{-1}[v] and W_L obey
+// the recurrences of I with forcings K that are filters of the differences
+// (no value of the size of v is subtracted from another; D of a constant is
+// zero).  The decays' products -- inside the lane, over the lanes of a warp,
+// over the warps of a line -- depend on the tables alone and are formed once
+// per CTA; an application of D then scans one value per lane and direction.
+// Boundary constants (Sec. 2.3, the 2x2 algebra of Sec. 3.3): line_constant.
+// Bound by instructions and by the table reads, 12 values a point (WENO-Z 44)
+// per application and CTA, from L2: G lines share them.
+template <typename T, typename TIO, bool WENO, int E, int G>
+__global__ void __launch_bounds__(512) nonuniform_kernel(const NuArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  const int n = a.g.n;
-  const int nw = blockDim.x >> 5, part = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long line = blockIdx.x;
-  T* v = reinterpret_cast<T*>(smem_raw);
-  T* w = v + n + 6;
-  T* maps = w + n;
-  const int seg = ((n + nw - 1) / nw + 127) / 128 * 128;
-  const long long base = line_base(a.g, line);
-  const long long st = a.g.stride;
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int V = nu_group<T, WENO>(), NS = WENO ? kNuWenoSlots : kNuLinSlots;
+  const int n = a.g.n, nw = a.nw, LS = a.LS;
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5, tl = threadIdx.x;
+  const int e0 = tl * E;
+  T* totals = reinterpret_cast<T*>(smem_raw);        // [G + 1][nw][2]; the last row: the warps' decays
+  T* lines = totals + (G + 1) * kNuMaxWarps * 2;
+  const T* tab = static_cast<const T*>(a.tab);
+  const int tstride = 32 * nw * V;                    // elements of one group of all lanes
+  const long long line0 = (long long)blockIdx.x * G;
   const TIO* in = static_cast<const TIO*>(a.in);
   TIO* out = static_cast<TIO*>(a.out);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) v[3 + i] = T(in[base + i * st]);
-  __syncthreads();
   const bool dir = a.bc == 1;
-  const double k1 = dir ? 0.0 : a.inv1mmu;
+  long long base[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    base[g] = line_base(a.g, line0 + g < a.g.nlines ? line0 + g : a.g.nlines - 1);
+    T* v = lines + g * LS;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += blockDim.x) v[phys<E>(i)] = T(in[base[g] + i * a.g.stride]);
+  }
+  // decays and their products
+  T qR[E], qL[E];
+  auto load_q = [&](int slot, T (&q)[E]) {
+#pragma unroll
+    for (int j = 0; j < E / V; ++j) {
+      NuVec<T, V> x;
+      nu_load(x, tab + (size_t(slot) * (E / V) + j) * tstride + tl * V);
+#pragma unroll
+      for (int k = 0; k < V; ++k) q[j * V + k] = x.v[k];
+    }
+  };
+  load_q(0, qR);
+  load_q(1, qL);
+  T mR[5], mL[5], pwR, pwL;     // multipliers of the warp scan's steps; decay inside the warp before the lane
+  T mX[4], qwR, qwL;            // the same over the warps of the line
+  {
+    T pr = T(1), pl = T(1);
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+      pr *= qR[k];
+      pl *= qL[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      const int o = 1 << k;
+      mR[k] = pr;
+      mL[k] = pl;
+      const T xr = shfl_up(pr, o), xl = shfl_down(pl, o);
+      if (lane >= o) pr *= xr;
+      if (lane + o < 32) pl *= xl;
+    }
+    pwR = shfl_up(pr, 1);
+    pwL = shfl_down(pl, 1);
+    if (lane == 0) pwR = T(1);
+    if (lane == 31) pwL = T(1);
+    T* wd = totals + G * kNuMaxWarps * 2;
+    if (lane == 31) wd[2 * part] = pr;
+    if (lane == 0) wd[2 * part + 1] = pl;
+    __syncthreads();
+    const int j = lane & 15;
+    T x = T(1);
+    if (j < nw) x = lane >= 16 ? wd[2 * (nw - 1 - j) + 1] : wd[2 * j];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      mX[k] = x;
+      const T xp = __shfl_up_sync(FULL, x, 1 << k, 16);
+      if (j >= (1 << k)) x *= xp;
+    }
+    T ex = __shfl_up_sync(FULL, x, 1, 16);
+    if (j == 0) ex = T(1);
+    qwR = __shfl_sync(FULL, ex, part);
+    qwL = __shfl_sync(FULL, ex, 15 + nw - part);
+  }
+  T S[G][E];
   for (int p = 0; p < a.P; ++p) {
-    if (threadIdx.x < 3) {
-      const int j = threadIdx.x + 1;
-      if (dir) {
-        // odd reflection about the end values (mirrored ghost nodes, Sec. 2.3)
-        v[3 - j] = T(2) * v[3] - v[3 + j];
-        v[3 + n - 1 + j] = T(2) * v[3 + n - 1] - v[3 + n - 1 - j];
+    // ghosts (periodic images, or odd reflection about the end values)
+    if (threadIdx.x < 6 * G) {
+      const int g = threadIdx.x / 6, k = threadIdx.x - 6 * g;
+      T* v = lines + g * LS;
+      if (k < 3) {
+        const int j = k + 1;
+        v[phys<E>(-j)] = dir ? T(2) * v[phys<E>(0)] - v[phys<E>(j)] : v[phys<E>(((n - j) % n + n) % n)];
       } else {
-        v[3 - j] = v[3 + ((n - j) % n + n) % n];
-        v[3 + n - 1 + j] = v[3 + (j - 1) % n];
+        const int j = k - 2;
+        v[phys<E>(n - 1 + j)] =
+            dir ? T(2) * v[phys<E>(n - 1)] - v[phys<E>(n - 1 - j)] : v[phys<E>((j - 1) % n)];
       }
     }
     __syncthreads();
-    // D into w: R alone, L alone, or W_R first and then the L pass of L_0.
-    // Dirichlet start values (Sec. 2.3, the 2x2 algebra of Sec. 3.3):
-    // L_R^{-1}(a) = v(a) and L_L^{-1}(b) = v(b), so W starts from 0; for L_0
-    // the passes start from 2A and 2B with [[1, mu], [mu, 1]] (A, B) =
-    // (v(a) - I_0(a), v(b) - I_0(b)), which in terms of the W totals from
-    // zero starts, W_R^0(b) and W_L^0(a), is W_R(a) = (kd/2) (mu W_R^0(b) -
-    // W_L^0(a)) and W_L(b) = (kd/2) (mu W_L^0(a) - W_R^0(b)), kd =
-    // 2/(1 - mu^2): the L total comes first
-    if (a.mode == MODE_R) nu_direction<T, false, 1, WENO>(tb, v, w, n, nw, part, seg, k1, 0.0, dir, maps, lane);
-    if (a.mode == MODE_L) nu_direction<T, true, 1, WENO>(tb, v, w, n, nw, part, seg, k1, 0.0, dir, maps, lane);
-    if (a.mode == MODE_0) {
-      if (!dir) {
-        nu_direction<T, false, 1, WENO>(tb, v, w, n, nw, part, seg, k1, 0.0, false, maps, lane);
-        nu_direction<T, true, 3, WENO>(tb, v, w, n, nw, part, seg, k1, 0.0, false, maps, lane);
-      } else {
-        const double hk = 0.5 * a.kdir, km = hk * a.mu;
-        const double WL =
-            double(nu_direction<T, true, 0, WENO>(tb, v, w, n, nw, part, seg, 0.0, 0.0, true, maps, lane));
-        const double WR =
-            double(nu_direction<T, false, 1, WENO>(tb, v, w, n, nw, part, seg, km, -hk * WL, true, maps, lane));
-        nu_direction<T, true, 3, WENO>(tb, v, w, n, nw, part, seg, km, -hk * WR, true, maps, lane);
+    // differences of the lane's window: dd[j] = v_{e0-2+j} - v_{e0-3+j}
+    T dd[G][E + 5];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const T* c = lines + g * LS + (E + 1) * tl;
+      T w[E + 6];
+#pragma unroll
+      for (int j = 0; j < E + 6; ++j) w[j] = c[chunk_off<E>(j - 3)];
+#pragma unroll
+      for (int j = 0; j < E + 5; ++j) dd[g][j] = w[j + 1] - w[j];
+    }
+    // forcings
+    T KR[G][E], KL[G][E];
+#pragma unroll
+    for (int j = 0; j < E / V; ++j) {
+#pragma unroll
+      for (int side = 0; side < 2; ++side) {
+        NuVec<T, V> t[NS];
+#pragma unroll
+        for (int s = 0; s < NS; ++s)
+          nu_load(t[s], tab + (size_t(2 + side * NS + s) * (E / V) + j) * tstride + tl * V);
+#pragma unroll
+        for (int kk = 0; kk < V; ++kk) {
+          const int k = j * V + kk;
+#pragma unroll
+          for (int g = 0; g < G; ++g) {
+            const T* d = dd[g];
+            T K;
+            if constexpr (WENO) {
+              T w[NS];
+#pragma unroll
+              for (int s = 0; s < NS; ++s) w[s] = t[s].v[kk];
+              K = side == 0 ? nu_wenoz_defect<T>(w, d[k + 2], d[k + 1], d[k], d[k + 3])
+                            : nu_wenoz_defect<T>(w, -d[k + 3], -d[k + 4], -d[k + 5], -d[k + 2]);
+            } else {
+              K = T(0);
+#pragma unroll
+              for (int s = 0; s < 5; ++s) K = fma(t[s].v[kk], side == 0 ? d[k + s] : -d[k + 5 - s], K);
+            }
+            // points past the end, and Dirichlet nodes where a scan starts
+            const int e = e0 + k;
+            if (e >= n || (dir && e == (side == 0 ? 0 : n - 1))) K = T(0);
+            (side == 0 ? KR : KL)[g][k] = K;
+          }
+        }
       }
     }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const T d = w[i];
-      TIO* o = out + base + i * st;
-      *o = p == 0 ? TIO(d) : TIO(T(*o) + d);
-      v[3 + i] = d;
+    // scans from zero
+    T bR[G], bL[G], cR[G], cL[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      bR[g] = bL[g] = T(0);
+#pragma unroll
+      for (int k = 0; k < E; ++k) {
+        bR[g] = fma(qR[k], bR[g], KR[g][k]);
+        bL[g] = fma(qL[E - 1 - k], bL[g], KL[g][E - 1 - k]);
+      }
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        const int o = 1 << k;
+        const T xr = shfl_up(bR[g], o), xl = shfl_down(bL[g], o);
+        const T nr = fma(mR[k], xr, bR[g]), nl = fma(mL[k], xl, bL[g]);
+        bR[g] = lane >= o ? nr : bR[g];
+        bL[g] = lane + o < 32 ? nl : bL[g];
+      }
+      cR[g] = shfl_up(bR[g], 1);
+      cL[g] = shfl_down(bL[g], 1);
+      if (lane == 0) cR[g] = T(0);
+      if (lane == 31) cL[g] = T(0);
+      T* tot = totals + g * kNuMaxWarps * 2;
+      if (lane == 31) tot[2 * part] = bR[g];
+      if (lane == 0) tot[2 * part + 1] = bL[g];
     }
     __syncthreads();
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const T* tot = totals + g * kNuMaxWarps * 2;
+      const int j = lane & 15;
+      T x = T(0);
+      if (j < nw) x = lane >= 16 ? tot[2 * (nw - 1 - j) + 1] : tot[2 * j];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if ((1 << k) < nw) {
+          const T xp = __shfl_up_sync(FULL, x, 1 << k, 16);
+          const T nx = fma(mX[k], xp, x);
+          x = j >= (1 << k) ? nx : x;
+        }
+      }
+      T ex = __shfl_up_sync(FULL, x, 1, 16);
+      if (j == 0) ex = T(0);
+      T inR = __shfl_sync(FULL, ex, part), inL = __shfl_sync(FULL, ex, 15 + nw - part);
+      if (a.close) {
+        const T tR = __shfl_sync(FULL, x, nw - 1), tL = __shfl_sync(FULL, x, 15 + nw);
+        inR = fma(qwR, line_constant<T>(a, tR, tL), inR);
+        inL = fma(qwL, line_constant<T>(a, tL, tR), inL);
+      }
+      T yR = fma(pwR, inR, cR[g]), yL = fma(pwL, inL, cL[g]);
+#pragma unroll
+      for (int k = 0; k < E; ++k) {
+        yR = fma(qR[k], yR, KR[g][k]);
+        KR[g][k] = yR;
+        yL = fma(qL[E - 1 - k], yL, KL[g][E - 1 - k]);
+        KL[g][E - 1 - k] = yL;
+      }
+      T* c = lines + g * LS + (E + 1) * tl;
+#pragma unroll
+      for (int k = 0; k < E; ++k) {
+        const T D = a.mode == MODE_0 ? T(0.5) * (KR[g][k] + KL[g][k]) : (a.mode == MODE_R ? KR[g][k] : KL[g][k]);
+        S[g][k] = p == 0 ? D : S[g][k] + D;
+        // (every lane read its window before the totals' barrier)
+        if (e0 + k < n) c[chunk_off<E>(k)] = p + 1 < a.P ? D : S[g][k];
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    if (line0 + g >= a.g.nlines) break;
+    const T* v = lines + g * LS;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += blockDim.x) out[base[g] + i * a.g.stride] = TIO(v[phys<E>(i)]);
   }
 }
 
