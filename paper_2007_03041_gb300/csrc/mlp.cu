@@ -28,6 +28,7 @@ using namespace molt;
 namespace {
 
 constexpr int kGradWarps = 4;   // warps per CTA of the gradient kernel
+constexpr int kBlobBlocks = (int(sizeof(MlpBlob) / 2) + 127) / 128;
 
 int sm_count() {
   int dev = 0, sms = 148;
@@ -38,47 +39,46 @@ int sm_count() {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-// FP32 master parameters -> BF16 blob, by all threads of one CTA.  The blob
-// is one array of BF16: W1 (32x16), W2 (32x32), W3 (8x32), b1, b2, b3 (8).
-__device__ void pack_blob(const float* theta, MlpBlob* blob) {
-  __nv_bfloat16* o = &blob->W1[0][0];
-  for (int f = threadIdx.x; f < int(sizeof(MlpBlob) / 2); f += blockDim.x) {
-    float v = 0.f;
-    if (f < 512) {
-      const int r = f >> 4, c = f & 15;
-      if (c < 5) v = theta[kOffW1 + r * 5 + c];
-    } else if (f < 1536) {
-      v = theta[kOffW2 + (f - 512)];
-    } else if (f < 1792) {
-      const int r = (f - 1536) >> 5, c = (f - 1536) & 31;
-      if (r < 3) v = theta[kOffW3 + r * 32 + c];
-    } else if (f < 1824) {
-      v = theta[kOffB1 + (f - 1792)];
-    } else if (f < 1856) {
-      v = theta[kOffB2 + (f - 1824)];
-    } else if (f - 1856 < 3) {
-      v = theta[kOffB3 + (f - 1856)];
-    }
-    o[f] = __float2bfloat16_rn(v);
-  }
+// Parameter behind element f of the blob (-1: padding).
+__device__ __forceinline__ int blob_param(int f) {
+  if (f < 512) return (f & 15) < 5 ? kOffW1 + (f >> 4) * 5 + (f & 15) : -1;
+  if (f < 1536) return kOffW2 + (f - 512);
+  if (f < 1792) return f - 1536 < 96 ? kOffW3 + (f - 1536) : -1;
+  if (f < 1824) return kOffB1 + (f - 1792);
+  if (f < 1856) return kOffB2 + (f - 1824);
+  return f - 1856 < 3 ? kOffB3 + (f - 1856) : -1;
 }
 
-__global__ void mlp_pack_kernel(const float* __restrict__ theta, MlpBlob* blob) { pack_blob(theta, blob); }
+// FP32 master parameters -> BF16 blob (one array of BF16: W1 32x16, W2 32x32,
+// W3 8x32, b1, b2, b3).
+__global__ void mlp_pack_kernel(const float* __restrict__ theta, MlpBlob* blob) {
+  const int f = blockIdx.x * blockDim.x + threadIdx.x;
+  if (f >= int(sizeof(MlpBlob) / 2)) return;
+  const int i = blob_param(f);
+  (&blob->W1[0][0])[f] = __float2bfloat16_rn(i >= 0 ? theta[i] : 0.f);
+}
 
+// One thread per element of the BF16 blob, each parameter's step taken by the
+// thread that packs it: one pass, no barrier, spread over CTAs (one CTA for
+// the whole network, packing from memory after a barrier, took 5.9 us).
 // b1, b2 and their complements 1-b1, 1-b2 come rounded from FP64 (1 - 0.999f
 // in FP32 would be off by 1.3e-5 relative).
 __global__ void mlp_adam_kernel(float* theta, float* m, float* v, const float* __restrict__ grad, float lr, float b1,
                                 float omb1, float b2, float omb2, float eps, float bc1, float bc2, MlpBlob* blob) {
-  for (int i = threadIdx.x; i < kMlpParams; i += blockDim.x) {
+  const int f = blockIdx.x * blockDim.x + threadIdx.x;
+  if (f >= int(sizeof(MlpBlob) / 2)) return;
+  const int i = blob_param(f);
+  float t = 0.f;
+  if (i >= 0) {
     const float g = grad[i];
     const float mi = fmaf(b1, m[i], omb1 * g);
     const float vi = fmaf(b2, v[i], omb2 * g * g);
     m[i] = mi;
     v[i] = vi;
-    theta[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+    t = theta[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+    theta[i] = t;
   }
-  __syncthreads();
-  pack_blob(theta, blob);
+  (&blob->W1[0][0])[f] = __float2bfloat16_rn(t);
 }
 
 __device__ __forceinline__ void load_stencil(const float* x, long long row, float (&v)[5]) {
@@ -183,11 +183,7 @@ __global__ void __launch_bounds__(32 * kGradWarps) mlp_grad_kernel(const MlpBlob
   __shared__ __align__(16) __nv_bfloat16 W2T[32][kLd2];   // [in][out]
   __shared__ __align__(16) __nv_bfloat16 W3T[32][kLd1];   // [hidden][out], outputs 3.. zero
   __shared__ __align__(16) WarpStage stage[kGradWarps];
-  __shared__ float gacc[kMlpParams];
-  __shared__ float lacc;
   mlp_load_net(net, blob);
-  for (int i = threadIdx.x; i < kMlpParams; i += blockDim.x) gacc[i] = 0.f;
-  if (threadIdx.x == 0) lacc = 0.f;
   __syncthreads();
   for (int i = threadIdx.x; i < 32 * kLd2; i += blockDim.x) {
     const int r = i / kLd2, c = i - r * kLd2;   // r = in, c = out
@@ -343,25 +339,39 @@ __global__ void __launch_bounds__(32 * kGradWarps) mlp_grad_kernel(const MlpBlob
     __syncwarp();
   }
 
-  // reduce: registers -> CTA (shared atomics) -> global
+  // reduce: each warp's sums to its own row of shared memory (every value has
+  // one owning lane; biases over the row groups by shuffles), the rows to
+  // global memory.  (FP32 atomics on shared memory are compare-and-swap loops.)
+  // The rows lie over the warps' operand stages, whose last reads are done.
+  static_assert(sizeof(WarpStage) >= (kMlpParams + 1) * sizeof(float), "a row of sums fits a stage");
+  float* ga = reinterpret_cast<float*>(&stage[warp]);
+  auto over_rows = [](float x) {
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+  };
 #pragma unroll
   for (int nt = 0; nt < 4; ++nt) {
     if (g < 3) {
-      atomicAdd(&gacc[kOffW3 + g * 32 + nt * 8 + 2 * t], dW3[nt][0]);
-      atomicAdd(&gacc[kOffW3 + g * 32 + nt * 8 + 2 * t + 1], dW3[nt][1]);
+      ga[kOffW3 + g * 32 + nt * 8 + 2 * t] = dW3[nt][0];
+      ga[kOffW3 + g * 32 + nt * 8 + 2 * t + 1] = dW3[nt][1];
     }
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt) {
       const int o = mt * 16 + g, i = nt * 8 + 2 * t;
-      atomicAdd(&gacc[kOffW2 + o * 32 + i], dW2[mt][nt][0]);
-      atomicAdd(&gacc[kOffW2 + o * 32 + i + 1], dW2[mt][nt][1]);
-      atomicAdd(&gacc[kOffW2 + (o + 8) * 32 + i], dW2[mt][nt][2]);
-      atomicAdd(&gacc[kOffW2 + (o + 8) * 32 + i + 1], dW2[mt][nt][3]);
+      ga[kOffW2 + o * 32 + i] = dW2[mt][nt][0];
+      ga[kOffW2 + o * 32 + i + 1] = dW2[mt][nt][1];
+      ga[kOffW2 + (o + 8) * 32 + i] = dW2[mt][nt][2];
+      ga[kOffW2 + (o + 8) * 32 + i + 1] = dW2[mt][nt][3];
     }
-    atomicAdd(&gacc[kOffB1 + nt * 8 + 2 * t], db1[nt][0]);
-    atomicAdd(&gacc[kOffB1 + nt * 8 + 2 * t + 1], db1[nt][1]);
-    atomicAdd(&gacc[kOffB2 + nt * 8 + 2 * t], db2[nt][0]);
-    atomicAdd(&gacc[kOffB2 + nt * 8 + 2 * t + 1], db2[nt][1]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float s1 = over_rows(db1[nt][h]), s2 = over_rows(db2[nt][h]);
+      if (g == 0) {
+        ga[kOffB1 + nt * 8 + 2 * t + h] = s1;
+        ga[kOffB2 + nt * 8 + 2 * t + h] = s2;
+      }
+    }
   }
 #pragma unroll
   for (int mt = 0; mt < 2; ++mt) {
@@ -370,21 +380,26 @@ __global__ void __launch_bounds__(32 * kGradWarps) mlp_grad_kernel(const MlpBlob
     for (int h = 0; h < 2; ++h) {
       const int i = 2 * t + h;
       if (i < 5) {
-        atomicAdd(&gacc[kOffW1 + o * 5 + i], dW1[mt][h]);
-        atomicAdd(&gacc[kOffW1 + (o + 8) * 5 + i], dW1[mt][2 + h]);
+        ga[kOffW1 + o * 5 + i] = dW1[mt][h];
+        ga[kOffW1 + (o + 8) * 5 + i] = dW1[mt][2 + h];
       }
     }
   }
-  if (t == 0) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) atomicAdd(&gacc[kOffB3 + k], db3[k]);
+  for (int k = 0; k < 3; ++k) {
+    const float s3 = over_rows(db3[k]);   // (t = 0 lanes hold the sums)
+    if (lane == 0) ga[kOffB3 + k] = s3;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-  if (lane == 0) atomicAdd(&lacc, lsum);
+  lsum = over_rows(lsum);
+  if (lane == 0) ga[kMlpParams] = lsum;
   __syncthreads();
-  for (int i = threadIdx.x; i < kMlpParams; i += blockDim.x) atomicAdd(&grad[i], gacc[i]);
-  if (threadIdx.x == 0) atomicAdd(loss, lacc / float(n));
+  for (int i = threadIdx.x; i <= kMlpParams; i += blockDim.x) {
+    float x = 0.f;
+#pragma unroll
+    for (int w = 0; w < kGradWarps; ++w) x += reinterpret_cast<const float*>(&stage[w])[i];
+    if (i < kMlpParams) atomicAdd(&grad[i], x);
+    else atomicAdd(loss, x / float(n));
+  }
 }
 
 __global__ void mlp_harvest_kernel(const float* __restrict__ u, long long nx, long long ny,
@@ -463,7 +478,7 @@ molt_status molt_quadrature_weights(int quad_points, double nu, double* c, doubl
 
 molt_status molt_mlp_pack(const float* theta, void* blob, void* cuda_stream) {
   if (!theta || !blob || !aligned16(theta) || !aligned16(blob)) return MOLT_EINVAL;
-  mlp_pack_kernel<<<1, 512, 0, static_cast<cudaStream_t>(cuda_stream)>>>(theta, static_cast<MlpBlob*>(blob));
+  mlp_pack_kernel<<<kBlobBlocks, 128, 0, static_cast<cudaStream_t>(cuda_stream)>>>(theta, static_cast<MlpBlob*>(blob));
   return launched();
 }
 
@@ -502,7 +517,7 @@ molt_status molt_mlp_adam(float* theta, float* m, float* v, const float* grad, i
     return MOLT_EINVAL;
   const double bc1 = 1.0 - std::pow(beta1, double(step));
   const double bc2 = 1.0 - std::pow(beta2, double(step));
-  mlp_adam_kernel<<<1, 512, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
+  mlp_adam_kernel<<<kBlobBlocks, 128, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
       theta, m, v, grad, float(lr), float(beta1), float(1.0 - beta1), float(beta2), float(1.0 - beta2), float(eps),
       float(bc1), float(bc2),
       static_cast<MlpBlob*>(blob));
