@@ -988,8 +988,8 @@ def config_line(name, steps, warmup, compare=True, error=True, size=None):
              "paper_ex1_advection": (("hj_x", M.KERNEL_HJ_X), ("hj_y", M.KERNEL_HJ_Y),
                                      ("transpose", M.KERNEL_TRANSPOSE)),
              "paper_ex2_diffusion": (("sweep_final", M.KERNEL_HEAT_FINAL), ("sweep_acc", M.KERNEL_ACC_SET)),
-             "advdiff_burgers4096": (("flux", M.KERNEL_FLUX), ("sweeps", M.KERNEL_ACC_ADD),
-                                     ("sweeps_lanes", M.KERNEL_LANES_ACC_ADD), ("update", M.KERNEL_UPDATE)),
+             "advdiff_burgers4096": (("axes", M.KERNEL_ACC_ADD), ("transpose", M.KERNEL_TRANSPOSE),
+                                     ("update", M.KERNEL_UPDATE)),
              "paper_ex3_hj": (("hj_x", M.KERNEL_HJ_X), ("hj_y", M.KERNEL_HJ_Y))}[name]
     flush = bool(cfg.get("flush_l2"))
     ms, us, per_kind, stats, clk = _timed_steps(name, steps, warmup, blob=blob, profile_kinds=kinds, clocks=True,

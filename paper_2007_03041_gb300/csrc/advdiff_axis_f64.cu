@@ -1,0 +1,6 @@
+// The fused advection-diffusion axis kernel (csrc/advdiff_axis.cuh), FP64.
+#include "advdiff_axis_launch.h"
+
+namespace molt {
+template cudaError_t launch_advdiff_axis_t<double>(bool, int, const AdvArgs&, int, int, size_t, cudaStream_t);
+}  // namespace molt

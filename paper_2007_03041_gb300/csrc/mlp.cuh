@@ -42,31 +42,38 @@ static_assert(sizeof(MlpBlob) == 3728, "blob layout");
 // Shared-memory copy with padded rows: the B-fragment loads of a warp (word
 // 12g+t resp. 20g+t) fall in 32 distinct banks.
 constexpr int kLd1 = 24, kLd2 = 40;
-struct MlpNet {
+struct alignas(16) MlpNet {
   __nv_bfloat16 W1[32][kLd1];
   __nv_bfloat16 W2[32][kLd2];
   __nv_bfloat16 W3[8][kLd2];
   float b1[32], b2[32], b3[8];
 };
 
+// 16-byte copies (the blob is 16-byte aligned; columns beyond a row's own are
+// never read).
 __device__ __forceinline__ void mlp_load_net(MlpNet& s, const MlpBlob* g) {
-  const __nv_bfloat16 z = __float2bfloat16(0.f);
-  for (int i = threadIdx.x; i < 32 * kLd1; i += blockDim.x) {
-    const int r = i / kLd1, c = i - r * kLd1;
-    s.W1[r][c] = c < 16 ? g->W1[r][c] : z;
-  }
-  for (int i = threadIdx.x; i < 32 * kLd2; i += blockDim.x) {
-    const int r = i / kLd2, c = i - r * kLd2;
-    s.W2[r][c] = c < 32 ? g->W2[r][c] : z;
-  }
-  for (int i = threadIdx.x; i < 8 * kLd2; i += blockDim.x) {
-    const int r = i / kLd2, c = i - r * kLd2;
-    s.W3[r][c] = c < 32 ? g->W3[r][c] : z;
-  }
-  for (int i = threadIdx.x; i < 32; i += blockDim.x) {
-    s.b1[i] = __bfloat162float(g->b1[i]);
-    s.b2[i] = __bfloat162float(g->b2[i]);
-    if (i < 8) s.b3[i] = __bfloat162float(g->b3[i]);
+  const uint4* src = reinterpret_cast<const uint4*>(g);
+  constexpr int kW1 = 32 * 2, kW2 = 32 * 4, kW3 = 8 * 4, kAll = int(sizeof(MlpBlob) / 16);
+  for (int f = threadIdx.x; f < kAll; f += blockDim.x) {
+    const uint4 x = src[f];
+    if (f < kW1) {
+      *reinterpret_cast<uint4*>(&s.W1[f >> 1][8 * (f & 1)]) = x;
+    } else if (f < kW1 + kW2) {
+      const int k = f - kW1;
+      *reinterpret_cast<uint4*>(&s.W2[k >> 2][8 * (k & 3)]) = x;
+    } else if (f < kW1 + kW2 + kW3) {
+      const int k = f - kW1 - kW2;
+      *reinterpret_cast<uint4*>(&s.W3[k >> 2][8 * (k & 3)]) = x;
+    } else {
+      const int k = f - kW1 - kW2 - kW3;   // biases: 4 + 4 + 1 groups of 8
+      float* b = k < 4 ? s.b1 + 8 * k : (k < 8 ? s.b2 + 8 * (k - 4) : s.b3);
+      const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        b[2 * h] = __uint_as_float(w[h] << 16);
+        b[2 * h + 1] = __uint_as_float(w[h] & 0xFFFF0000u);
+      }
+    }
   }
 }
 
@@ -75,9 +82,13 @@ __device__ __forceinline__ void mlp_load_net(MlpNet& s, const MlpBlob* g) {
 __device__ __forceinline__ void mlp_load_net_half(MlpNet& s, const MlpBlob* g) {
   mlp_load_net(s, g);
   __syncthreads();
-  const __nv_bfloat16 half = __float2bfloat16(0.5f);
-  for (int i = threadIdx.x; i < 32 * kLd1; i += blockDim.x) (&s.W1[0][0])[i] = __hmul((&s.W1[0][0])[i], half);
-  for (int i = threadIdx.x; i < 32 * kLd2; i += blockDim.x) (&s.W2[0][0])[i] = __hmul((&s.W2[0][0])[i], half);
+  const __nv_bfloat162 half = __floats2bfloat162_rn(0.5f, 0.5f);
+  auto halve = [&](__nv_bfloat16* p) {
+    __nv_bfloat162* q = reinterpret_cast<__nv_bfloat162*>(p);
+    *q = __hmul2(*q, half);
+  };
+  for (int i = threadIdx.x; i < 32 * 8; i += blockDim.x) halve(&s.W1[i >> 3][2 * (i & 7)]);
+  for (int i = threadIdx.x; i < 32 * 16; i += blockDim.x) halve(&s.W2[i >> 4][2 * (i & 15)]);
   for (int i = threadIdx.x; i < 32; i += blockDim.x) {
     s.b1[i] *= 0.5f;
     s.b2[i] *= 0.5f;

@@ -18,6 +18,7 @@
 #include "sweep_launch.h"
 #include "sweep_lanes_launch.h"
 #include "batch.cuh"
+#include "advdiff_axis.cuh"
 
 using namespace molt;
 
@@ -1544,6 +1545,127 @@ __global__ void advdiff_update_kernel(const TC* __restrict__ acc, const TS* un, 
   if (bad) atomicOr(status, ST_NONFINITE);
 }
 
+// The last axis's sums on the transposed grid (st, x-major) with the update:
+// dst = a0 u^n + a1 (u_s + (acc + st^T)), through 64 x 64 tiles.
+template <typename T>
+__global__ void advdiff_update_t_kernel(const T* __restrict__ acc, const T* __restrict__ st, const T* un, const T* us,
+                                        T* dst, double a0, double a1, long long ny, long long nx, int* status) {
+  __shared__ T tile[64][65];
+  const long long x0 = (long long)blockIdx.x * 64, y0 = (long long)blockIdx.y * 64;
+  T v[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const long long x = x0 + threadIdx.y + 8 * (k >> 1), y = y0 + threadIdx.x + 32 * (k & 1);
+    v[k] = (x < nx && y < ny) ? st[x * ny + y] : T(0);
+  }
+#pragma unroll
+  for (int k = 0; k < 16; ++k) tile[threadIdx.y + 8 * (k >> 1)][threadIdx.x + 32 * (k & 1)] = v[k];
+  __syncthreads();
+  T w[16], z[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const int j = threadIdx.y + 8 * (k >> 1), i = threadIdx.x + 32 * (k & 1);
+    const long long x = x0 + i, y = y0 + j;
+    if (x < nx && y < ny) {
+      v[k] = acc[y * nx + x] + tile[i][j];
+      w[k] = un[y * nx + x];
+      z[k] = us[y * nx + x];
+    }
+  }
+  bool bad = false;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const long long x = x0 + threadIdx.x + 32 * (k & 1), y = y0 + threadIdx.y + 8 * (k >> 1);
+    if (x < nx && y < ny) {
+      const T r = fma(T(a0), w[k], T(a1) * (z[k] + v[k]));
+      dst[y * nx + x] = r;
+      bad |= nonfinite(r);
+    }
+  }
+  if (bad) atomicOr(status, ST_NONFINITE);
+}
+
+// The fused axis kernel takes stages with one term per sum on uniform axes
+// (periodic: molt_create takes no others) and a state in the sweeps' type
+// (mixed precision forms the fluxes from the FP64 state).
+bool advdiff_fused(const Problem& p) {
+  if (p.d.P != 1 || is_mixed(p.d) || p.d.weights == MOLT_W_LEARNED) return false;
+  for (int ax = 0; ax < p.d.ndim; ++ax)
+    if (!p.nodes[ax].empty()) return false;
+  return true;
+}
+
+molt_status advdiff_stage_fused(molt_ctx* c, Problem& p, const void* un, const void* us, void* dst, double a0,
+                                double a1) {
+  const double dt = p.d.dt, cb = p.d.c, beta = p.d.beta, kappa = p.d.diffusivity;
+  const bool f64 = is_f64_sweep(p.d), weno = p.d.weights == MOLT_W_WENOZ;
+  const size_t el = state_bytes(p.d);
+  cudaError_t e;
+  molt_status st;
+  auto axis = [&](const Problem& q, int ax, double vel, int epi, const void* in, void* acc) {
+    Plan pl, dif;
+    if ((st = plan_axis(c, q, ax, MODE_R, 1, beta / (cb * dt), &pl)) != MOLT_OK) return st;
+    AdvArgs A{};
+    if (kappa > 0) {
+      if ((st = plan_axis(c, q, ax, MODE_0, 1, beta / std::sqrt(kappa * dt), &dif)) != MOLT_OK) return st;
+      A.dif = dif.a;
+    }
+    pl.a.in = in;
+    pl.a.acc = acc;
+    pl.a.un = un;
+    pl.a.us = us;
+    pl.a.dst = dst;
+    pl.a.a0 = a0;
+    pl.a.a1 = a1;
+    A.a = pl.a;
+    A.burgers = q.d.flux == MOLT_FLUX_BURGERS ? 1 : 0;
+    A.diffusive = kappa > 0 ? 1 : 0;
+    A.c = cb;
+    A.vel = vel;
+    // -dt alpha S_R[g^+] + dt alpha S_L[g^-]  (dt alpha = beta / c)
+    A.cR = -beta / cb;
+    A.cL = beta / cb;
+    A.cD = -beta * beta;
+    molt_ctx::Rec rec;
+    record_begin(c, &rec, MOLT_KERNEL_ACC_ADD);
+    e = f64 ? launch_advdiff_axis_t<double>(weno, epi, A, pl.grid, pl.block, pl.smem, c->stream)
+            : launch_advdiff_axis_t<float>(weno, epi, A, pl.grid, pl.block, pl.smem, c->stream);
+    record_end(c, &rec);
+    return e == cudaSuccess ? MOLT_OK : cuda_fail(c, e, "advection-diffusion axis");
+  };
+  for (int ax = 0; ax < p.d.ndim; ++ax) {
+    const bool last = ax + 1 == p.d.ndim;
+    if (last && p.d.ndim == 2) {
+      // long y lines: a tile's rows of them would not fill a 32-byte sector
+      Plan pl;
+      if ((st = plan_axis(c, p, ax, MODE_R, 1, beta / (cb * dt), &pl)) != MOLT_OK) return st;
+      if (size_t(pl.a.W) * el < 32) {
+        const long long nx = p.n[0], ny = p.n[1];
+        const Problem pt = transposed(p);
+        if ((st = transpose(c, p, us, p.gp, ny, nx, el)) != MOLT_OK) return st;
+        if ((st = axis(pt, 0, p.d.velocity[1], EPI_ACC_SET, p.gp, p.gm)) != MOLT_OK) return st;
+        molt_ctx::Rec rec;
+        record_begin(c, &rec, MOLT_KERNEL_UPDATE);
+        const dim3 grid(unsigned((nx + 63) / 64), unsigned((ny + 63) / 64)), block(32, 8);
+        if (f64)
+          advdiff_update_t_kernel<double><<<grid, block, 0, c->stream>>>(
+              static_cast<const double*>(p.acc), static_cast<const double*>(p.gm), static_cast<const double*>(un),
+              static_cast<const double*>(us), static_cast<double*>(dst), a0, a1, ny, nx, c->status_dev);
+        else
+          advdiff_update_t_kernel<float><<<grid, block, 0, c->stream>>>(
+              static_cast<const float*>(p.acc), static_cast<const float*>(p.gm), static_cast<const float*>(un),
+              static_cast<const float*>(us), static_cast<float*>(dst), a0, a1, ny, nx, c->status_dev);
+        record_end(c, &rec);
+        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "advection-diffusion update");
+        continue;
+      }
+    }
+    const int epi = last ? EPI_ADV_FINAL : (ax == 0 ? EPI_ACC_SET : EPI_ACC_ADD);
+    if ((st = axis(p, ax, p.d.velocity[ax], epi, us, p.d.ndim == 1 ? nullptr : p.acc)) != MOLT_OK) return st;
+  }
+  return MOLT_OK;
+}
+
 molt_status advdiff_step(molt_ctx* c, Problem& p, void* u) {
   static const double rk[3][2] = {{0.0, 1.0}, {0.75, 0.25}, {1.0 / 3.0, 2.0 / 3.0}};
   const bool euler = p.d.integrator == MOLT_INT_EULER;
@@ -1554,7 +1676,13 @@ molt_status advdiff_step(molt_ctx* c, Problem& p, void* u) {
   const double alpha_nu = kappa > 0 ? beta / std::sqrt(kappa * dt) : 0.0;
   const bool f64 = is_f64_sweep(p.d), f32s = is_f32_state(p.d);
   cudaError_t e;
+  const bool fused = advdiff_fused(p);
   for (int s = 0; s < (euler ? 1 : 3); ++s) {
+    if (fused) {
+      const molt_status st = advdiff_stage_fused(c, p, u, ins[s], dsts[s], rk[s][0], rk[s][1]);
+      if (st != MOLT_OK) return st;
+      continue;
+    }
     if ((e = cudaMemsetAsync(p.acc, 0, compute_bytes(p.d) * size_t(p.total), c->stream)) != cudaSuccess)
       return cuda_fail(c, e, "memset");
     for (int ax = 0; ax < p.d.ndim; ++ax) {

@@ -61,7 +61,8 @@ enum Epi {
   EPI_HJ_Y = 6,        // u -= dt*H^; speed max
   EPI_HJ_XG = 7,       // EPI_HJ_X for every Hamiltonian (HamKind)
   EPI_HJ_YG = 8,       // EPI_HJ_Y for every Hamiltonian, a source F(x, t), speed-only passes
-  EPI_ACC_AXPY = 9     // acc += coefS * S (advection-diffusion terms)
+  EPI_ACC_AXPY = 9,    // acc += coefS * S (advection-diffusion terms)
+  EPI_ADV_FINAL = 10   // dst = a0*un + a1*(us + (acc + S)) (advection-diffusion, fused axis kernel)
 };
 // The general Hamilton-Jacobi kernels (XG/YG) carry more operands per point;
 // the |grad u|^2/2 kernels without a source keep their own instantiations.
@@ -88,16 +89,9 @@ struct LineGeom {
   long long stride;   // element stride along the line
 };
 
-struct SweepArgs {
-  LineGeom g;
-  int W, nwl, LS;     // lines per CTA, warps per line, shared line stride (elements)
-  int E;              // points per lane of the plain kernel (16, 8 or 4; others mean 16)
-  int bc;             // 0 periodic, 1 Dirichlet
-  int mode;           // Mode
-  int P;
-  int contiguous;     // stride == 1
-  // line constants (csrc/line_constants.h); the FP32 copies are rounded on
-  // the host (converting on the device would use the FP64 pipe)
+// Constants of the scans along a line (csrc/line_constants.h); the FP32 copies
+// are rounded on the host (converting on the device would use the FP64 pipe).
+struct LineConst {
   int d0;             // JQ_D0: 1 residual form, 0 K filters
   int close;          // boundary constants: 0 none, 1 kA, 2 kA and kB
   double b[5];        // K_R taps on the differences d_{i-2} .. d_{i+2}
@@ -107,9 +101,20 @@ struct SweepArgs {
   double qp[13];      // q^(2^k), q = e^{-nu}
   double qlast, qlw;  // q^(valid points of the last lane / of the last warp)
   double kA, kB;      // boundary constants C = kA T_same + kB T_other
-  double alpha;
-  float bf[5], f0f, f1f, kapf, wkf[6], df[3], qpf[13], qlastf, qlwf, alphaf;
+  float bf[5], f0f, f1f, kapf, wkf[6], df[3], qpf[13], qlastf, qlwf;
   float kAh, kAl, kBh, kBl;   // kA, kB as FP32 pairs
+};
+
+struct SweepArgs : LineConst {
+  LineGeom g;
+  int W, nwl, LS;     // lines per CTA, warps per line, shared line stride (elements)
+  int E;              // points per lane of the plain kernel (16, 8 or 4; others mean 16)
+  int bc;             // 0 periodic, 1 Dirichlet
+  int mode;           // Mode
+  int P;
+  int contiguous;     // stride == 1
+  double alpha;
+  float alphaf;
   // epilogue operands
   const void* in;     // sweep input (TIN)
   void* out;          // EPI_STORE destination / HJ: H^_x buffer (state type)
@@ -283,16 +288,16 @@ __device__ __forceinline__ double weight_rcp(double x) { return 1.0 / x; }
 // K = sum_r w_r K_r with K_r = q e0 + sum_j c^{(r)}_j (v_i - v_j) a filter of
 // the differences (wk, csrc/line_constants.h; the e0 weight of K_0 is 1).
 // WENO-Z (Sec. 2.4): w~_r = d_r (1 + tau/(eps+beta_r)), tau = |beta_0-beta_2|.
+// The indicators arrive with eps added.
 template <typename T>
-__device__ __forceinline__ T wenoz_defect(T e0, T e1, T e2, T f, const T (&beta)[3], const T (&wk)[6],
-                                          const T (&d)[3]) {
+__device__ __forceinline__ T wenoz_defect(T e0, T e1, T e2, T f, T b0, T b1, T b2, const T (&wk)[6], const T (&d)[3]) {
   const T K[3] = {fma(wk[1], e2, fma(wk[0], e1, e0)), fma(wk[3], e1, wk[2] * e0), fma(wk[5], f, wk[4] * e0)};
-  const T tau = fabs(beta[0] - beta[2]);
-  const T eps = T(1e-6);
+  const T b[3] = {b0, b1, b2};
+  const T tau = fabs(b0 - b2);
   T wt[3], sum = T(0);
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
-    wt[r] = fma(d[r] * tau, weight_rcp(eps + beta[r]), d[r]);   // d_r (1 + tau/(eps+beta_r))
+    wt[r] = fma(d[r] * tau, weight_rcp(b[r]), d[r]);   // d_r (1 + tau/(eps+beta_r))
     sum += wt[r];
   }
   return (wt[0] * K[0] + wt[1] * K[1] + wt[2] * K[2]) * weight_rcp(sum);
@@ -302,22 +307,23 @@ __device__ __forceinline__ T wenoz_defect(T e0, T e1, T e2, T f, const T (&beta)
 // quadratic through the node triple (a, b, c) of substencil r; with s1 =
 // (c - a)/2 and s2 = a - 2b + c, beta_r = s1^2 + k_r s1 s2 + m_r s2^2 (k = 3,
 // 1, -1; m = 10/3, 4/3, 4/3).  A triple serves three points' J_R and,
-// mirrored (s1 -> -s1), three points' J_L, so the products are formed once
-// per triple, from its differences da = b - a, db = c - b.
+// mirrored (s1 -> -s1), three points' J_L, with four different values: as
+// substencil 0 of J_R, 0 of J_L, 1 of J_R (2 of J_L) and 2 of J_R (1 of J_L).
+// They are formed once per triple, with eps = 1e-6 added, from its differences
+// da = b - a, db = c - b (the compiler shares them among the points).
 template <typename T>
-__device__ __forceinline__ void triple_products(T da, T db, T* p11, T* p12, T* p22) {
-  const T s1 = T(0.5) * (da + db);
-  const T s2 = db - da;
-  *p11 = s1 * s1;
-  *p12 = s1 * s2;
-  *p22 = s2 * s2;
-}
-template <typename T>
-__device__ __forceinline__ T beta_from_products(int r, T p11, T p12, T p22, bool mirrored) {
-  const T k = r == 0 ? T(3) : (r == 1 ? T(1) : T(-1));
-  const T m = r == 0 ? T(10.0 / 3.0) : T(4.0 / 3.0);
-  return p11 + (mirrored ? -k : k) * p12 + m * p22;
-}
+struct Indicators {
+  T outer, outer_mir, plus, minus;
+  __device__ __forceinline__ Indicators(T da, T db) {
+    const T s1 = T(0.5) * (da + db), s2 = db - da;
+    const T p12 = s1 * s2, p22 = s2 * s2, p11 = fma(s1, s1, T(1e-6));
+    const T A = fma(T(4.0 / 3.0), p22, p11), B = fma(T(10.0 / 3.0), p22, p11);
+    outer = fma(T(3), p12, B);
+    outer_mir = fma(T(-3), p12, B);
+    plus = A + p12;
+    minus = A - p12;
+  }
+};
 
 // -------------------------------------------------------------- tile staging
 // Barrier of the warps that share line lw of a tile (named barrier 1 + lw;
@@ -422,12 +428,12 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 
 // ------------------------------------------------------------- line constants
 template <typename T>
-__device__ __forceinline__ T qpow_bit(const SweepArgs& a, int k) { return pick<T>(a.qp[k], a.qpf[k]); }
+__device__ __forceinline__ T qpow_bit(const LineConst& a, int k) { return pick<T>(a.qp[k], a.qpf[k]); }
 
 // q^e for 0 <= e < 2^COUNT, times 2^LO: the product of the stored powers
 // q^(2^(LO + k)) over the bits of e.
 template <typename T, int LO, int COUNT>
-__device__ __forceinline__ T qpow(const SweepArgs& a, int e) {
+__device__ __forceinline__ T qpow(const LineConst& a, int e) {
   T r = T(1);
 #pragma unroll
   for (int k = 0; k < COUNT; ++k)
@@ -550,6 +556,330 @@ __device__ __forceinline__ T ghost_value(const T* b, int e, int n, int bc) {
   return T(2) * b[phys<E>(n - 1)] - b[phys<E>(2 * (n - 1) - e)];
 }
 
+// A lane's place in its line, for the scans below.
+template <typename T, bool ONE, bool RAGGED, int E>
+struct LineLane {
+  T* totals;
+  T* buf;              // the line
+  T* cbase;            // the lane's chunk: phys<E>(e0 + j) = (E+1)*ch + chunk_off<E>(j)
+  int n, nwl, lw, part, lane, e0, ch;
+  bool mir;            // one-sided L scans run the line mirrored
+  bool dir, own;
+  bool end0, endN;     // the chunk holds a Dirichlet end node (x_0, x_{n-1})
+  int lastR;           // the lane whose last point closes the R scan of its warp
+
+  __device__ __forceinline__ LineLane(const SweepArgs& a, const TileSmem& sm) {
+    static_assert(phys<E>(E * 3 + 2) == (E + 1) * 3 + chunk_off<E>(2), "lane base / chunk offset mismatch");
+    nwl = a.nwl;
+    n = a.g.n;
+    totals = static_cast<T*>(sm.totals);
+    const int warp = threadIdx.x >> 5;
+    lane = threadIdx.x & 31;
+    lw = warp / nwl;
+    part = warp - lw * nwl;
+    buf = static_cast<T*>(sm.lines) + lw * a.LS;
+    mir = ONE && a.mode == MODE_L;
+    const int tl = part * 32 + lane;
+    ch = mir ? nwl * 32 - 1 - tl : tl;
+    e0 = ch * E;
+    cbase = buf + (E + 1) * ch;
+    dir = a.bc == 1;
+    own = nwl == 1;
+    lastR = (RAGGED && !mir && part == nwl - 1) ? ((n - 1) / E) & 31 : 31;
+    end0 = dir && e0 == 0;
+    endN = dir && n - 1 >= e0 && n - 1 < e0 + E;
+  }
+  // point k of the chunk in scan order lies on the line
+  __device__ __forceinline__ bool valid(int k) const { return !RAGGED || (mir ? e0 + E - 1 - k : e0 + k) < n; }
+  // writes the chunk's values (scan order) back to the line
+  __device__ __forceinline__ void store(const T (&x)[E]) const {
+    if (!mir) {
+#pragma unroll
+      for (int k = 0; k < E; ++k)
+        if (valid(k)) cbase[chunk_off<E>(k)] = x[k];
+    } else {
+#pragma unroll
+      for (int k = 0; k < E; ++k)
+        if (valid(k)) cbase[chunk_off<E>(E - 1 - k)] = x[k];
+    }
+  }
+};
+
+// Powers of q: up to this lane inside its warp, up to this warp (R: from the
+// left end, L: from the right end; one-sided: in scan order), and the decay
+// of the lane that closes the warp's R scan.
+template <typename T>
+struct LinePowers {
+  T pwR, pwL, qwR, qwL, mulR;
+};
+template <typename T, bool ONE, bool RAGGED, int E>
+__device__ __forceinline__ LinePowers<T> line_powers(const LineConst& L, const LineLane<T, ONE, RAGGED, E>& ln) {
+  constexpr int LE = log2i<E>();
+  LinePowers<T> p{T(1), T(1), T(1), T(1), T(1)};
+  const bool ragged_first = RAGGED && (ONE ? ln.mir && ln.part == 0 : ln.part == ln.nwl - 1);
+  p.pwR = qpow<T, LE, 5>(L, ln.lane);
+  if (!ONE || ln.mir) {
+    T pl = ONE ? p.pwR : __shfl_sync(0xffffffffu, p.pwR, 31 - ln.lane);
+    if (ragged_first) {
+      const int before = ln.n - ln.e0 - E;
+      pl = before > 0 ? qpow<T, 0, LE + 5>(L, before) : T(1);
+    }
+    if (ONE) p.pwR = pl; else p.pwL = pl;
+  }
+  if (!ln.own) {
+    const T qlw = pick<T>(L.qlw, L.qlwf);
+    if (!ln.mir) p.qwR = qpow<T, LE + 5, 4>(L, ln.part);
+    else if (ln.part > 0) p.qwR = qlw * qpow<T, LE + 5, 4>(L, ln.part - 1);
+    if (!ONE && ln.part < ln.nwl - 1) p.qwL = qlw * qpow<T, LE + 5, 4>(L, ln.nwl - 2 - ln.part);
+  }
+  p.mulR = (RAGGED && !ln.mir && ln.part == ln.nwl - 1) ? pick<T>(L.qlast, L.qlastf) : qpow_bit<T>(L, LE);
+  return p;
+}
+
+// The chunk's window with three points on either side (ragged lines: their
+// ghost cells are in place).
+template <typename T, bool ONE, bool RAGGED, int E>
+__device__ __forceinline__ void load_window(const LineLane<T, ONE, RAGGED, E>& ln, T (&win)[E + 6]) {
+  // window of the chunk in scan orientation: win[j] = v at offset j - 3
+  // from the chunk's first point
+  if (!ln.mir) {
+#pragma unroll
+    for (int j = 0; j < E + 6; ++j) win[j] = ln.cbase[chunk_off<E>(j - 3)];
+  } else {
+#pragma unroll
+    for (int j = 0; j < E + 6; ++j) win[j] = ln.cbase[chunk_off<E>(E + 2 - j)];
+  }
+  if constexpr (!RAGGED) {
+    // ghosts of an exact-fit line: only the end lanes need them
+    if (ln.e0 == 0 || ln.e0 + E == ln.n) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const int el = ln.mir ? ln.e0 + E + 2 - j : ln.e0 + j - 3;
+        const int er = ln.mir ? ln.e0 - 1 - j : ln.e0 + E + j;
+        if (el < 0 || el >= ln.n) win[j] = ghost_value<T, E>(ln.buf, el, ln.n, (ln.dir ? 1 : 0));
+        if (er < 0 || er >= ln.n) win[E + 3 + j] = ghost_value<T, E>(ln.buf, er, ln.n, (ln.dir ? 1 : 0));
+      }
+    }
+  }
+}
+
+// K_R into X and K_L into F of the linear rule (ONE: X alone, in scan order)
+// from the window's differences dd[j] = win[j+1] - win[j].
+template <typename T, bool ONE, int E>
+__device__ __forceinline__ void linear_forcings(const LineConst& a, const T (&dd)[E + 5], T (&X)[E + 1], T (&F)[E]) {
+#pragma unroll
+  for (int k = 0; k < E; ++k) {
+    T r = T(0), l = T(0);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      r = fma(pick<T>(a.b[i], a.bf[i]), dd[k + i], r);
+      if constexpr (!ONE) l = fma(-pick<T>(a.b[i], a.bf[i]), dd[k + 5 - i], l);
+    }
+    X[k] = r;
+    if (!ONE) F[k] = l;
+  }
+}
+
+// The same with WENO-Z weights: dR the differences of the values J_R
+// integrates, dL those of J_L (the same ones but for split fluxes).
+template <typename T, bool ONE, int E>
+__device__ __forceinline__ void wenoz_forcings(const LineConst& a, const T (&dR)[E + 5], const T (&dL)[E + 5],
+                                               T (&X)[E + 1], T (&F)[E]) {
+  T wc[6], dw[3];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) wc[i] = pick<T>(a.wk[i], a.wkf[i]);
+#pragma unroll
+  for (int r = 0; r < 3; ++r) dw[r] = pick<T>(a.d[r], a.df[r]);
+  // J_R of point k uses the triples k, k+1, k+2, J_L the triples k+4, k+3,
+  // k+2 mirrored
+#pragma unroll
+  for (int k = 0; k < E; ++k) {
+    const Indicators<T> i0(dR[k], dR[k + 1]), i1(dR[k + 1], dR[k + 2]), i2(dR[k + 2], dR[k + 3]);
+    X[k] = wenoz_defect<T>(dR[k + 2], dR[k + 1], dR[k], dR[k + 3], i0.outer, i1.plus, i2.minus, wc, dw);
+    if constexpr (!ONE) {
+      const Indicators<T> l2(dL[k + 2], dL[k + 3]), l1(dL[k + 3], dL[k + 4]), l0(dL[k + 4], dL[k + 5]);
+      F[k] = wenoz_defect<T>(-dL[k + 3], -dL[k + 4], -dL[k + 5], -dL[k + 2], l0.outer_mir, l1.minus, l2.plus, wc, dw);
+    }
+  }
+}
+
+// Forcings of D_0 with linear weights: the residual form (X the differences
+// d_k, k = 0..E, F the FIR part), or the K filters.
+template <typename T, int E>
+__device__ __forceinline__ void d0_forcings(const LineConst& a, const T (&dd)[E + 5], T (&X)[E + 1], T (&F)[E]) {
+  if (a.d0) {
+    const T f0 = pick<T>(a.f0, a.f0f), f1 = pick<T>(a.f1, a.f1f);
+    if (f1 != T(0)) {
+#pragma unroll
+      for (int k = 0; k < E; ++k) {
+        const T s0 = dd[k + 2] - dd[k + 1], s1 = dd[k + 3] - dd[k + 2], s2 = dd[k + 4] - dd[k + 3];
+        F[k] = fma(f1, s0 + s2, f0 * s1);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < E; ++k) F[k] = f0 * (dd[k + 3] - dd[k + 2]);
+    }
+#pragma unroll
+    for (int k = 0; k <= E; ++k) X[k] = dd[k + 2];
+  } else {
+    linear_forcings<T, false, E>(a, dd, X, F);
+  }
+}
+
+// Scans of the forcings, R in X and L in F (ONE: X alone; D_0's residual
+// form, L.d0: X the differences, F the FIR part): scans from zero (lane
+// folds, warp scan, warps of the line), boundary constants, and the scans
+// again from their carries.  Leaves W_R in X and W_L in F; ONE, D0: D in F.
+template <typename T, bool D0, bool ONE, bool RAGGED, int E>
+__device__ __forceinline__ void line_scans(const LineConst& L, const LineLane<T, ONE, RAGGED, E>& ln,
+                                           const LinePowers<T>& pw, T (&X)[E + 1], T (&F)[E]) {
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int LE = log2i<E>();
+  const T q = qpow_bit<T>(L, 0);
+  // Dirichlet ends: no forcing at the node where a scan starts
+  const bool resid = D0 && L.d0;
+  if (ONE) {
+    if (ln.dir) {
+#pragma unroll
+      for (int k = 0; k < E; ++k) {
+        const int e = ln.mir ? ln.e0 + E - 1 - k : ln.e0 + k;
+        if (e == (ln.mir ? ln.n - 1 : 0)) X[k] = T(0);
+      }
+    }
+  } else {
+    if (ln.end0) X[0] = T(0);
+    if (ln.endN) {
+#pragma unroll
+      for (int k = 0; k < E; ++k)
+        if (RAGGED ? ln.e0 + k == ln.n - 1 : k == E - 1) {
+          if (resid) X[k + 1] = T(0); else F[k] = T(0);
+        }
+    }
+  }
+
+  // scans from zero: lane folds, warp scan, warps of the line
+  T bR = T(0), bL = T(0);
+#pragma unroll
+  for (int k = 0; k < E; ++k)
+    if (ln.valid(k)) bR = fma(q, bR, X[k]);
+  if constexpr (!ONE) {
+    if (resid) {
+#pragma unroll
+      for (int k = E - 1; k >= 0; --k)
+        if (ln.valid(k)) bL = fma(q, bL, -X[k + 1]);
+    } else {
+#pragma unroll
+      for (int k = E - 1; k >= 0; --k)
+        if (ln.valid(k)) bL = fma(q, bL, F[k]);
+    }
+  }
+  const T ownR = bR;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const int o = 1 << k;
+    const T m = qpow_bit<T>(L, LE + k);
+    const T bp = shfl_up(bR, o);
+    const T sR = fma(m, bp, bR);
+    bR = ln.lane >= o ? sR : bR;
+    if constexpr (!ONE) {
+      const T bn = shfl_down(bL, o);
+      const T sL = fma(m, bn, bL);
+      bL = ln.lane + o < 32 ? sL : bL;
+    }
+  }
+  T cR = shfl_up(bR, 1), cL = T(0);     // value entering the lane from zero before the warp
+  if (ln.lane == 0) cR = T(0);
+  if constexpr (!ONE) {
+    cL = shfl_down(bL, 1);
+    if (ln.lane == 31) cL = T(0);
+  }
+  const T endR = fma(pw.mulR, cR, ownR);   // at lane lastR: the warp's R end value
+  T inR = T(0), inL = T(0), tR, tL = T(0);
+  if (ln.own) {
+    tR = __shfl_sync(FULL, endR, ln.lastR);
+    if constexpr (!ONE) tL = __shfl_sync(FULL, bL, 0);
+  } else {
+    T* tot = ln.totals + ln.lw * ln.nwl * 2;
+    if (ln.lane == ln.lastR) tot[2 * ln.part] = endR;
+    if (!ONE && ln.lane == 0) tot[2 * ln.part + 1] = bL;
+    line_sync(ln.nwl, ln.lw);
+    const int j = ln.lane & 15;
+    const bool left = ln.lane >= 16;
+    T x = T(0);
+    if (j < ln.nwl && !(ONE && left)) x = left ? tot[2 * (ln.nwl - 1 - j) + 1] : tot[2 * j];
+    const T x0 = x;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if ((1 << k) < ln.nwl) {
+        const T xp = __shfl_up_sync(FULL, x, 1 << k, 16);
+        const T sx = fma(qpow_bit<T>(L, LE + 5 + k), xp, x);
+        x = j >= (1 << k) ? sx : x;
+      }
+    }
+    T ex = __shfl_up_sync(FULL, x, 1, 16);   // value entering warp j
+    if (j == 0) ex = T(0);
+    const T lastw = (left || ln.mir) ? qpow_bit<T>(L, LE + 5) : pick<T>(L.qlw, L.qlwf);
+    const T te = fma(lastw, ex, x0);
+    tR = __shfl_sync(FULL, te, ln.nwl - 1);
+    inR = __shfl_sync(FULL, ex, ln.part);
+    if constexpr (!ONE) {
+      tL = __shfl_sync(FULL, te, 15 + ln.nwl);
+      inL = __shfl_sync(FULL, ex, 15 + ln.nwl - ln.part);
+    }
+  }
+  // boundary constants, carried to the lane
+  if (L.close) {
+    inR = fma(pw.qwR, line_constant<T>(L, tR, tL), inR);
+    if constexpr (!ONE) inL = fma(pw.qwL, line_constant<T>(L, tL, tR), inL);
+  }
+  if (L.close || !ln.own) {
+    cR = fma(pw.pwR, inR, cR);
+    if constexpr (!ONE) cL = fma(pw.pwL, inL, cL);
+  }
+  // the scans from their carries -> D of the power (in F; two-sided
+  // forms keep W_R, W_L)
+  T y = cR;
+  if (resid) {
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+      if (ln.valid(k)) y = fma(q, y, X[k]);
+      F[k] = fma(pick<T>(L.kap, L.kapf), y, F[k]);
+    }
+    y = cL;
+#pragma unroll
+    for (int k = E - 1; k >= 0; --k) {
+      if (ln.valid(k)) y = fma(q, y, -X[k + 1]);
+      F[k] = fma(pick<T>(L.kap, L.kapf), y, F[k]);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+      if (ln.valid(k)) y = fma(q, y, X[k]);
+      X[k] = y;
+    }
+    if constexpr (ONE) {
+#pragma unroll
+      for (int k = 0; k < E; ++k) F[k] = X[k];
+    } else {
+      y = cL;
+#pragma unroll
+      for (int k = E - 1; k >= 0; --k) {
+        if (ln.valid(k)) y = fma(q, y, F[k]);
+        F[k] = D0 ? T(0.5) * (X[k] + y) : y;
+      }
+    }
+  }
+  if constexpr (D0) {
+    // D_0 vanishes at Dirichlet ends
+    if (ln.end0) F[0] = T(0);
+    if (ln.endN) {
+#pragma unroll
+      for (int k = 0; k < E; ++k)
+        if (RAGGED ? ln.e0 + k == ln.n - 1 : k == E - 1) F[k] = T(0);
+    }
+  }
+}
+
 // Applies D P times to the staged lines and leaves S_P (or, for MODE_RL, the
 // per-axis Lax-Friedrichs Hamiltonian) in the line buffers.  Returns the
 // thread's largest one-sided derivative magnitude (MODE_RL).  Ends
@@ -588,56 +918,11 @@ __device__ __forceinline__ T ghost_value(const T* b, int e, int n, int bc) {
 template <typename T, int JQ, bool RAGGED, int E = kE, bool GEN = false>
 __device__ __forceinline__ double compute_lines(const SweepArgs& a, const TileSmem& sm, bool line_ok) {
   static_assert(JQ != JQ_LEARNED || sizeof(T) == 4, "learned weights run in FP32");
-  constexpr unsigned FULL = 0xffffffffu;
   constexpr bool ONE = JQ == JQ_LINEAR1 || JQ == JQ_WENOZ1;
   constexpr bool WENO = JQ == JQ_WENOZ || JQ == JQ_WENOZ1;
-  constexpr int LE = log2i<E>();
-  const int nwl = a.nwl, n = a.g.n;
-  T* totals = static_cast<T*>(sm.totals);
-  T* lines = static_cast<T*>(sm.lines);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int lw = warp / nwl, part = warp - lw * nwl;
-  const int tl = part * 32 + lane;
-  T* buf = lines + lw * a.LS;
-  // the lane's chunk: points e0 .. e0+E-1 (one-sided L scans run the line mirrored)
-  const bool mir = ONE && a.mode == MODE_L;
-  const int ch = mir ? nwl * 32 - 1 - tl : tl;
-  const int e0 = ch * E;
-  T* cbase = buf + (E + 1) * ch;   // phys<E>(e0 + j) = (E+1)*ch + chunk_off<E>(j)
-  static_assert(phys<E>(E * 3 + 2) == (E + 1) * 3 + chunk_off<E>(2), "lane base / chunk offset mismatch");
-  const bool dir = a.bc == 1;
-  const T q = qpow_bit<T>(a, 0);
-  const bool own = nwl == 1;
-
-  // powers of q: up to this lane inside its warp, up to this warp (R: from
-  // the left end, L: from the right end; one-sided: in scan order)
-  T pwR = T(1), pwL = T(1), qwR = T(1), qwL = T(1);
-  auto lane_powers = [&]() {
-    const bool ragged_first = RAGGED && (ONE ? mir && part == 0 : part == nwl - 1);
-    pwR = qpow<T, LE, 5>(a, lane);
-    if (!ONE || mir) {
-      T pl = ONE ? pwR : __shfl_sync(FULL, pwR, 31 - lane);
-      if (ragged_first) {
-        const int before = n - e0 - E;
-        pl = before > 0 ? qpow<T, 0, LE + 5>(a, before) : T(1);
-      }
-      if (ONE) pwR = pl; else pwL = pl;
-    }
-    if (!own) {
-      const T qlw = pick<T>(a.qlw, a.qlwf);
-      if (!mir) qwR = qpow<T, LE + 5, 4>(a, part);
-      else if (part > 0) qwR = qlw * qpow<T, LE + 5, 4>(a, part - 1);
-      if (!ONE && part < nwl - 1) qwL = qlw * qpow<T, LE + 5, 4>(a, nwl - 2 - part);
-    }
-  };
-  if constexpr (JQ != JQ_LEARNED) lane_powers();   // (not live across the network)
-  // the lane whose last point closes the R scan of its warp
-  const int lastR = (RAGGED && !mir && part == nwl - 1) ? ((n - 1) / E) & 31 : 31;
-  const T mulR = (RAGGED && !mir && part == nwl - 1) ? pick<T>(a.qlast, a.qlastf) : qpow_bit<T>(a, LE);
-  // Dirichlet: the scans start from zero at the end nodes
-  const bool end0 = dir && e0 == 0;
-  const bool endN = dir && n - 1 >= e0 && n - 1 < e0 + E;
-
+  const LineLane<T, ONE, RAGGED, E> ln(a, sm);
+  LinePowers<T> pw;
+  if constexpr (JQ != JQ_LEARNED) pw = line_powers<T, ONE, RAGGED, E>(a, ln);   // (not live across the network)
   T S[E];
   T rmax = T(0);
 
@@ -648,251 +933,35 @@ __device__ __forceinline__ double compute_lines(const SweepArgs& a, const TileSm
     // with L descending) the moves that build the pairs cost more than the
     // halved FMA count saved (64 heat problems 11.4 against 12.4 ms a pass).
     T X[E + 1], F[E];
+    if constexpr (JQ == JQ_LEARNED || RAGGED) {
+      if (ln.part == 0) warp_fill_ghosts<T, E>(a, ln.buf, ln.lane);
+      line_sync(ln.nwl, ln.lw);
+    }
     if constexpr (JQ == JQ_LEARNED) {
-      if (part == 0) warp_fill_ghosts<T, E>(a, buf, lane);
-      line_sync(nwl, lw);
-      float* jrl = sm.jloc + lw * 2 * a.LS;
+      float* jrl = sm.jloc + ln.lw * 2 * a.LS;
       if (line_ok)
-        learned_local_integrals<E>(a, *sm.net, buf, jrl, jrl + a.LS, sm.mlp_scratch + warp * kMlpScratchBytes,
-                                   part * 32 * E, n, lane);
+        learned_local_integrals<E>(a, *sm.net, ln.buf, jrl, jrl + a.LS,
+                                   sm.mlp_scratch + (threadIdx.x >> 5) * kMlpScratchBytes, ln.part * 32 * E, ln.n,
+                                   ln.lane);
       __syncwarp();
-      lane_powers();
+      pw = line_powers<T, ONE, RAGGED, E>(a, ln);
 #pragma unroll
       for (int k = 0; k < E; ++k) {
-        X[k] = jrl[(E + 1) * tl + chunk_off<E>(k)];
-        F[k] = jrl[a.LS + (E + 1) * tl + chunk_off<E>(k)];
+        X[k] = jrl[(E + 1) * ln.ch + chunk_off<E>(k)];
+        F[k] = jrl[a.LS + (E + 1) * ln.ch + chunk_off<E>(k)];
       }
     } else {
-      if constexpr (RAGGED) {
-        if (part == 0) warp_fill_ghosts<T, E>(a, buf, lane);
-        line_sync(nwl, lw);
-      }
-      // window of the chunk in scan orientation: win[j] = v at offset j - 3
-      // from the chunk's first point
-      T win[E + 6];
-      if (!mir) {
-#pragma unroll
-        for (int j = 0; j < E + 6; ++j) win[j] = cbase[chunk_off<E>(j - 3)];
-      } else {
-#pragma unroll
-        for (int j = 0; j < E + 6; ++j) win[j] = cbase[chunk_off<E>(E + 2 - j)];
-      }
-      if constexpr (!RAGGED) {
-        // ghosts of an exact-fit line: only the end lanes need them
-        if (e0 == 0 || e0 + E == n) {
-#pragma unroll
-          for (int j = 0; j < 3; ++j) {
-            const int el = mir ? e0 + E + 2 - j : e0 + j - 3;
-            const int er = mir ? e0 - 1 - j : e0 + E + j;
-            if (el < 0 || el >= n) win[j] = ghost_value<T, E>(buf, el, n, a.bc);
-            if (er < 0 || er >= n) win[E + 3 + j] = ghost_value<T, E>(buf, er, n, a.bc);
-          }
-        }
-      }
-      T dd[E + 5];   // dd[j] = win[j+1] - win[j]
+      T win[E + 6], dd[E + 5];
+      load_window<T, ONE, RAGGED, E>(ln, win);
 #pragma unroll
       for (int j = 0; j < E + 5; ++j) dd[j] = win[j + 1] - win[j];
-      if (JQ == JQ_D0 && a.d0) {
-        const T f0 = pick<T>(a.f0, a.f0f), f1 = pick<T>(a.f1, a.f1f);
-        if (f1 != T(0)) {
-#pragma unroll
-          for (int k = 0; k < E; ++k) {
-            const T s0 = dd[k + 2] - dd[k + 1], s1 = dd[k + 3] - dd[k + 2], s2 = dd[k + 4] - dd[k + 3];
-            F[k] = fma(f1, s0 + s2, f0 * s1);
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < E; ++k) F[k] = f0 * (dd[k + 3] - dd[k + 2]);
-        }
-#pragma unroll
-        for (int k = 0; k <= E; ++k) X[k] = dd[k + 2];
-      } else if constexpr (!WENO) {
-#pragma unroll
-        for (int k = 0; k < E; ++k) {
-          T r = T(0), l = T(0);
-#pragma unroll
-          for (int i = 0; i < 5; ++i) {
-            r = fma(pick<T>(a.b[i], a.bf[i]), dd[k + i], r);
-            if constexpr (!ONE) l = fma(-pick<T>(a.b[i], a.bf[i]), dd[k + 5 - i], l);
-          }
-          X[k] = r;
-          if (!ONE) F[k] = l;
-        }
-      } else {
-        // WENO-Z: indicators from per-triple products; J_R of point k uses
-        // the triples k, k+1, k+2, J_L the triples k+4, k+3, k+2 mirrored
-        T wc[6], dw[3];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) wc[i] = pick<T>(a.wk[i], a.wkf[i]);
-#pragma unroll
-        for (int r = 0; r < 3; ++r) dw[r] = pick<T>(a.d[r], a.df[r]);
-        constexpr int NT = ONE ? E + 2 : E + 4;
-        T p11[NT], p12[NT], p22[NT];
-#pragma unroll
-        for (int t = 0; t < NT; ++t) triple_products<T>(dd[t], dd[t + 1], &p11[t], &p12[t], &p22[t]);
-#pragma unroll
-        for (int k = 0; k < E; ++k) {
-          T be[3];
-#pragma unroll
-          for (int r = 0; r < 3; ++r) be[r] = beta_from_products<T>(r, p11[k + r], p12[k + r], p22[k + r], false);
-          const T r = wenoz_defect<T>(dd[k + 2], dd[k + 1], dd[k], dd[k + 3], be, wc, dw);
-          if constexpr (ONE) {
-            X[k] = r;
-          } else {
-#pragma unroll
-            for (int j = 0; j < 3; ++j)
-              be[j] = beta_from_products<T>(j, p11[k + 4 - j], p12[k + 4 - j], p22[k + 4 - j], true);
-            const T l = wenoz_defect<T>(-dd[k + 3], -dd[k + 4], -dd[k + 5], -dd[k + 2], be, wc, dw);
-            X[k] = r;
-            F[k] = l;
-          }
-        }
-      }
+      if constexpr (WENO) wenoz_forcings<T, ONE, E>(a, dd, dd, X, F);
+      else if constexpr (JQ == JQ_D0) d0_forcings<T, E>(a, dd, X, F);
+      else linear_forcings<T, ONE, E>(a, dd, X, F);
     }
-    // Dirichlet ends: no forcing at the node where a scan starts
-    const bool resid = JQ == JQ_D0 && a.d0;
-    if (ONE) {
-      if (dir) {
-#pragma unroll
-        for (int k = 0; k < E; ++k) {
-          const int e = mir ? e0 + E - 1 - k : e0 + k;
-          if (e == (mir ? n - 1 : 0)) X[k] = T(0);
-        }
-      }
-    } else {
-      if (end0) X[0] = T(0);
-      if (endN) {
-#pragma unroll
-        for (int k = 0; k < E; ++k)
-          if (RAGGED ? e0 + k == n - 1 : k == E - 1) {
-            if (resid) X[k + 1] = T(0); else F[k] = T(0);
-          }
-      }
-    }
-
-    // ---- 2. scans from zero: lane folds, warp scan, warps of the line
-    auto valid = [&](int k) { return !RAGGED || (mir ? e0 + E - 1 - k : e0 + k) < n; };
-    T bR = T(0), bL = T(0);
-#pragma unroll
-    for (int k = 0; k < E; ++k)
-      if (valid(k)) bR = fma(q, bR, X[k]);
-    if constexpr (!ONE) {
-      if (JQ == JQ_D0 && a.d0) {
-#pragma unroll
-        for (int k = E - 1; k >= 0; --k)
-          if (valid(k)) bL = fma(q, bL, -X[k + 1]);
-      } else {
-#pragma unroll
-        for (int k = E - 1; k >= 0; --k)
-          if (valid(k)) bL = fma(q, bL, F[k]);
-      }
-    }
-    const T ownR = bR;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      const int o = 1 << k;
-      const T m = qpow_bit<T>(a, LE + k);
-      const T bp = shfl_up(bR, o);
-      const T sR = fma(m, bp, bR);
-      bR = lane >= o ? sR : bR;
-      if constexpr (!ONE) {
-        const T bn = shfl_down(bL, o);
-        const T sL = fma(m, bn, bL);
-        bL = lane + o < 32 ? sL : bL;
-      }
-    }
-    T cR = shfl_up(bR, 1), cL = T(0);     // value entering the lane from zero before the warp
-    if (lane == 0) cR = T(0);
-    if constexpr (!ONE) {
-      cL = shfl_down(bL, 1);
-      if (lane == 31) cL = T(0);
-    }
-    const T endR = fma(mulR, cR, ownR);   // at lane lastR: the warp's R end value
-    T inR = T(0), inL = T(0), tR, tL = T(0);
-    if (own) {
-      tR = __shfl_sync(FULL, endR, lastR);
-      if constexpr (!ONE) tL = __shfl_sync(FULL, bL, 0);
-    } else {
-      T* tot = totals + lw * nwl * 2;
-      if (lane == lastR) tot[2 * part] = endR;
-      if (!ONE && lane == 0) tot[2 * part + 1] = bL;
-      line_sync(nwl, lw);
-      const int j = lane & 15;
-      const bool left = lane >= 16;
-      T x = T(0);
-      if (j < nwl && !(ONE && left)) x = left ? tot[2 * (nwl - 1 - j) + 1] : tot[2 * j];
-      const T x0 = x;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if ((1 << k) < nwl) {
-          const T xp = __shfl_up_sync(FULL, x, 1 << k, 16);
-          const T sx = fma(qpow_bit<T>(a, LE + 5 + k), xp, x);
-          x = j >= (1 << k) ? sx : x;
-        }
-      }
-      T ex = __shfl_up_sync(FULL, x, 1, 16);   // value entering warp j
-      if (j == 0) ex = T(0);
-      const T lastw = (left || mir) ? qpow_bit<T>(a, LE + 5) : pick<T>(a.qlw, a.qlwf);
-      const T te = fma(lastw, ex, x0);
-      tR = __shfl_sync(FULL, te, nwl - 1);
-      inR = __shfl_sync(FULL, ex, part);
-      if constexpr (!ONE) {
-        tL = __shfl_sync(FULL, te, 15 + nwl);
-        inL = __shfl_sync(FULL, ex, 15 + nwl - part);
-      }
-    }
-    // ---- 3. boundary constants, carried to the lane
-    if (a.close) {
-      inR = fma(qwR, line_constant<T>(a, tR, tL), inR);
-      if constexpr (!ONE) inL = fma(qwL, line_constant<T>(a, tL, tR), inL);
-    }
-    if (a.close || !own) {
-      cR = fma(pwR, inR, cR);
-      if constexpr (!ONE) cL = fma(pwL, inL, cL);
-    }
-    // ---- 4. the scans from their carries -> D of the power (in F; two-sided
-    // forms keep W_R, W_L)
-    T y = cR;
-    if (resid) {
-#pragma unroll
-      for (int k = 0; k < E; ++k) {
-        if (valid(k)) y = fma(q, y, X[k]);
-        F[k] = fma(pick<T>(a.kap, a.kapf), y, F[k]);
-      }
-      y = cL;
-#pragma unroll
-      for (int k = E - 1; k >= 0; --k) {
-        if (valid(k)) y = fma(q, y, -X[k + 1]);
-        F[k] = fma(pick<T>(a.kap, a.kapf), y, F[k]);
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < E; ++k) {
-        if (valid(k)) y = fma(q, y, X[k]);
-        X[k] = y;
-      }
-      if constexpr (ONE) {
-#pragma unroll
-        for (int k = 0; k < E; ++k) F[k] = X[k];
-      } else {
-        y = cL;
-#pragma unroll
-        for (int k = E - 1; k >= 0; --k) {
-          if (valid(k)) y = fma(q, y, F[k]);
-          F[k] = JQ == JQ_D0 ? T(0.5) * (X[k] + y) : y;
-        }
-      }
-    }
-    if constexpr (JQ == JQ_D0) {
-      // D_0 vanishes at Dirichlet ends
-      if (end0) F[0] = T(0);
-      if (endN) {
-#pragma unroll
-        for (int k = 0; k < E; ++k)
-          if (RAGGED ? e0 + k == n - 1 : k == E - 1) F[k] = T(0);
-      }
-    }
-    // ---- 5. sum over the powers, write back for the next one
+    // ---- 2. scans and boundary constants
+    line_scans<T, JQ == JQ_D0, ONE, RAGGED, E>(a, ln, pw, X, F);
+    // ---- 3. sum over the powers, write back for the next one
     if constexpr (JQ != JQ_D0 && !ONE) {
       if (a.mode == MODE_RL) {
         // one-sided derivatives v^- = alpha D_R, v^+ = -alpha D_L and the
@@ -906,13 +975,13 @@ __device__ __forceinline__ double compute_lines(const SweepArgs& a, const TileSm
             const T r = fmax(fabs(vm), fabs(vp));
             const T mean = T(0.5) * (vm + vp);
             S[k] = T(0.5) * mean * mean + r * T(0.5) * (vm - vp);
-            if (line_ok && (!RAGGED || e0 + k < n)) rmax = fmax(rmax, r);
+            if (line_ok && (!RAGGED || ln.e0 + k < ln.n)) rmax = fmax(rmax, r);
           }
         } else if constexpr (GEN) {
           // H_d' = a_d (LINEAR) has |H_d'| = |a_d| everywhere; AFFINE_SQ
           // leaves (sigma, delta) and the last pass takes the box maximum
           const T av = pick<T>(a.vel, a.velf), aa = fabs(av);
-          T* cbase2 = static_cast<T*>(sm.lines2) + (cbase - lines);
+          T* cbase2 = static_cast<T*>(sm.lines2) + (ln.cbase - static_cast<T*>(sm.lines));
 #pragma unroll
           for (int k = 0; k < E; ++k) {
             const T vm = al * X[k];
@@ -922,7 +991,7 @@ __device__ __forceinline__ double compute_lines(const SweepArgs& a, const TileSm
               S[k] = av * mean + aa * T(0.5) * (vm - vp);
             } else {
               S[k] = av * mean;
-              if (RAGGED ? e0 + k < n : true) cbase2[chunk_off<E>(k)] = aa * T(0.5) * (vp - vm);
+              if (RAGGED ? ln.e0 + k < ln.n : true) cbase2[chunk_off<E>(k)] = aa * T(0.5) * (vp - vm);
             }
           }
           if (a.ham == HAM_LINEAR && line_ok) rmax = aa;
@@ -944,33 +1013,17 @@ __device__ __forceinline__ double compute_lines(const SweepArgs& a, const TileSm
       if (p + 1 < a.P) {
         // every lane of the line has read its window: of a line of several
         // warps, before the totals' barrier
-        if (own) __syncwarp();
-        if (!mir) {
-#pragma unroll
-          for (int k = 0; k < E; ++k)
-            if (RAGGED ? e0 + k < n : true) cbase[chunk_off<E>(k)] = F[k];
-        } else {
-#pragma unroll
-          for (int k = 0; k < E; ++k)
-            if (RAGGED ? e0 + E - 1 - k < n : true) cbase[chunk_off<E>(E - 1 - k)] = F[k];
-        }
-        line_sync(nwl, lw);
+        if (ln.own) __syncwarp();
+        ln.store(F);
+        line_sync(ln.nwl, ln.lw);
       }
     }
   }
 
-  if (own) __syncwarp();
-  if (!mir) {
-#pragma unroll
-    for (int k = 0; k < E; ++k)
-      if (RAGGED ? e0 + k < n : true) cbase[chunk_off<E>(k)] = S[k];
-  } else {
-#pragma unroll
-    for (int k = 0; k < E; ++k)
-      if (RAGGED ? e0 + E - 1 - k < n : true) cbase[chunk_off<E>(E - 1 - k)] = S[k];
-  }
-  // the epilogue reads contiguous lines by their own warps, strided ones by rows
-  if (a.contiguous) line_sync(nwl, lw); else __syncthreads();
+  if (ln.own) __syncwarp();
+  ln.store(S);
+  // the epilogue reads contiguous lines by their ln.own warps, strided ones by rows
+  if (a.contiguous) line_sync(ln.nwl, ln.lw); else __syncthreads();
   return cvt<double>(rmax);
 }
 
@@ -993,10 +1046,10 @@ struct Epilogue {
     EpiOps<T, TST> o{T(0), TST(0), TST(0)};
     if constexpr (EPI == EPI_ACC_ADD || EPI == EPI_ACC_AXPY) {
       o.acc = gload<CG>(static_cast<const T*>(a.acc) + gidx);
-    } else if constexpr (EPI == EPI_HEAT_FINAL || EPI == EPI_WAVE_FINAL) {
+    } else if constexpr (EPI == EPI_HEAT_FINAL || EPI == EPI_WAVE_FINAL || EPI == EPI_ADV_FINAL) {
       if (a.acc) o.acc = gload<CG>(static_cast<const T*>(a.acc) + gidx);
       o.x = gload<CG>(static_cast<const TST*>(a.un) + gidx);
-      if (EPI == EPI_HEAT_FINAL || !a.from_rest) o.y = gload<CG>(static_cast<const TST*>(a.us) + gidx);
+      if (EPI != EPI_WAVE_FINAL || !a.from_rest) o.y = gload<CG>(static_cast<const TST*>(a.us) + gidx);
     } else if constexpr (epi_hj_y(EPI)) {
       o.x = gload<CG>(static_cast<const TST*>(a.un) + gidx);
       if (a.out) o.y = gload<CG>(static_cast<const TST*>(a.out) + gidx);
@@ -1018,6 +1071,10 @@ struct Epilogue {
       const TST r = fma(TST(a.a0), o.x, TST(a.a1) * fma(TST(a.coefS), cvt<TST>(o.acc + s), o.y));
       static_cast<TST*>(a.dst)[gidx] = r;
       if (a.shadow) a.shadow[gidx] = cvt<float>(r);
+      if (nonfinite(r)) atomicOr(a.status, ST_NONFINITE);
+    } else if constexpr (EPI == EPI_ADV_FINAL) {
+      const TST r = fma(TST(a.a0), o.x, TST(a.a1) * (o.y + cvt<TST>(o.acc + s)));
+      static_cast<TST*>(a.dst)[gidx] = r;
       if (nonfinite(r)) atomicOr(a.status, ST_NONFINITE);
     } else if constexpr (EPI == EPI_WAVE_FINAL) {
       // u^{n+1} = 2u^n - u^{n-1} + coefS (acc + S)   (from rest: u^n + coefS/2 (acc + S))
