@@ -69,10 +69,10 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-#ifndef MOLT_BATCH_CHUNK
-#define MOLT_BATCH_CHUNK 4096
-#endif
-constexpr int kChunk = MOLT_BATCH_CHUNK;  // points per update work item
+// points per update work item: two a thread (64 problems, 2 steps: 8 / 4 / 2 /
+// 1 points a thread 11.1 / 10.8 / 10.6 / 10.8 ms, an L2 prefetch of the next
+// item 0.2 ms slower)
+constexpr int kChunk = 1024;
 
 // Grid barrier with a bounded wait (cooperative launch: all CTAs resident).
 __device__ __forceinline__ bool grid_sync(const BatchParams& p, bool skip) {
@@ -148,15 +148,6 @@ __device__ __forceinline__ int find_problem(const BatchParams& p, long long item
   return count - 1;
 }
 
-__device__ __forceinline__ int find_update(const BatchParams& p, long long chunk) {
-  int lo = 0, hi = p.nprob - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (p.updates[mid].first_chunk <= chunk) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
 // Compiled for two CTAs per SM (64 registers; more spills than at 128, but
 // the second resident CTA covers the phases' memory latency: 64 problems,
 // 7.09 -> 6.81 ms per RK3 step).
@@ -223,57 +214,40 @@ __global__ void __launch_bounds__(512, MOLT_BATCH_MIN_BLOCKS) batch_heat_kernel(
     if (p.phase_mask & 4) {
       const double a0 = rk[s][0], a1 = rk[s][1];
       bool bad = false;
-      for (long long c = blockIdx.x; c < p.chunks; c += gridDim.x) {
-        const BatchUpdate& U = p.updates[find_update(p, c)];
-        const long long i0 = (c - U.first_chunk) * kChunk;
-        const long long i1 = i0 + kChunk < U.total ? i0 + kChunk : U.total;
+      // chunk c of all problems goes to CTA c mod gridDim.x
+      for (int q = 0; q < p.nprob; ++q) {
+        const BatchUpdate& U = p.updates[q];
+        const long long rot = U.first_chunk % gridDim.x;
         const double* us = s == 0 ? U.u : (s == 1 ? U.st1 : U.st2);
         double* dstp = s == 0 ? U.st1 : (s == 1 ? U.st2 : U.u);
-        // L2 prefetch of the CTA's next chunk (u, the stage input, acc)
-        {
-          const long long cn = c + gridDim.x;
-          if (cn < p.chunks) {
-            const BatchUpdate& V = p.updates[find_update(p, cn)];
-            const long long j0 = (cn - V.first_chunk) * kChunk;
-            const long long j1 = j0 + kChunk < V.total ? j0 + kChunk : V.total;
-            const double* vs = s == 0 ? V.u : (s == 1 ? V.st1 : V.st2);
-            for (long long j = j0 + 16LL * threadIdx.x; j < j1; j += 16LL * blockDim.x) {
-              prefetch_l2(V.u + j);
-              prefetch_l2(j + 8 < j1 ? V.u + j + 8 : V.u + j);
-              if (vs != V.u) {
-                prefetch_l2(vs + j);
-                prefetch_l2(j + 8 < j1 ? vs + j + 8 : vs + j);
-              }
-              prefetch_l2(V.acc + j);
-              prefetch_l2(V.accy + j);
+        for (long long i0 = ((blockIdx.x + gridDim.x - rot) % gridDim.x) * kChunk; i0 < U.total;
+              i0 += (long long)gridDim.x * kChunk) {
+          const long long i1 = i0 + kChunk < U.total ? i0 + kChunk : U.total;
+          // (all loads of a thread's points are issued before its stores)
+          constexpr int kPer = kChunk / 512;
+          double uu[kPer], ss[kPer];
+          float aa[kPer], ay[kPer];
+#pragma unroll
+          for (int k = 0; k < kPer; ++k) {
+            const long long i = i0 + threadIdx.x + (long long)k * blockDim.x;
+            if (i < i1) {
+              ss[k] = __ldcg(us + i);
+              uu[k] = s == 0 ? 0.0 : __ldcg(U.u + i);
+              aa[k] = __ldcg(U.acc + i);
+              ay[k] = __ldcg(U.accy + i);
             }
           }
-        }
-        // all loads of a thread's points are issued before its stores (the
-        // CTA is the SM's only one, so memory parallelism comes from here)
-        constexpr int kPer = kChunk / 512;
-        double uu[kPer], ss[kPer];
-        float aa[kPer], ay[kPer];
 #pragma unroll
-        for (int k = 0; k < kPer; ++k) {
-          const long long i = i0 + threadIdx.x + (long long)k * blockDim.x;
-          if (i < i1) {
-            uu[k] = __ldcg(U.u + i);
-            ss[k] = __ldcg(us + i);
-            aa[k] = __ldcg(U.acc + i);
-            ay[k] = __ldcg(U.accy + i);
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < kPer; ++k) {
-          const long long i = i0 + threadIdx.x + (long long)k * blockDim.x;
-          if (i < i1) {
-            // the axis sums meet in FP64: no FP32 rounding at their joint size
-            const double t = fma(p.coefS, f2d(aa[k]), fma(p.coefS, f2d(ay[k]), ss[k]));
-            const double r = s == 0 ? t : fma(a0, uu[k], a1 * t);
-            dstp[i] = r;
-            U.copy[i] = d2f(r);
-            bad |= nonfinite(r);
+          for (int k = 0; k < kPer; ++k) {
+            const long long i = i0 + threadIdx.x + (long long)k * blockDim.x;
+            if (i < i1) {
+              // the axis sums meet in FP64: no FP32 rounding at their joint size
+              const double t = fma(p.coefS, f2d(aa[k]), fma(p.coefS, f2d(ay[k]), ss[k]));
+              const double r = s == 0 ? t : fma(a0, uu[k], a1 * t);
+              dstp[i] = r;
+              U.copy[i] = d2f(r);
+              bad |= nonfinite(r);
+            }
           }
         }
       }

@@ -153,18 +153,19 @@ struct SweepArgs : LineConst {
 // D_0 with linear weights (D0), or one side alone (LINEAR1, WENOZ1).
 enum JQuad { JQ_LINEAR = 0, JQ_WENOZ = 1, JQ_LEARNED = 2, JQ_D0 = 3, JQ_LINEAR1 = 4, JQ_WENOZ1 = 5 };
 
-// Registers per thread of the scan kernels: 128 (512 threads per SM), and 80
-// for the FP64 D_0 and one-sided linear sweeps, which are bound by the FP64
-// pipe: a spilled value costs them nothing, a second or third resident CTA
-// keeps the pipe busy while another loads or stores (5277^2 diffusion, 2
-// steps: 128 / 80 / 64 registers 5.11 / 3.87 / 3.97 ms; the two-sided
-// Hamilton-Jacobi sweeps of a 1759^2 FP64 run 2.05 / 2.29 / 2.36 ms).
-#ifndef MOLT_SWEEP_REGS_F64
-#define MOLT_SWEEP_REGS_F64 80
-#endif
-template <typename T, int JQ>
+// Registers per thread of the scan kernels: 128 (512 threads per SM), and
+// fewer for the D_0 and one-sided linear sweeps, whose other warps cover what
+// a spilled value costs.  FP64 (bound by the FP64 pipe: a second or third
+// resident CTA keeps it busy while another loads or stores) 80: 5277^2
+// diffusion, 2 steps, 128 / 80 / 64 registers 5.11 / 3.87 / 3.97 ms (the
+// two-sided Hamilton-Jacobi sweeps of a 1759^2 FP64 run 2.05 / 2.29 / 2.36 ms).
+// FP32 tiles of 8 and 4 points a lane 64 and 48: 201x151x101 wave, 5 steps,
+// 128 and 128 / 80 and 64 / 64 and 48 registers 0.80 / 0.70 / 0.68 ms; of 16
+// points 128 (96 and 80 measured the same).
+template <typename T, int JQ, int E = kE>
 __host__ __device__ constexpr int sweep_regs() {
-  return sizeof(T) == 8 && (JQ == JQ_D0 || JQ == JQ_LINEAR1) ? MOLT_SWEEP_REGS_F64 : 128;
+  if (JQ != JQ_D0 && JQ != JQ_LINEAR1) return 128;
+  return sizeof(T) == 8 ? 80 : (E == 4 ? 48 : (E == 8 ? 64 : 128));
 }
 
 // Shared-memory index of point e of a line whose lanes own E points each: one
@@ -208,6 +209,33 @@ __device__ __forceinline__ long long line_base(const LineGeom& g, long long l) {
 static __device__ __noinline__ float d2f_rare(double x) { return __double2float_rn(x); }
 static __device__ __noinline__ double f2d_rare(float x) { return double(x); }
 
+// The rare operands by integer operations: subnormal results (the 24-bit
+// significand moves right by 1..24 bits), overflow, infinities, NaN.
+__device__ __forceinline__ float d2f_slow(double x) {
+  const unsigned int hi = __double2hiint(x), lo = __double2loint(x);
+  const unsigned int sign = hi & 0x80000000u, e11 = (hi >> 20) & 0x7FFu;
+  if (e11 > 1150u) {
+    const bool nan = e11 == 0x7FFu && ((hi & 0xFFFFFu) | lo) != 0u;
+    return __uint_as_float(sign | (nan ? 0x7FFFFFFFu : 0x7F800000u));
+  }
+  const unsigned int sh = 897u - e11, full = ((hi & 0xFFFFFu) << 3) | (lo >> 29) | 0x800000u;
+  const unsigned int out = full & ((1u << sh) - 1u), mant = full >> sh;
+  const unsigned int half = 1u << (sh - 1u), below = (out & (half - 1u)) | (lo & 0x1FFFFFFFu);
+  const unsigned int up = (out & half) && (below || (mant & 1u));
+  return __uint_as_float(sign | (mant + up));
+}
+__device__ __forceinline__ double f2d_slow(float x) {
+  unsigned int u = __float_as_uint(x), off = 1792u;
+  if (((u >> 23) & 0xFFu) == 255u) {
+    if (u & 0x7FFFFFu) u |= 0x400000u;              // infinities, NaN
+  } else {
+    u = __float_as_uint(x * 4294967296.f);          // 2^32 x is normal
+    off = 864u;
+  }
+  const unsigned int hi = (u & 0x80000000u) | ((((u >> 23) & 0xFFu) + off) << 20) | ((u & 0x7FFFFFu) >> 3);
+  return __hiloint2double(int(hi), int(u << 29));
+}
+
 // double -> float, round to nearest even: normal results by integer
 // operations; results that round to zero (|x| < 2^-150) give the signed
 // zero; subnormal results, overflow, inf and NaN take the hardware conversion.
@@ -217,7 +245,7 @@ __device__ __forceinline__ float d2f(double x) {
   const unsigned int e11 = (hi >> 20) & 0x7FFu;
   if (e11 < 897u || e11 > 1150u) {
     if (e11 < 873u) return __uint_as_float(hi & 0x80000000u);
-    if constexpr (MOLT_CONV_SELECT) return __double2float_rn(x);
+    if constexpr (MOLT_CONV_SELECT) return d2f_slow(x);
     else return d2f_rare(x);
   }
   const unsigned int mant = ((hi & 0xFFFFFu) << 3) | (lo >> 29);
@@ -235,7 +263,7 @@ __device__ __forceinline__ double f2d(float x) {
   const unsigned int e8 = (u >> 23) & 0xFFu;
   if (e8 == 0u || e8 == 255u) {
     if ((u << 1) == 0u) return __hiloint2double(int(u & 0x80000000u), 0);
-    if constexpr (MOLT_CONV_SELECT) return double(x);
+    if constexpr (MOLT_CONV_SELECT) return f2d_slow(x);
     else return f2d_rare(x);
   }
   const unsigned int hi = (u & 0x80000000u) | ((e8 + 896u) << 20) | ((u & 0x7FFFFFu) >> 3);
@@ -1273,7 +1301,7 @@ __device__ __forceinline__ void publish_speed(const SweepArgs& a, double rmax) {
 
 // One tile per CTA, plain coalesced loads (any size / alignment).
 template <typename T, typename TIN, typename TST, int JQ, int EPI, bool RAGGED, int E = kE>
-__global__ void __maxnreg__((sweep_regs<T, JQ>())) sweep_kernel(const SweepArgs a) {
+__global__ void __maxnreg__((sweep_regs<T, JQ, E>())) sweep_kernel(const SweepArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   size_t used;
   const TileSmem sm = carve<T, JQ>(smem_raw, a, &used);
