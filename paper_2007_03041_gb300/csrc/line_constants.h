@@ -82,6 +82,12 @@ inline void set_line_constants(SweepArgs& a, const QuadTable& qt, int N, int E, 
   a.kAl = float(a.kA - double(a.kAh));
   a.kBh = float(a.kB);
   a.kBl = float(a.kB - double(a.kBh));
+  // one-sided derivatives alpha D: D carries the factor (1-q)/(1-q32); the
+  // two-sided linear kernels of a Hamilton-Jacobi pass take it in their taps
+  const double al = f32_sweeps ? a.alpha * std::expm1(lq) / std::expm1(-nu) : a.alpha;
+  a.alphaf = float(al);
+  if (a.mode == MODE_RL)
+    for (int i = 0; i < 5; ++i) a.b[i] *= al;
   // FP32 copies
   for (int i = 0; i < 5; ++i) a.bf[i] = float(a.b[i]);
   a.f0f = float(a.f0);
@@ -93,7 +99,6 @@ inline void set_line_constants(SweepArgs& a, const QuadTable& qt, int N, int E, 
   a.qlastf = float(a.qlast);
   a.qlwf = float(a.qlw);
   // one-sided derivatives alpha D: D carries the factor (1-q)/(1-q32)
-  a.alphaf = float(f32_sweeps ? a.alpha * std::expm1(lq) / std::expm1(-nu) : a.alpha);
 }
 
 }  // namespace molt

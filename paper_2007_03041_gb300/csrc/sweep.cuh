@@ -993,8 +993,9 @@ __device__ __forceinline__ double compute_lines(const SweepArgs& a, const TileSm
     if constexpr (JQ != JQ_D0 && !ONE) {
       if (a.mode == MODE_RL) {
         // one-sided derivatives v^- = alpha D_R, v^+ = -alpha D_L and the
-        // per-axis part of the Lax-Friedrichs Hamiltonian (Sec. 2.5)
-        const T al = pick<T>(a.alpha, a.alphaf);
+        // per-axis part of the Lax-Friedrichs Hamiltonian (Sec. 2.5); the
+        // linear rule's taps carry the factor alpha
+        const T al = JQ == JQ_LINEAR ? T(1) : pick<T>(a.alpha, a.alphaf);
         if (!GEN || a.ham == HAM_HALF_SQ) {
 #pragma unroll
           for (int k = 0; k < E; ++k) {
@@ -1008,21 +1009,19 @@ __device__ __forceinline__ double compute_lines(const SweepArgs& a, const TileSm
         } else if constexpr (GEN) {
           // H_d' = a_d (LINEAR) has |H_d'| = |a_d| everywhere; AFFINE_SQ
           // leaves (sigma, delta) and the last pass takes the box maximum
-          const T av = pick<T>(a.vel, a.velf), aa = fabs(av);
+          const T ah = T(0.5) * al * pick<T>(a.vel, a.velf), aa = fabs(ah);
           T* cbase2 = static_cast<T*>(sm.lines2) + (ln.cbase - static_cast<T*>(sm.lines));
 #pragma unroll
           for (int k = 0; k < E; ++k) {
-            const T vm = al * X[k];
-            const T vp = -al * F[k];
-            const T mean = T(0.5) * (vm + vp);
+            const T mean2 = X[k] - F[k], diff = X[k] + F[k];   // v^- + v^+, v^- - v^+ (over al)
             if (a.ham == HAM_LINEAR) {
-              S[k] = av * mean + aa * T(0.5) * (vm - vp);
+              S[k] = fma(ah, mean2, aa * diff);
             } else {
-              S[k] = av * mean;
-              if (RAGGED ? ln.e0 + k < ln.n : true) cbase2[chunk_off<E>(k)] = aa * T(0.5) * (vp - vm);
+              S[k] = ah * mean2;
+              if (ln.valid(k)) cbase2[chunk_off<E>(k)] = -aa * diff;
             }
           }
-          if (a.ham == HAM_LINEAR && line_ok) rmax = aa;
+          if (a.ham == HAM_LINEAR && line_ok) rmax = fabs(pick<T>(a.vel, a.velf));
         }
       } else {
 #pragma unroll
@@ -1138,8 +1137,8 @@ struct Epilogue {
     return F;
   }
 
-  // s2: the second line buffer's value (two_out).  Returns the point's
-  // scaled wave speed where the last pass determines it (AFFINE_SQ), else 0.
+  // s2: the second line buffer's value (two_out).  Returns the point's wave
+  // speed over vmax where the last pass determines it (AFFINE_SQ), else 0.
   __device__ __forceinline__ T store_general(long long gidx, T s, const EpiOps<T, TST>& o, TST z, T s2) const {
     if constexpr (EPI == EPI_HJ_XG) {
       if (a.out) static_cast<TST*>(a.out)[gidx] = TST(s);
@@ -1157,7 +1156,7 @@ struct Epilogue {
         const TST sbar = TST(a.h0) + o.y + TST(s);
         const TST m = fabs(sbar) + fabs(z) + fabs(TST(s2));
         H = TST(0.5) * sbar * sbar - m * (z + TST(s2));
-        speed = T(TST(a.vmax) * m);
+        speed = T(m);   // times vmax, once a thread
       } else {
         H = o.y + TST(s);
       }
@@ -1184,7 +1183,7 @@ constexpr int kEpiBatch = MOLT_EPI_BATCH;
 // p0, p0 + pstep, ... of a line: shared values sp[k*pdelta] and sp2[k*pdelta]
 // (second line buffer, or null), global index g + k*gstep, B points per
 // batch with all loads of a batch issued before its stores.  Returns the
-// largest scaled wave speed it determined.
+// largest wave speed it determined, over vmax.
 template <typename T, typename TST, int EPI, bool CG, int B>
 __device__ __forceinline__ double epilogue_general(const Epilogue<T, TST, EPI, CG>& ep, const T* sp, const T* sp2,
                                                    long long g, int p0, int n, int pstep, long long gstep,
@@ -1253,8 +1252,8 @@ __device__ __forceinline__ double epilogue_tile(const SweepArgs& a, const T* lin
   (void)sstep;
   if constexpr (epi_hj_gen(EPI)) {
     // more operands per point: a smaller batch
-    return epilogue_general<T, TST, EPI, CG, 4>(ep, sp, lines2 ? lines2 + (sp - lines) : nullptr, g0, p0, n, pstep,
-                                                 gstep, pdelta);
+    return a.vmax * epilogue_general<T, TST, EPI, CG, 4>(ep, sp, lines2 ? lines2 + (sp - lines) : nullptr, g0, p0, n,
+                                                          pstep, gstep, pdelta);
   } else {
     long long g = g0;
     for (int pb = p0; pb < n; pb += kEpiBatch * pstep) {
