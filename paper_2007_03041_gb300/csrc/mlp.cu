@@ -176,6 +176,12 @@ __device__ __forceinline__ void frag_b(const __nv_bfloat16 (*M)[LD], int c0, int
   b1 = pair_of(M[8 + 2 * t][c0 + g], M[9 + 2 * t][c0 + g]);
 }
 
+__global__ void mlp_zero_kernel(float* grad, float* loss) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < kMlpParams) grad[i] = 0.f;
+  else if (i == kMlpParams) *loss = 0.f;
+}
+
 __global__ void __launch_bounds__(32 * kGradWarps) mlp_grad_kernel(const MlpBlob* blob, const float* __restrict__ x,
                                                                    const float* __restrict__ y, long long n,
                                                                    float* __restrict__ grad, float* loss) {
@@ -499,9 +505,9 @@ molt_status molt_mlp_loss_grad(const void* blob, const float* x, const float* y,
                                void* cuda_stream) {
   if (n < 0 || !blob || !grad || !loss || !aligned16(blob) || !aligned16(grad)) return MOLT_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  if (cudaMemsetAsync(grad, 0, sizeof(float) * kMlpParams, s) != cudaSuccess ||
-      cudaMemsetAsync(loss, 0, sizeof(float), s) != cudaSuccess)
-    return MOLT_ECUDA;
+  // one launch for both sums (two memsets took 2 us more a minibatch)
+  mlp_zero_kernel<<<(kMlpParams + 1 + 127) / 128, 128, 0, s>>>(grad, loss);
+  if (cudaGetLastError() != cudaSuccess) return MOLT_ECUDA;
   if (n == 0) return MOLT_OK;
   if (!x || !y || !aligned16(x) || !aligned16(y)) return MOLT_EINVAL;
   const long long groups = (n + 15) / 16;
