@@ -57,7 +57,7 @@ WORKLOAD = {
 # write acc; last sweep with the FP64 leapfrog update: read copy + acc + u^n
 # + u^{n-1} (FP64), write u^{n+1} (FP64) + its FP32 copy; separate update:
 # read acc + u^n + u^{n-1}, write u^{n+1} + copy
-BYTES_PER_DOF = {"x": 8, "yz": 12, "last_update": 36, "update": 32}
+BYTES_PER_DOF = {"x": 8, "yz": 12, "last_update": 36, "update": 32, "update_x": 36}
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per DOF per launch
 # from one ncu capture of each kernel on the 512^3 step itself (one-pass
 # metrics); a kernel changed since its capture has no entry
@@ -384,6 +384,8 @@ def run_ours(args):
                                 (M.KERNEL_ACC_ADD, "sweep_tma_kernel ACC_ADD (y and z lines)"))),
                         ("last_update", ((M.KERNEL_LANES_WAVE_FINAL,
                                           "lanes_sweep_kernel WAVE_FINAL (z lines + FP64 leapfrog update)"),)),
+                        ("update_x", ((M.KERNEL_XLINES_WAVE,
+                                       "xline_wave_kernel (FP64 leapfrog update + next step's x sweep)"),)),
                         ("update", ((M.KERNEL_UPDATE, "wave_update_kernel (FP64 leapfrog update)"),))):
         for kind, kname in kinds:
             tot, cnt = M.molt_profile_read(ctx, kind)

@@ -323,7 +323,9 @@ typedef enum {
                                      wave step with the FP64 leapfrog update  */
   MOLT_KERNEL_XLINES_STORE = 15,   /* warp-per-line x sweeps (MOLT_OPT_XLINES): */
   MOLT_KERNEL_XLINES_ACC_SET = 16, /*   STORE, ACC_SET, and ACC_ADD / the       */
-  MOLT_KERNEL_XLINES_ACC_ADD = 17  /*   advection-diffusion accumulations       */
+  MOLT_KERNEL_XLINES_ACC_ADD = 17, /*   advection-diffusion accumulations,      */
+  MOLT_KERNEL_XLINES_WAVE = 18     /*   and a wave step's FP64 update with the
+                                        next step's x sweep                     */
 } molt_kernel_kind;
 
 /* With MOLT_OPT_PROFILE on: synchronises the stream, returns the summed

@@ -156,7 +156,7 @@ __device__ __forceinline__ int find_problem(const BatchParams& p, long long item
 #endif
 #ifndef MOLT_BATCH_KERNEL_TU
 // defined in csrc/batch.cu (its own translation unit: FP32 <-> FP64
-// conversions selected in place, MOLT_CONV_SELECT)
+// conversions in place, MOLT_CONV_SELECT)
 __global__ void batch_heat_kernel(const BatchParams p);
 #else
 __global__ void __launch_bounds__(512, MOLT_BATCH_MIN_BLOCKS) batch_heat_kernel(const BatchParams p) {

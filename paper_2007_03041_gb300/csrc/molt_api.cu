@@ -238,16 +238,12 @@ int device_sms() {
 
 // Points per lane for a line of n points: the largest of 16, 8, 4 whose
 // tile fits the line exactly (n = 32 * E * nwl, nwl <= 16 warps), else
-// masked (ragged) tiles of the shape with the least work.  FP64 sweeps of grids with few lines (fewer
-// than 16 warps per SM at that E; nlines counts the lines of every sweep
-// running at the same time) are bound by the latency of their recurrences
-// on the FP64 pipe, not by bandwidth, and take a shorter chain per lane:
-// two warps per line from 512 points on, and the largest E that still puts
-// 3 warps per SM in flight, else the smallest that fits.  Measured FP64 heat
-// steps (ms; axes one after another / both at once):
-//   256^2:  E=4 0.130/0.095  E=8 0.166/0.089
-//   512^2:  E=4 0.345/0.285  E=8 0.301/0.255  E=16 0.337/0.588
-//   1024^2: E=8 1.064        E=16 0.996      2048^2: E=8 3.91  E=16 3.68
+// masked (ragged) tiles of the shape with the least work.  FP64 sweeps of
+// grids with few lines (fewer than 16 warps per SM at that E; nlines counts the
+// lines of every sweep running at the same time) are bound by the FP64 pipe of
+// the schedulers that hold their few warps and spread over more of them: two
+// warps per line from 512 points on, and the largest E that still puts 3 warps
+// per SM in flight, else the smallest that fits.
 #ifndef MOLT_PREFER_E
 #define MOLT_PREFER_E 16
 #endif
@@ -707,6 +703,11 @@ bool plan_xlines(const molt_ctx* c, const Problem& p, int epi, const Plan& pl, b
     X.bR[i] = L.bR[i];
     X.bL[i] = L.bL[i];
   }
+  // residual form of D_0 (the planner's constants)
+  X.d0 = a.mode == MODE_0 ? a.d0 : 0;
+  X.f0 = a.f0f;
+  X.f1 = a.f1f;
+  X.kap = a.kapf;
   X.q = L.q;
   // Kogge-Stone multipliers (q^16)^(2^k), from the FP32 q the scans run
   double qk = std::pow(double(L.q), double(kXlSeg));
@@ -1570,7 +1571,7 @@ __global__ void advdiff_update_t_kernel(const T* __restrict__ acc, const T* __re
     const long long x = x0 + i, y = y0 + j;
     if (x < nx && y < ny) {
       v[k] = acc[y * nx + x] + tile[i][j];
-      w[k] = un[y * nx + x];
+      w[k] = a0 != 0.0 ? un[y * nx + x] : T(0);
       z[k] = us[y * nx + x];
     }
   }
@@ -1749,9 +1750,40 @@ molt_status advdiff_step(molt_ctx* c, Problem& p, void* u) {
 #ifndef MOLT_WAVE_FUSED_UPDATE
 #define MOLT_WAVE_FUSED_UPDATE 0
 #endif
-molt_status wave_step(molt_ctx* c, Problem& p, void* cur, void* prev, bool from_rest, bool in_place_variant) {
+// The fused kernel (xline_wave_kernel) that takes the place of step n's update
+// and step n+1's x sweep inside one molt_step call, and of the state's FP32
+// copy and the first x sweep; false: the problem's x lines do not run on the
+// warp-per-line kernel.
+bool plan_wave_x(molt_ctx* c, const Problem& p, const void* a0, const void* a1, XLineArgs* xa) {
+  if (!p.shadow || MOLT_WAVE_FUSED_UPDATE || p.d.ndim < 2) return false;
+  if ((reinterpret_cast<uintptr_t>(a0) | reinterpret_cast<uintptr_t>(a1)) & 15) return false;
+  Plan pl;
+  if (plan_axis(c, p, 0, MODE_0, p.d.P, step_alpha(p), &pl) != MOLT_OK) return false;
+  pl.a.in = p.shadow;
+  pl.a.acc = p.acc;
+  return plan_xlines(c, p, EPI_ACC_SET, pl, true, xa);
+}
+
+// The FP32 copy of the state at the start of a call, with the first x sweep.
+molt_status wave_copy_x(molt_ctx* c, const Problem& p, const void* u, const XLineArgs& xa) {
+  XWaveArgs w{};
+  w.un = static_cast<const double*>(u);
+  w.shadow = p.shadow;
+  w.copy_only = 1;
+  w.status = c->status_dev;
+  molt_ctx::Rec rec;
+  record_begin(c, &rec, MOLT_KERNEL_XLINES_ACC_SET);
+  const cudaError_t e = launch_xlines_wave(xa, w, c->stream);
+  record_end(c, &rec);
+  return e == cudaSuccess ? MOLT_OK : cuda_fail(c, e, "state copy and x sweep");
+}
+
+// One leapfrog step; x_done: the x sums of this step are in acc already;
+// next_x: the step's update also runs the next step's x sweep.
+molt_status wave_step(molt_ctx* c, Problem& p, void* cur, void* prev, bool from_rest, bool in_place_variant,
+                      bool x_done = false, const XLineArgs* next_x = nullptr) {
   const double alpha = step_alpha(p);
-  for (int ax = 0; ax < p.d.ndim; ++ax) {
+  for (int ax = x_done ? 1 : 0; ax < p.d.ndim; ++ax) {
     Plan pl;
     molt_status st = plan_axis(c, p, ax, MODE_0, p.d.P, alpha, &pl);
     if (st != MOLT_OK) return st;
@@ -1794,7 +1826,17 @@ molt_status wave_step(molt_ctx* c, Problem& p, void* cur, void* prev, bool from_
       }
     }
     if ((st = run(c, p, epi, pl)) != MOLT_OK) return st;
-    if (last && split_update) {
+    if (last && split_update && next_x) {
+      const XWaveArgs w{static_cast<const double*>(cur), static_cast<const double*>(prev),
+                        static_cast<double*>(in_place_variant ? cur : prev),
+                        in_place_variant ? static_cast<double*>(prev) : nullptr, p.shadow, -p.d.beta * p.d.beta,
+                        from_rest ? 1 : 0, 0, c->status_dev};
+      molt_ctx::Rec rec;
+      record_begin(c, &rec, MOLT_KERNEL_XLINES_WAVE);
+      const cudaError_t e = launch_xlines_wave(*next_x, w, c->stream);
+      record_end(c, &rec);
+      if (e != cudaSuccess) return cuda_fail(c, e, "wave update and x sweep");
+    } else if (last && split_update) {
       molt_ctx::Rec rec;
       record_begin(c, &rec, MOLT_KERNEL_UPDATE);
       wave_update_kernel<<<stream_grid(p.total), 256, 0, c->stream>>>(
@@ -2469,8 +2511,12 @@ molt_status molt_step(molt_ctx* c, void* const* u, void* const* u_prev, int nste
   if ((e = cudaMemcpyAsync(c->t_dev, t0.data(), sizeof(double) * np, cudaMemcpyHostToDevice, c->stream)) !=
       cudaSuccess)
     return cuda_fail(c, e, "t upload");
+  std::vector<XLineArgs> wave_x(np);
+  std::vector<char> fuse(np, 0);   // wave problems whose x sweeps run with the update (or the copy) before them
   for (int i = 0; i < np && nsteps > 0; ++i) {
-    molt_status st = refresh_shadow(c, c->probs[i], u[i]);
+    Problem& p = c->probs[i];
+    fuse[i] = p.d.pde == MOLT_PDE_WAVE && plan_wave_x(c, p, u[i], u_prev[i], &wave_x[i]);
+    const molt_status st = fuse[i] ? wave_copy_x(c, p, u[i], wave_x[i]) : refresh_shadow(c, p, u[i]);
     if (st != MOLT_OK) return st;
   }
   molt_status bst = batch_prepare(c);
@@ -2493,7 +2539,7 @@ molt_status molt_step(molt_ctx* c, void* const* u, void* const* u_prev, int nste
         void* cur = even ? u[i] : u_prev[i];
         void* prev = even ? u_prev[i] : u[i];
         const bool variant = (k == nsteps - 1) && even;   // keep u = newest on return
-        st = wave_step(c, p, cur, prev, from_rest, variant);
+        st = wave_step(c, p, cur, prev, from_rest, variant, fuse[i], fuse[i] && k + 1 < nsteps ? &wave_x[i] : nullptr);
         t_inout[i] += p.d.dt;
       } else if (p.d.pde == MOLT_PDE_ADVDIFF) {
         st = advdiff_step(c, p, u[i]);

@@ -282,22 +282,21 @@ inline std::vector<double> pack_nonuniform(const std::vector<double>& cR, const 
   return t;
 }
 
-// One group of V values of a table.  The loads are volatile: left free, the
-// compiler gathers a whole chunk's tables ahead of the arithmetic and spills
-// them (2 KB a thread with WENO-Z weights).
+// One group of V values of a table.  ORDERED loads are volatile: left free,
+// the compiler gathers a whole chunk's WENO-Z tables ahead of the arithmetic
+// and spills them (2 KB a thread); the linear rule's it may move.
 template <typename T, int V> struct NuVec { T v[V]; };
-__device__ __forceinline__ void nu_load(NuVec<float, 4>& x, const float* p) {
-  asm volatile("ld.global.nc.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x.v[0]), "=f"(x.v[1]), "=f"(x.v[2]), "=f"(x.v[3]) : "l"(p));
-}
-__device__ __forceinline__ void nu_load(NuVec<float, 2>& x, const float* p) {
-  asm volatile("ld.global.nc.v2.f32 {%0,%1}, [%2];" : "=f"(x.v[0]), "=f"(x.v[1]) : "l"(p));
-}
-__device__ __forceinline__ void nu_load(NuVec<double, 2>& x, const double* p) {
-  asm volatile("ld.global.nc.v2.f64 {%0,%1}, [%2];" : "=d"(x.v[0]), "=d"(x.v[1]) : "l"(p));
-}
-__device__ __forceinline__ void nu_load(NuVec<double, 1>& x, const double* p) {
-  asm volatile("ld.global.nc.f64 %0, [%1];" : "=d"(x.v[0]) : "l"(p));
-}
+#define MOLT_NU_LOAD(TYPE, V, TEXT, ...)                                          \
+  template <bool ORDERED>                                                          \
+  __device__ __forceinline__ void nu_load(NuVec<TYPE, V>& x, const TYPE* p) {      \
+    if constexpr (ORDERED) asm volatile(TEXT : __VA_ARGS__ : "l"(p));              \
+    else asm(TEXT : __VA_ARGS__ : "l"(p));                                         \
+  }
+MOLT_NU_LOAD(float, 4, "ld.global.nc.v4.f32 {%0,%1,%2,%3}, [%4];", "=f"(x.v[0]), "=f"(x.v[1]), "=f"(x.v[2]), "=f"(x.v[3]))
+MOLT_NU_LOAD(float, 2, "ld.global.nc.v2.f32 {%0,%1}, [%2];", "=f"(x.v[0]), "=f"(x.v[1]))
+MOLT_NU_LOAD(double, 2, "ld.global.nc.v2.f64 {%0,%1}, [%2];", "=d"(x.v[0]), "=d"(x.v[1]))
+MOLT_NU_LOAD(double, 1, "ld.global.nc.f64 %0, [%1];", "=d"(x.v[0]))
+#undef MOLT_NU_LOAD
 // Values per group: 16 bytes, with WENO-Z weights (44 values a point) 8.
 template <typename T, bool WENO>
 __host__ __device__ constexpr int nu_group() { return (WENO ? 8 : 16) / int(sizeof(T)); }
@@ -370,7 +369,7 @@ __global__ void __launch_bounds__(512) nonuniform_kernel(const NuArgs a) {
 #pragma unroll
     for (int j = 0; j < E / V; ++j) {
       NuVec<T, V> x;
-      nu_load(x, tab + (size_t(slot) * (E / V) + j) * tstride + tl * V);
+      nu_load<WENO>(x, tab + (size_t(slot) * (E / V) + j) * tstride + tl * V);
 #pragma unroll
       for (int k = 0; k < V; ++k) q[j * V + k] = x.v[k];
     }
@@ -453,7 +452,7 @@ __global__ void __launch_bounds__(512) nonuniform_kernel(const NuArgs a) {
         NuVec<T, V> t[NS];
 #pragma unroll
         for (int s = 0; s < NS; ++s)
-          nu_load(t[s], tab + (size_t(2 + side * NS + s) * (E / V) + j) * tstride + tl * V);
+          nu_load<WENO>(t[s], tab + (size_t(2 + side * NS + s) * (E / V) + j) * tstride + tl * V);
 #pragma unroll
         for (int kk = 0; kk < V; ++kk) {
           const int k = j * V + kk;

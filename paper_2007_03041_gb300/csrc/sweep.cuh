@@ -5,31 +5,30 @@
 //
 // Mapping.  A CTA owns W lines of one axis.  The lines are staged in shared
 // memory (converted to the compute type T) with ghost cells on both ends;
-// each line is processed by `nwl` warps and every lane owns kE consecutive
+// each line is processed by `nwl` warps and every lane owns E consecutive
 // points of it in registers.  Per application of D:
-//   1. local integrals J_R(x_e) = sum_l c_l v_{e+l} and J_L(x_e) =
-//      sum_l c_l v_{e-l} (Sec. 2.4 / App. C, optionally WENO-Z weighted) from
-//      a register window of the lane's points plus 3 neighbours per side;
-//   2. the recurrences I_R(x_i) = q I_R(x_{i-1}) + J_R(x_i) and
-//      I_L(x_i) = q I_L(x_{i+1}) + J_L(x_i) (Sec. 2.4) as affine scans:
-//      a serial fold per lane, a shuffle scan across the warp, a shared-
-//      memory scan across the warps of a line (the exact block split of the
-//      convolution sums, Sec. 3, without any truncation);
-//   3. the boundary constants from the line totals in FP64 (Sec. 2.3:
-//      periodic A = I(b)/(1-mu), B = I(a)/(1-mu); Dirichlet: the 2x2 system
-//      with determinant 1-mu^2, Sec. 3.3), folded into the scans as their
-//      initial values so that A e^{-alpha(x-a)} needs no pow();
-//   4. a fix-up pass giving L^{-1} (in FP32 the recurrence is accumulated
-//      with a compensation term: exact product error by FMA, TwoSum for the
-//      addition), then D = v - L^{-1}.
+//   1. forcings of the recurrences from a register window of the lane's points
+//      plus 3 neighbours per side, as filters of the differences d_i = v_i -
+//      v_{i-1} (Sec. 2.4 / App. C; linear, WENO-Z or learned weights);
+//   2. the recurrences of v - L_R^{-1}[v] and v - L_L^{-1}[v] as scans: a serial
+//      fold per lane, a shuffle scan across the warp, a scan of the warps'
+//      totals (the exact block split of the convolution sums, Sec. 3, without
+//      any truncation);
+//   3. the boundary constants from the line totals (Sec. 2.3: periodic
+//      C = T/(1-mu); Dirichlet: the 2x2 system with determinant 1-mu^2,
+//      Sec. 3.3), folded into the scans as their initial values;
+//   4. the scans again from their carries, which give D.
 // D is written back to shared memory for the next power.  The epilogue runs
-// in the coalesced load mapping.
+// in the coalesced load mapping.  compute_lines() has the algebra.
 //
 // Precision plumbing.  GB300 executes FP64 arithmetic and FP64<->FP32
-// conversions at a small fraction of the FP32 rate, so per-point FP64 work is
-// kept to the update itself: sweeps read an FP32 copy of the state (written
-// by the previous update), conversions are done with integer bit operations,
-// and only the state update uses FP64 fused multiply-adds.
+// conversions at a small fraction of the FP32 rate (two FP64 FMAs per clock
+// and SM, 64 cycles of a scheduler's pipe per warp instruction), so FP32
+// sweeps keep FP64 to the update itself: they read an FP32 copy of the state
+// (written by the previous update), conversions are done with integer bit
+// operations, and only the state update uses FP64 fused multiply-adds.  FP64
+// sweeps are bound by that pipe: their form is the one with the fewest
+// operations a point.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -197,12 +196,12 @@ __device__ __forceinline__ long long line_base(const LineGeom& g, long long l) {
 // The hardware conversions between FP32 and FP64 run on the FP64 pipe, which
 // is narrow on this part; the common operands are converted by integer
 // operations on the bit patterns instead.  The rare operands leave through a
-// call, so that the hardware conversion runs for them alone (a plain branch
-// to it would be if-converted, executing it for every operand).  A
-// translation unit whose kernels have no registers to spare for a call
-// defines MOLT_CONV_SELECT 1: the hardware conversion is then selected in
-// place (measured: the batched heat step, 6.78 ms with it, 8.18 with calls;
-// the 512^3 wave step, 1.93 ms with it, 1.76 with calls).
+// call to the hardware conversion (a plain branch to it would be if-converted,
+// executing it for every operand).  A translation unit whose kernels have no
+// registers to spare for a call defines MOLT_CONV_SELECT 1: the rare operands
+// then take integer operations in place too (same results; measured: the
+// batched heat step 6.8 ms with calls against 5.1; the 512^3 wave step 1.77 ms
+// with calls against 1.85 in place).
 #ifndef MOLT_CONV_SELECT
 #define MOLT_CONV_SELECT 0
 #endif
@@ -449,10 +448,6 @@ __device__ __forceinline__ TileSmem carve(unsigned char* smem, const SweepArgs& 
   }
   return t;
 }
-
-// Packed FP32x2 arithmetic of sm_100+ (line-per-lane and x-line sweeps).
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 
 // ------------------------------------------------------------- line constants
 template <typename T>

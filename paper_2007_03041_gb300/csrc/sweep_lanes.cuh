@@ -70,6 +70,9 @@
 
 namespace molt {
 
+// Packed FP32x2 arithmetic of sm_100+.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
 constexpr int kLE = 16;      // points per thread (one segment)
 constexpr int kLW = 32;      // lines per tile (one per lane)
 constexpr int kLMaxSeg = 32; // segments per line (warps per CTA)

@@ -19,4 +19,7 @@ cudaError_t launch_lanes(int epi, const LanesArgs& a, const CUtensorMap& map, cu
 // launch of 8-warp CTAs, at most (SMs x resident CTAs).
 cudaError_t launch_xlines(int epi, const XLineArgs& a, cudaStream_t s);
 
+// The update of one wave step and the x sweep (ACC_SET into a.acc) of the next.
+cudaError_t launch_xlines_wave(const XLineArgs& a, const XWaveArgs& w, cudaStream_t s);
+
 }  // namespace molt

@@ -17,8 +17,10 @@
 //
 // Arithmetic (the difference form of the recurrences, Sec. 2.4).  As in the
 // line-per-lane kernel: per power, the first differences of the segment's
-// window, K_R and K_L as 5-tap filters of them, the scans of the segment from
-// zero -> the segment totals (b_R, b_L).  The value entering segment s from
+// window, for D_0 the residual form of csrc/sweep.cuh (the scans take the
+// differences, the quadrature is a 3-tap filter of the second differences),
+// else K_R and K_L as 5-tap filters, the scans of the segment from zero -> the
+// segment totals (b_R, b_L).  The value entering segment s from
 // the left is sum_{i<s} (q^16)^{s-1-i} b_R[i] + (q^16)^s C_R: the inclusive
 // scan X_s = b_R[s] + q^16 X_{s-1} over the lanes runs as a Kogge-Stone scan
 // in log2 S shuffle steps with multipliers q^(16 d) (no look-back
@@ -28,7 +30,7 @@
 // Dirichlet solve of Sec. 3.3) C = kA T_same + kB T_other run in FP64 on the
 // lanes within reach of an end (segments whose weight (q^16)^s is at least
 // 2^-26), one FP64 product chain per lane; the scans again from the carries
-// give D = W_R + W_L.  The second power starts from D of the first, whose
+// give D.  The second power starts from D of the first, whose
 // ghost points come from the neighbouring lanes' registers.
 #pragma once
 
@@ -51,13 +53,6 @@ constexpr int kXlBuf = 512;       // floats of one warp's line group (G n)
 #define MOLT_XL_STAGES 4
 #endif
 constexpr int kXlStages = MOLT_XL_STAGES;
-// 1: the 5-tap filters of both directions as packed FP32x2 operations (same
-// sums in the same order; measured on the 512^3 wave x sweep: 0.304 ms
-// against 0.287 with scalar taps -- building the operand pairs costs more
-// than the halved FMA count saves)
-#ifndef MOLT_XL_PAIRED_TAPS
-#define MOLT_XL_PAIRED_TAPS 0
-#endif
 constexpr size_t kXlSmemBytes = size_t(kXlWarps) * kXlStages * kXlBuf * sizeof(float);
 
 struct XLineArgs {
@@ -70,6 +65,8 @@ struct XLineArgs {
   int lb;                // segments within reach of an end: (q^16)^s >= 2^-26 for s < lb
   int needA, needB;      // the boundary constants use T of the same / the other direction
   float bR[5], bL[5];    // K_R = sum_i bR[i] d[t+i], K_L = sum_i bL[i] d[u+5-i] (window indices)
+  int d0;                // D_0 in residual form (csrc/sweep.cuh): f0, f1, kap
+  float f0, f1, kap;
   float q;               // e^{-nu} (FP32)
   float qd[5];           // (q^16)^(2^k): multipliers of the Kogge-Stone steps
   double kA, kB;         // boundary constants C = kA T_same + kB T_other (FP64)
@@ -159,9 +156,10 @@ __device__ __forceinline__ void xl_apply_D(const XLineArgs& a, const XlLane& L, 
   const bool active = SF ? true : L.s < S;
   const int first = SF ? 0 : L.lane - L.s, last = first + S - 1;
   const int rs = active ? S - 1 - L.s : -1;          // segments to the right
-  float2 Y[kXlSeg];
-  float2 y;
+  float X[kXlSeg + 1];
+  float r = 0.f, l = 0.f;
   {
+    float d[21];
     // window w[k] = v_{p0-3+k}: own points at k = 3..18, ghosts from the neighbours
     float w[22];
 #pragma unroll
@@ -185,47 +183,55 @@ __device__ __forceinline__ void xl_apply_D(const XLineArgs& a, const XlLane& L, 
         for (int k = 19; k < 22; ++k) w[k] = 2.f * w[18] - w[36 - k];
       }
     }
-    float d[21];
 #pragma unroll
     for (int k = 0; k < 21; ++k) d[k] = w[k + 1] - w[k];
-#if MOLT_XL_PAIRED_TAPS
-    // Y[t] = (K_R(p0+t), K_L(p0+15-t)) as packed FP32x2 filters: with
-    // P[k] = (d[k], d[20-k]), Y[t] = sum_i (bR[i], bL[i]) P[t+i]
+    if (a.d0) {
+      // residual form: X the differences, D the FIR part
 #pragma unroll
-    for (int t = 0; t < kXlSeg; ++t) {
-      float2 r = mul2(make_float2(a.bR[0], a.bL[0]), make_float2(d[t], d[20 - t]));
+      for (int t = 0; t < kXlSeg; ++t) {
+        const float s0 = d[t + 2] - d[t + 1], s1 = d[t + 3] - d[t + 2], s2 = d[t + 4] - d[t + 3];
+        D[t] = fmaf(a.f1, s0 + s2, a.f0 * s1);
+      }
 #pragma unroll
-      for (int i = 1; i < 5; ++i)
-        r = fma2(make_float2(a.bR[i], a.bL[i]), make_float2(d[t + i], d[20 - t - i]), r);
-      Y[t] = r;
+      for (int t = 0; t <= kXlSeg; ++t) X[t] = d[t + 2];
+    } else {
+      // X = K_R, D = K_L
+#pragma unroll
+      for (int t = 0; t < kXlSeg; ++t) {
+        float kr = a.bR[0] * d[t], kl = a.bL[0] * d[t + 5];
+#pragma unroll
+        for (int i = 1; i < 5; ++i) {
+          kr = fmaf(a.bR[i], d[t + i], kr);
+          kl = fmaf(a.bL[i], d[t + 5 - i], kl);
+        }
+        X[t] = kr;
+        D[t] = kl;
+      }
     }
-#else
-#pragma unroll
-    for (int t = 0; t < kXlSeg; ++t) {
-      float r = a.bR[0] * d[t];
-#pragma unroll
-      for (int i = 1; i < 5; ++i) r = fmaf(a.bR[i], d[t + i], r);
-      Y[t].x = r;
-    }
-#pragma unroll
-    for (int u = kXlSeg - 1; u >= 0; --u) {
-      float l = a.bL[0] * d[u + 5];
-#pragma unroll
-      for (int i = 1; i < 5; ++i) l = fmaf(a.bL[i], d[u + 5 - i], l);
-      Y[kXlSeg - 1 - u].y = l;
-    }
-#endif
   }
+  const float q = a.q;
   if constexpr (BC == 1) {
-    if (L.s == 0) Y[0].x = 0.f;      // K_R(x_0): the right-moving recurrence starts here
-    if (rs == 0) Y[0].y = 0.f;     // K_L(x_{n-1})
+    if (L.s == 0) X[0] = 0.f;          // the right-moving recurrence starts at x_0
+    if (rs == 0) {                     // the left-moving one at x_{n-1}
+      if (a.d0) X[kXlSeg] = 0.f;
+      else D[kXlSeg - 1] = 0.f;
+    }
   }
-  const float2 q2 = make_float2(a.q, a.q);
-  y = make_float2(0.f, 0.f);
+  if (a.d0) {
 #pragma unroll
-  for (int t = 0; t < kXlSeg; ++t) y = fma2(q2, y, Y[t]);
+    for (int t = 0; t < kXlSeg; ++t) {
+      r = fmaf(q, r, X[t]);
+      l = fmaf(q, l, -X[kXlSeg - t]);
+    }
+  } else {
+#pragma unroll
+    for (int t = 0; t < kXlSeg; ++t) {
+      r = fmaf(q, r, X[t]);
+      l = fmaf(q, l, D[kXlSeg - 1 - t]);
+    }
+  }
   // inclusive scans over the segments: X_s = b[s] + q^16 X_{s-1} (R), mirrored (L)
-  float XR = y.x, XL = y.y;
+  float XR = r, XL = l;
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
     const int dd = 1 << k;
@@ -265,14 +271,52 @@ __device__ __forceinline__ void xl_apply_D(const XLineArgs& a, const XlLane& L, 
       }
     }
   }
-  y = make_float2(cR, cL);
+  if (a.d0) {
 #pragma unroll
-  for (int t = 0; t < kXlSeg; ++t) {
-    y = fma2(q2, y, Y[t]);
-    Y[t] = y;
+    for (int t = 0; t < kXlSeg; ++t) {
+      cR = fmaf(q, cR, X[t]);
+      D[t] = fmaf(a.kap, cR, D[t]);
+    }
+#pragma unroll
+    for (int t = kXlSeg - 1; t >= 0; --t) {
+      cL = fmaf(q, cL, -X[t + 1]);
+      D[t] = fmaf(a.kap, cL, D[t]);
+    }
+  } else {
+#pragma unroll
+    for (int t = 0; t < kXlSeg; ++t) X[t] = cR = fmaf(q, cR, X[t]);
+#pragma unroll
+    for (int t = kXlSeg - 1; t >= 0; --t) {
+      cL = fmaf(q, cL, D[t]);
+      D[t] = X[t] + cL;
+    }
   }
+  if constexpr (BC == 1) {
+    if (a.mode == MODE_0) {   // D_0 vanishes at Dirichlet ends
+      if (L.s == 0) D[0] = 0.f;
+      if (rs == 0) D[kXlSeg - 1] = 0.f;
+    }
+  }
+}
+
+// S_P of the line group in `buf` (P <= 2), written back over it.
+template <int BC, int SF>
+__device__ __forceinline__ void xl_sweep_group(const XLineArgs& a, const XlLane& L, float* buf) {
+  float D[kXlSeg];
+  {
+    float v[kXlSeg];
+    xl_load_own(buf, L.lane, v);
+    xl_apply_D<BC, SF>(a, L, v, D);
+  }
+  if (a.P == 2) {
+    xl_store_own(buf, L.lane, D);       // D of the first power, reread below
+    float D2[kXlSeg];
+    xl_apply_D<BC, SF>(a, L, D, D2);
+    xl_load_own(buf, L.lane, D);
 #pragma unroll
-  for (int t = 0; t < kXlSeg; ++t) D[t] = Y[t].x + Y[kXlSeg - 1 - t].y;
+    for (int t = 0; t < kXlSeg; ++t) D[t] += D2[t];
+  }
+  xl_store_own(buf, L.lane, D);
 }
 
 template <int EPI, int BC, int SF>
@@ -302,23 +346,9 @@ __global__ void __launch_bounds__(kXlWarps * 32, MOLT_XL_MIN_BLOCKS) xline_sweep
     xl_commit();
     xl_wait_ahead();
     __syncwarp();
-    float D[kXlSeg];
-    {
-      float v[kXlSeg];
-      xl_load_own(buf, L.lane, v);
-      xl_apply_D<BC, SF>(a, L, v, D);
-    }
-    if (a.P == 2) {
-      xl_store_own(buf, L.lane, D);       // D of the first power, reread below
-      float D2[kXlSeg];
-      xl_apply_D<BC, SF>(a, L, D, D2);
-      xl_load_own(buf, L.lane, D);
-#pragma unroll
-      for (int t = 0; t < kXlSeg; ++t) D[t] += D2[t];
-    }
+    xl_sweep_group<BC, SF>(a, L, buf);
     // epilogue: through the buffer, so that every global access of the warp
     // is one contiguous 512-byte row
-    xl_store_own(buf, L.lane, D);
     __syncwarp();
     const long long line0 = grp * a.G;
     const long long rem = a.nlines - line0;
@@ -344,6 +374,84 @@ __global__ void __launch_bounds__(kXlWarps * 32, MOLT_XL_MIN_BLOCKS) xline_sweep
     __syncwarp();
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// The FP64 leapfrog update of one wave step and the x sweep of the next in
+// one pass over the rows: u^{n+1} = 2u^n - u^{n-1} + coefS acc (from rest: u^n
+// + coefS/2 acc) with its FP32 copy, then acc = S_x of that copy.  The update
+// alone is bound by HBM (32 B a point) and the x sweep by instructions: the
+// sweep's arithmetic passes under the update's traffic, and the FP32 copy is
+// not read back (512^3: 0.87 ms against 0.69 + 0.28; loads of two or four
+// chunks at once, an L2 prefetch of the next group, two or four CTAs per SM all
+// measured slower).
+struct XWaveArgs {
+  const double* un;
+  const double* us;      // u^{n-1} (unused from rest)
+  double* dst;           // u^{n+1}; may be u^n's or u^{n-1}'s array
+  double* dst2;          // receives u^n, or null
+  float* shadow;         // FP32 copy of u^{n+1}
+  double coefS;
+  int from_rest;
+  int copy_only;         // no update: the FP32 copy of u^n and its x sweep (dst, us, acc unread)
+  int* status;
+};
+
+template <int BC, int SF>
+__global__ void __launch_bounds__(kXlWarps * 32, MOLT_XL_MIN_BLOCKS)
+    xline_wave_kernel(const XLineArgs a, const XWaveArgs w) {
+  __shared__ __align__(128) float xw_smem[kXlWarps][kXlBuf];
+  float* buf = xw_smem[threadIdx.x >> 5];
+  XlLane L;
+  L.lane = threadIdx.x & 31;
+  L.s = (SF == 0 && a.G > 1) ? (L.lane & (a.S - 1)) : L.lane;
+  const long long nw = (long long)gridDim.x * kXlWarps;
+  const double half = 0.5 * w.coefS;
+  bool bad = false;
+  for (long long grp = (long long)blockIdx.x * kXlWarps + (threadIdx.x >> 5); grp < a.ngroups; grp += nw) {
+    const long long line0 = grp * a.G;
+    const long long rem = a.nlines - line0;
+    const int avail = SF ? kXlBuf : int((rem < a.G ? rem : a.G) * a.n);
+    const long long g0 = line0 * a.n;
+#pragma unroll 1
+    for (int c = L.lane; 4 * c < avail; c += 32) {
+      const long long g = g0 + 4 * c;
+      const double2 x0 = *reinterpret_cast<const double2*>(w.un + g), x1 = *reinterpret_cast<const double2*>(w.un + g + 2);
+      double2 r0 = x0, r1 = x1;
+      if (!w.copy_only) {
+        double2 y0 = make_double2(0.0, 0.0), y1 = y0;
+        if (!w.from_rest) {
+          y0 = *reinterpret_cast<const double2*>(w.us + g);
+          y1 = *reinterpret_cast<const double2*>(w.us + g + 2);
+        }
+        const float4 s4 = *reinterpret_cast<const float4*>(a.acc + g);
+        auto upd = [&](double x, double y, float s) {
+          const double wd = f2d(s);
+          const double r = w.from_rest ? fma(half, wd, x) : fma(w.coefS, wd, fma(2.0, x, -y));
+          bad |= nonfinite(r);
+          return r;
+        };
+        r0 = make_double2(upd(x0.x, y0.x, s4.x), upd(x0.y, y0.y, s4.y));
+        r1 = make_double2(upd(x1.x, y1.x, s4.z), upd(x1.y, y1.y, s4.w));
+        if (w.dst2) {
+          *reinterpret_cast<double2*>(w.dst2 + g) = x0;
+          *reinterpret_cast<double2*>(w.dst2 + g + 2) = x1;
+        }
+        *reinterpret_cast<double2*>(w.dst + g) = r0;
+        *reinterpret_cast<double2*>(w.dst + g + 2) = r1;
+      }
+      const float4 f4 = make_float4(d2f(r0.x), d2f(r0.y), d2f(r1.x), d2f(r1.y));
+      *reinterpret_cast<float4*>(w.shadow + g) = f4;
+      *reinterpret_cast<float4*>(buf + xl_chunk(c)) = f4;
+    }
+    __syncwarp();
+    xl_sweep_group<BC, SF>(a, L, buf);
+    __syncwarp();
+#pragma unroll 4
+    for (int c = L.lane; 4 * c < avail; c += 32)
+      *reinterpret_cast<float4*>(a.acc + g0 + 4 * c) = *reinterpret_cast<const float4*>(buf + xl_chunk(c));
+    __syncwarp();
+  }
+  if (bad) atomicOr(w.status, ST_NONFINITE);
 }
 
 }  // namespace molt

@@ -33,7 +33,7 @@ OPT_TMA, OPT_PROFILE, OPT_WAIT_LIMIT, OPT_TEST_SKIP_ARRIVE, OPT_LANES, OPT_AXIS_
 (KERNEL_STORE, KERNEL_ACC_SET, KERNEL_ACC_ADD, KERNEL_HEAT_FINAL, KERNEL_WAVE_FINAL, KERNEL_HJ_X, KERNEL_HJ_Y,
  KERNEL_UPDATE, KERNEL_BATCH, KERNEL_TRANSPOSE, KERNEL_FLUX, KERNEL_LANES_STORE, KERNEL_LANES_ACC_SET,
  KERNEL_LANES_ACC_ADD, KERNEL_LANES_WAVE_FINAL, KERNEL_XLINES_STORE, KERNEL_XLINES_ACC_SET,
- KERNEL_XLINES_ACC_ADD) = range(18)
+ KERNEL_XLINES_ACC_ADD, KERNEL_XLINES_WAVE) = range(19)
 
 
 class molt_desc(ctypes.Structure):
