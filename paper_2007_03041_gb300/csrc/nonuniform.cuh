@@ -307,7 +307,7 @@ __host__ __device__ constexpr int nu_group() { return (WENO ? 8 : 16) / int(size
 // eps = 1e-6 (Sec. 2.4).
 template <typename T>
 __device__ __forceinline__ T nu_wenoz_defect(const T (&w)[kNuWenoSlots], T e0, T e1, T e2, T f) {
-  const T K[3] = {fma(w[1], e2, fma(w[0], e1, e0)), fma(w[3], e1, w[2] * e0), fma(w[5], f, w[4] * e0)};
+  const T K[3] = {fma(w[1], e2, fma(w[0], e1, e0)), fma(w[2], e0, w[3] * e1), fma(w[4], e0, w[5] * f)};
   const T lo[3] = {e2, e1, e0}, hi[3] = {e1, e0, f};
   T beta[3];
 #pragma unroll
@@ -469,7 +469,10 @@ __global__ void __launch_bounds__(512) nonuniform_kernel(const NuArgs a) {
             } else {
               K = T(0);
 #pragma unroll
-              for (int s = 0; s < 5; ++s) K = fma(t[s].v[kk], side == 0 ? d[k + s] : -d[k + 5 - s], K);
+              for (int j = 0; j < 5; ++j) {
+                const int s = j < 2 ? j : (j < 4 ? j + 1 : 2);   // the large tap last: one rounding at its size
+                K = fma(t[s].v[kk], side == 0 ? d[k + s] : -d[k + 5 - s], K);
+              }
             }
             // points past the end, and Dirichlet nodes where a scan starts
             const int e = e0 + k;
