@@ -98,7 +98,6 @@ inline void set_line_constants(SweepArgs& a, const QuadTable& qt, int N, int E, 
   for (int k = 0; k < 13; ++k) a.qpf[k] = float(a.qp[k]);
   a.qlastf = float(a.qlast);
   a.qlwf = float(a.qlw);
-  // one-sided derivatives alpha D: D carries the factor (1-q)/(1-q32)
 }
 
 }  // namespace molt

@@ -318,7 +318,7 @@ __device__ __forceinline__ double weight_rcp(double x) { return 1.0 / x; }
 // The indicators arrive with eps added.
 template <typename T>
 __device__ __forceinline__ T wenoz_defect(T e0, T e1, T e2, T f, T b0, T b1, T b2, const T (&wk)[6], const T (&d)[3]) {
-  const T K[3] = {fma(wk[1], e2, fma(wk[0], e1, e0)), fma(wk[2], e0, wk[3] * e1), fma(wk[4], e0, wk[5] * f)};
+  const T K[3] = {fma(wk[1], e2, fma(wk[0], e1, e0)), fma(wk[3], e1, wk[2] * e0), fma(wk[5], f, wk[4] * e0)};
   const T b[3] = {b0, b1, b2};
   const T tau = fabs(b0 - b2);
   T wt[3], sum = T(0);
@@ -554,7 +554,7 @@ __device__ __forceinline__ void learned_local_integrals(const SweepArgs& a, cons
       // K = sum_r w_r K_r in difference form (wenoz_defect)
       const float f0 = v[3] - v[2], f1 = v[2] - v[1], f2 = v[1] - v[0], f = v[4] - v[3];
       const float K0 = fmaf(wk[1], f2, fmaf(wk[0], f1, f0));
-      const float K1 = fmaf(wk[2], f0, wk[3] * f1), K2 = fmaf(wk[4], f0, wk[5] * f);
+      const float K1 = fmaf(wk[3], f1, wk[2] * f0), K2 = fmaf(wk[5], f, wk[4] * f0);
       jk[phys<E>(e)] = fmaf(w[0], K0, fmaf(w[1], K1, w[2] * K2));
     }
   }
