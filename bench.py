@@ -545,9 +545,8 @@ CONFIGS = {
                                 bytes_per_dof=40, bound="fp64", dtype="f64", fp64_inst_per_dof=45.6,
                                 dram_per_dof=48.0),
     # Sec. 2.5 flux-split advection-diffusion: 2-D viscous Burgers, FP32,
-    # WENO-Z, forward Euler with P = 1; per step and axis: split fluxes (read
-    # u, write g+, g-), three accumulating sweeps (12 B each), plus the memset
-    # of acc and the update (read acc + u, write u)
+    # WENO-Z, forward Euler with P = 1; per step one fused pass per axis (u in,
+    # sums out), y on the transposed state, and the transposing update
     "advdiff_burgers4096": dict(metric="DOF updates/sec (2-D viscous Burgers, 4096^2, flux-split, WENO-Z, FP32) on GB300",
                                 # x axis 8, transpose 8, y axis 8, update (sums of both, state in and out) 16
                                 bytes_per_dof=40, bound="hbm", dtype="f32", flush_l2=True),
