@@ -3,9 +3,12 @@ D_0 with linear weights on both sides of the rule that picks the residual
 form or the K filters (nu about 1.7 for the 6-point rule), one-sided sweeps
 (the L side runs the line mirrored), and lines around the edges of lanes,
 warps and tiles, where the scans' carries change hands."""
+import numpy as np
 import pytest
 
+from oracle import sweep
 from paper_2007_03041_gb300 import molt as M
+from tests.gpu_util import need_gpu, to_dev
 from tests.test_gpu_apply_D import check, run_apply
 
 pytestmark = pytest.mark.gpu
@@ -42,3 +45,33 @@ def test_wenoz_line_edges(prec, bc, op):
     for n in (100, 128, 513, 1024, 2048):
         got, want = run_apply((3, n), 0, op, 1, 2.0 / 3.0, bc, 5, prec, weights=M.W_WENOZ, seed=n)
         check(got, want, prec, 2, 0, n)
+
+
+@pytest.mark.parametrize("npts", [3, 5, 6])
+@pytest.mark.parametrize("n", [500, 512])
+def test_symbol_of_D0_in_fp32(n, npts):
+    """The gain of D_0 on Fourier modes, by projection over many lines of
+    random phase (rounding noise averages out: 5e-9), is that of the exact
+    rule to 2^-25 / (1 - q).  Rounding q to FP32 moves the relative symbol by
+    up to 2^-25 (1 + 2q/(1-q)) between its ends; the other constants, fitted to
+    the rounded q, leave at most half of that and half an ulp of kap.  The
+    nearest FP32 constants leave the whole of it."""
+    need_gpu()
+    import torch
+    lines = 2048
+    phase = np.random.default_rng(n).uniform(0.0, 2 * np.pi, (lines, 1))
+    for nu in (0.2, 0.3, 0.6):
+        bound = 2.0 ** -25 / (-np.expm1(-nu)) + 5e-9
+        for k in (4, 25, 100):
+            u = np.cos(2 * np.pi * k * np.arange(n) / n + phase).astype(np.float32)
+            ctx = M.molt_create(M.make_desc((n, lines), P=1, quad_points=npts, prec=M.PREC_F32))
+            try:
+                uin = to_dev(u, torch.float32)
+                out = torch.empty_like(uin)
+                M.molt_apply_D(ctx, 0, 0, M.OP_0, 1, nu * n, uin, out)
+                got = out.double().cpu().numpy()
+            finally:
+                M.molt_destroy(ctx)
+            want = sweep.partial_sum(u.astype(np.float64), 1, nu * n, 1.0 / n, "0", "periodic", npts, 1, "linear")
+            gain = np.vdot(got, want) / np.vdot(want, want) - 1.0
+            assert abs(gain) <= bound, (nu, k, gain, bound)
