@@ -15,60 +15,56 @@ namespace molt {
 // rounding q by delta shifts the relative symbol by delta (1 + 2q/(1-q)) between
 // its low and its high end: 1.3e-7 at nu = 0.5, a change of the wave speed that
 // a run accumulates.  kap, f0 and f1 are therefore fitted to the q the scans run
-// (least squares of the relative error of g, wavelengths of 2 to 128 points,
-// each octave with the same weight): first kap, rounded to FP32, then f0 and f1
-// against the rounded kap.  Largest relative error of the symbol over those
-// wavelengths, nearest constants / fitted, 6-point rule: nu = 0.1 2.5e-7 /
-// 1.9e-7, 0.3 1.5e-7 / 5.9e-8, 0.53 1.5e-7 / 3.1e-8, 1.0 6.5e-8 / 5.7e-9.
-// p = 1 - q; the 3-point rule keeps f1 = 0 (the kernels skip its taps).
+// (least squares of the relative error of g at wavelengths of 2, 4, .. 128
+// points): first kap, rounded to FP32, then f0 and f1 against the rounded kap.
+// Largest relative error of the symbol, nearest constants / fitted, 6-point
+// rule: nu = 0.1 2.5e-7 / 1.3e-7, 0.3 1.5e-7 / 6.2e-8, 0.6 1.4e-7 / 2.5e-8, 1.0
+// 6.5e-8 / 6.5e-9.  p = 1 - e^{-nu} in full precision; the 3-point rule keeps
+// f1 = 0 (the kernels skip its taps).
 inline void fit_residual_f32(SweepArgs& a, double q, double p, bool has_f1) {
-  constexpr int K = 19;   // three samples an octave
-  const double q32 = double(float(q)), p32 = 1.0 - q32;
-  double col[3][K], r[K], w[K];
-  auto pole = [](double x, double q, double p) { return -(1.0 + q) / (p * p - q * x); };
+  constexpr int K = 7;
+  // x = -4 sin^2(pi / 2^(k+1)): a wavelength of 2^(k+1) points
+  static constexpr double x[K] = {-4.0, -2.0, -5.8578643762690497e-1, -1.5224093497742647e-1, -3.8429439193539104e-2,
+                                  -9.6305466556062275e-3, -2.4090875896552147e-3};
+  const double q32 = double(float(q)), p32 = 1.0 - q32, m = has_f1 ? 1.0 : 0.0;
+  // relative contributions of f0, f1 and kap to g, the first two orthonormalised
+  double A[K], B[K], P[K], r00 = 0.0, r01 = 0.0, r11 = 0.0;
   for (int k = 0; k < K; ++k) {
-    const double s = std::sin(0.5 * M_PI * std::exp2(-double(k) / 3.0)), x = -4.0 * s * s;
-    const double g = a.f0 + a.f1 * (2.0 + x) + a.kap * pole(x, q, p);
-    w[k] = 1.0 / g;
-    col[0][k] = pole(x, q32, p32) * w[k];
-    col[1][k] = w[k];
-    col[2][k] = (2.0 + x) * w[k];
-    r[k] = 1.0;
+    const double w = 1.0 / (a.f0 + a.f1 * (2.0 + x[k]) - a.kap * (1.0 + q) / (p * p - q * x[k]));
+    A[k] = w;
+    B[k] = m * (2.0 + x[k]) * w;
+    P[k] = -w * (1.0 + q32) / (p32 * p32 - q32 * x[k]);
+    r00 += A[k] * A[k];
   }
-  // least squares on the columns first..last by Gram-Schmidt: c minimises |t - sum c col|
-  auto solve = [&](int first, int last, const double* t, double* c) {
-    double Q[3][K], R[3][3] = {}, z[3];
-    for (int i = first; i <= last; ++i) {
-      for (int k = 0; k < K; ++k) Q[i][k] = col[i][k];
-      for (int pass = 0; pass < 2; ++pass)
-        for (int j = first; j < i; ++j) {
-          double d = 0.0;
-          for (int k = 0; k < K; ++k) d += Q[j][k] * Q[i][k];
-          R[j][i] += d;
-          for (int k = 0; k < K; ++k) Q[i][k] -= d * Q[j][k];
-        }
-      double n = 0.0;
-      for (int k = 0; k < K; ++k) n += Q[i][k] * Q[i][k];
-      R[i][i] = std::sqrt(n);
-      z[i] = 0.0;
-      for (int k = 0; k < K; ++k) z[i] += (Q[i][k] /= R[i][i]) * t[k];
-    }
-    for (int i = last; i >= first; --i) {
-      c[i] = z[i];
-      for (int j = i + 1; j <= last; ++j) c[i] -= R[i][j] * c[j];
-      c[i] /= R[i][i];
-    }
-  };
-  const int last = has_f1 ? 2 : 1;
-  double c[3] = {0.0, 0.0, 0.0};
-  solve(0, last, r, c);
-  const float kap = float(c[0]);
-  for (int k = 0; k < K; ++k) r[k] -= double(kap) * col[0][k];
-  solve(1, last, r, c);
-  if (!std::isfinite(kap) || !std::isfinite(c[1]) || !std::isfinite(c[2])) return;
+  r00 = std::sqrt(r00);
+  for (int k = 0; k < K; ++k) r01 += (A[k] /= r00) * B[k];
+  for (int k = 0; k < K; ++k) r11 += (B[k] -= r01 * A[k]) * B[k];
+  r11 = has_f1 ? std::sqrt(r11) : 1.0;
+  for (int k = 0; k < K; ++k) B[k] /= r11;
+  // kap: the pole's part orthogonal to both, against 1
+  double pa = 0.0, pb = 0.0, n = 0.0, z = 0.0;
+  for (int k = 0; k < K; ++k) {
+    pa += A[k] * P[k];
+    pb += B[k] * P[k];
+  }
+  for (int k = 0; k < K; ++k) {
+    const double o = P[k] - pa * A[k] - pb * B[k];
+    n += o * o;
+    z += o;
+  }
+  const float kap = float(z / n);
+  // f0 and f1: what the rounded kap leaves
+  double za = 0.0, zb = 0.0;
+  for (int k = 0; k < K; ++k) {
+    const double left = 1.0 - double(kap) * P[k];
+    za += A[k] * left;
+    zb += B[k] * left;
+  }
+  const double f1 = m * zb / r11, f0 = (za - r01 * f1) / r00;
+  if (!std::isfinite(kap) || !std::isfinite(f0) || !std::isfinite(f1)) return;
   a.kapf = kap;
-  a.f0f = float(c[1]);
-  a.f1f = float(c[2]);
+  a.f0f = float(f0);
+  a.f1f = float(f1);
 }
 
 // Fills the weight and decay fields of `a` for lines of N intervals and E
@@ -87,7 +83,7 @@ inline void fit_residual_f32(SweepArgs& a, double q, double p, bool has_f1) {
 //     and grow like e^{3 nu}; past kResidualMax their cancellation against
 //     kap (U + V) would show in the last digits, and the K filters run.
 constexpr double kResidualMax = 0.125;
-inline void set_line_constants(SweepArgs& a, const QuadTable& qt, int N, int E, bool f32_sweeps) {
+inline void set_line_constants(SweepArgs& a, const QuadTable& qt, int N, int E, bool f32_sweeps, bool linear = true) {
   const double nu = qt.nu, qx = qt.q;
   const double* c = qt.c;
   // difference taps
@@ -155,7 +151,7 @@ inline void set_line_constants(SweepArgs& a, const QuadTable& qt, int N, int E, 
   a.f0f = float(a.f0);
   a.f1f = float(a.f1);
   a.kapf = float(a.kap);
-  if (f32_sweeps && a.d0 && a.mode == MODE_0) fit_residual_f32(a, qx, p, a.f1 != 0.0);
+  if (f32_sweeps && linear && a.d0 && a.mode == MODE_0) fit_residual_f32(a, qx, p, a.f1 != 0.0);
   for (int i = 0; i < 6; ++i) a.wkf[i] = float(a.wk[i]);
   for (int r = 0; r < 3; ++r) a.df[r] = float(a.d[r]);
   for (int k = 0; k < 13; ++k) a.qpf[k] = float(a.qp[k]);

@@ -319,7 +319,7 @@ molt_status plan_axis(molt_ctx* c, const Problem& p, int ax, int mode, int P, do
   QuadTable qt;
   if (!build_quadrature(p.d.quad_points, nu, &qt)) return fail(c, MOLT_EINVAL, "quadrature table construction failed");
   const int N = a.bc == MOLT_BC_PERIODIC ? n : n - 1;  // intervals
-  set_line_constants(a, qt, N, E, compute_bytes(p.d) == 4);
+  set_line_constants(a, qt, N, E, compute_bytes(p.d) == 4, p.d.weights == MOLT_W_LINEAR);
   if (mode == MODE_RL) {
     a.ham = p.d.hamiltonian;
     a.vel = p.d.velocity[ax];
