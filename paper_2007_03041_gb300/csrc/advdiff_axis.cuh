@@ -31,10 +31,10 @@ __global__ void __maxnreg__(128) advdiff_axis_kernel(const AdvArgs A) {
   const LineLane<T, false, RAGGED, E> ln(a, sm);
   load_tile<T, T, E>(a, static_cast<const T*>(a.in), static_cast<T*>(sm.lines), line0, ln.lw,
                      ln.part * 32 + ln.lane, [](T* d, const T* g) { *d = *g; });
-  if (a.contiguous) line_sync(ln.nwl, ln.lw); else __syncthreads();
+  if (a.contiguous) line_sync<T, E>(ln.nwl, ln.lw); else __syncthreads();
   if constexpr (RAGGED) {
     if (ln.part == 0) warp_fill_ghosts<T, E>(a, ln.buf, ln.lane);
-    line_sync(ln.nwl, ln.lw);
+    line_sync<T, E>(ln.nwl, ln.lw);
   }
   T S[E], X[E + 1], F[E];
   {
@@ -68,7 +68,7 @@ __global__ void __maxnreg__(128) advdiff_axis_kernel(const AdvArgs A) {
     for (int k = 0; k < E; ++k) S[k] = fma(T(A.cL), F[k], T(A.cR) * X[k]);
   }
   if (A.diffusive) {
-    line_sync(ln.nwl, ln.lw);   // the totals are reused
+    line_sync<T, E>(ln.nwl, ln.lw);   // the totals are reused
     T win[E + 6], dd[E + 5];
     load_window<T, false, RAGGED, E>(ln, win);
 #pragma unroll
@@ -82,7 +82,7 @@ __global__ void __maxnreg__(128) advdiff_axis_kernel(const AdvArgs A) {
   // (every lane of the line read its window before the last scan's barrier)
   if (ln.own) __syncwarp();
   ln.store(S);
-  if (a.contiguous) line_sync(ln.nwl, ln.lw); else __syncthreads();
+  if (a.contiguous) line_sync<T, E>(ln.nwl, ln.lw); else __syncthreads();
   epilogue_tile<T, T, EPI, E>(a, static_cast<const T*>(sm.lines), line0, 0.0);
 }
 

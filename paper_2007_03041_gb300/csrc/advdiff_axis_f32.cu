@@ -1,4 +1,5 @@
 // The fused advection-diffusion axis kernel (csrc/advdiff_axis.cuh), FP32.
+#define MOLT_LINE_BARRIERS 1
 #include "advdiff_axis_launch.h"
 
 namespace molt {

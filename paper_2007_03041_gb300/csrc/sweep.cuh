@@ -353,11 +353,41 @@ struct Indicators {
 };
 
 // -------------------------------------------------------------- tile staging
-// Barrier of the warps that share line lw of a tile (named barrier 1 + lw;
-// tiles of several warps per line hold at most 8 lines).
+// Barrier of the warps that share line lw of a tile.  A barrier number held in
+// a register reserves all 16 barriers for the CTA, and an SM, with 64, then
+// takes no more than four CTAs of any size: the y lines of a 512^2 FP32 wave,
+// 512 CTAs of one warp, took 28.8 us a sweep, some SMs busy for 51 thousand
+// cycles and some for 30.  The sweep kernels therefore take the CTA's own
+// barrier (5 such steps 224 -> 191 us; 201 x 151 x 101 mixed wave, 5 steps, 685 ->
+// 653 us; 4096^2 WENO-Z, 4 steps, 1293 -> 1277 us), FP64 tiles of 16 points a
+// lane constant numbers 1 to 4, more than four lines of several warps sharing
+// one with their neighbours (5277^2 diffusion, 2 steps, register / CTA / constant
+// numbers 3890 / 3919 / 3824 us; the FP32 wave above 685 / 653 / 706 us).
+// Translation units that measured faster with a barrier a line define
+// MOLT_LINE_BARRIERS 1 and keep the register: the batched kernel (two CTAs of
+// 512 threads per SM in any case; 10.4 ms against 11.1 with the CTA's barrier)
+// and the advection-diffusion axis kernel (1500^2 FP32 WENO-Z, 2 steps, 194 us
+// against 203).
+#ifndef MOLT_LINE_BARRIERS
+#define MOLT_LINE_BARRIERS 0
+#endif
+template <typename T, int E>
 __device__ __forceinline__ void line_sync(int nwl, int lw) {
-  if (nwl == 1) __syncwarp();
-  else asm volatile("bar.sync %0, %1;" ::"r"(1 + lw), "r"(32 * nwl) : "memory");
+  if (nwl == 1) {
+    __syncwarp();
+  } else if constexpr (MOLT_LINE_BARRIERS) {
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + lw), "r"(32 * nwl) : "memory");
+  } else if constexpr (sizeof(T) == 8 && E == 16) {
+    const int share = blockDim.x > 128 * nwl ? 1 : 0, count = (32 * nwl) << share;
+    switch (lw >> share) {
+      case 0: asm volatile("bar.sync 1, %0;" ::"r"(count) : "memory"); break;
+      case 1: asm volatile("bar.sync 2, %0;" ::"r"(count) : "memory"); break;
+      case 2: asm volatile("bar.sync 3, %0;" ::"r"(count) : "memory"); break;
+      default: asm volatile("bar.sync 4, %0;" ::"r"(count) : "memory"); break;
+    }
+  } else {
+    __syncthreads();
+  }
 }
 
 // Contiguous lines: the nwl warps of line lw read it with consecutive lanes.
@@ -826,7 +856,7 @@ __device__ __forceinline__ void line_scans(const LineConst& L, const LineLane<T,
     T* tot = ln.totals + ln.lw * ln.nwl * 2;
     if (ln.lane == ln.lastR) tot[2 * ln.part] = endR;
     if (!ONE && ln.lane == 0) tot[2 * ln.part + 1] = bL;
-    line_sync(ln.nwl, ln.lw);
+    line_sync<T, E>(ln.nwl, ln.lw);
     const int j = ln.lane & 15;
     const bool left = ln.lane >= 16;
     T x = T(0);
@@ -959,7 +989,7 @@ __device__ __forceinline__ double compute_lines(const SweepArgs& a, const TileSm
     T X[E + 1], F[E];
     if constexpr (JQ == JQ_LEARNED || RAGGED) {
       if (ln.part == 0) warp_fill_ghosts<T, E>(a, ln.buf, ln.lane);
-      line_sync(ln.nwl, ln.lw);
+      line_sync<T, E>(ln.nwl, ln.lw);
     }
     if constexpr (JQ == JQ_LEARNED) {
       float* jrl = sm.jloc + ln.lw * 2 * a.LS;
@@ -1038,7 +1068,7 @@ __device__ __forceinline__ double compute_lines(const SweepArgs& a, const TileSm
         // warps, before the totals' barrier
         if (ln.own) __syncwarp();
         ln.store(F);
-        line_sync(ln.nwl, ln.lw);
+        line_sync<T, E>(ln.nwl, ln.lw);
       }
     }
   }
@@ -1046,7 +1076,7 @@ __device__ __forceinline__ double compute_lines(const SweepArgs& a, const TileSm
   if (ln.own) __syncwarp();
   ln.store(S);
   // the epilogue reads contiguous lines by their ln.own warps, strided ones by rows
-  if (a.contiguous) line_sync(ln.nwl, ln.lw); else __syncthreads();
+  if (a.contiguous) line_sync<T, E>(ln.nwl, ln.lw); else __syncthreads();
   return cvt<double>(rmax);
 }
 
@@ -1307,7 +1337,7 @@ __global__ void __maxnreg__((sweep_regs<T, JQ, E>())) sweep_kernel(const SweepAr
   const int tl = (warp - lw * a.nwl) * 32 + (threadIdx.x & 31);
   load_tile<T, TIN, E>(a, static_cast<const TIN*>(a.in), lines, line0, lw, tl,
                        [](T* d, const TIN* g) { *d = cvt<T>(*g); });
-  if (a.contiguous && JQ != JQ_LEARNED) line_sync(a.nwl, lw); else __syncthreads();
+  if (a.contiguous && JQ != JQ_LEARNED) line_sync<T, E>(a.nwl, lw); else __syncthreads();
   if constexpr (epi_hj_x(EPI) || epi_hj_y(EPI)) {
     const double rmax =
         compute_lines<T, JQ, RAGGED, E, epi_hj_gen(EPI)>(a, sm, line0 + lw < a.g.nlines) * a.inv_h;
