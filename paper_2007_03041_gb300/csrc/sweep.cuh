@@ -44,6 +44,9 @@ constexpr int kG = 16;   // ghost slots per side in shared memory (3 used)
 #define MOLT_MAX_THREADS 512
 #endif
 constexpr int kMaxThreads = MOLT_MAX_THREADS;
+static_assert(kMaxThreads <= 512,
+              "16 warps a line at most: their totals are scanned by half a warp, q^(points before a warp) has four bits, "
+              "and lines of several warps have at most eight barriers");
 // Shared memory per CTA (the GPU allows 227 KB): a sweep tile's budget, and the
 // dynamic size the sweep kernels opt into (a TMA tile plus its staging buffer
 // must fit it).
