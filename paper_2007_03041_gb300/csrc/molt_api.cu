@@ -1830,10 +1830,9 @@ molt_status wave_step(molt_ctx* c, Problem& p, void* cur, void* prev, bool from_
     }
     if ((st = run(c, p, epi, pl)) != MOLT_OK) return st;
     if (last && split_update && next_x) {
-      const XWaveArgs w{static_cast<const double*>(cur), static_cast<const double*>(prev),
-                        static_cast<double*>(in_place_variant ? cur : prev),
-                        in_place_variant ? static_cast<double*>(prev) : nullptr, p.shadow, -p.d.beta * p.d.beta,
-                        from_rest ? 1 : 0, 0, c->status_dev};
+      // (never the last step of a call, so never the in-place variant)
+      const XWaveArgs w{static_cast<const double*>(cur), static_cast<const double*>(prev), static_cast<double*>(prev),
+                        p.shadow, -p.d.beta * p.d.beta, from_rest ? 1 : 0, 0, c->status_dev};
       molt_ctx::Rec rec;
       record_begin(c, &rec, MOLT_KERNEL_XLINES_WAVE);
       const cudaError_t e = launch_xlines_wave(*next_x, w, c->stream);

@@ -387,8 +387,7 @@ __global__ void __launch_bounds__(kXlWarps * 32, MOLT_XL_MIN_BLOCKS) xline_sweep
 struct XWaveArgs {
   const double* un;
   const double* us;      // u^{n-1} (unused from rest)
-  double* dst;           // u^{n+1}; may be u^n's or u^{n-1}'s array
-  double* dst2;          // receives u^n, or null
+  double* dst;           // u^{n+1}, in u^{n-1}'s array
   float* shadow;         // FP32 copy of u^{n+1}
   double coefS;
   int from_rest;
@@ -432,10 +431,6 @@ __global__ void __launch_bounds__(kXlWarps * 32, MOLT_XL_MIN_BLOCKS)
         };
         r0 = make_double2(upd(x0.x, y0.x, s4.x), upd(x0.y, y0.y, s4.y));
         r1 = make_double2(upd(x1.x, y1.x, s4.z), upd(x1.y, y1.y, s4.w));
-        if (w.dst2) {
-          *reinterpret_cast<double2*>(w.dst2 + g) = x0;
-          *reinterpret_cast<double2*>(w.dst2 + g + 2) = x1;
-        }
         *reinterpret_cast<double2*>(w.dst + g) = r0;
         *reinterpret_cast<double2*>(w.dst + g + 2) = r1;
       }
