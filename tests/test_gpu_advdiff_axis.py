@@ -1,11 +1,16 @@
 """The fused advection-diffusion axis kernel against the oracle at the edges
-of its shapes: lines around lane, warp and tile ends (exact-fit lines of 512,
-1024 points; masked ones of 4, 8 and 16 points a lane), one to three axes,
-no diffusion, both integrators, and y lines long enough to run on the
-transposed state (rows of a tile under 32 bytes)."""
+of its shapes: lines around lane, warp and tile ends, one to three axes, no
+diffusion, both integrators.  In 2-D the y axis runs on the transposed state
+where a tile's rows would be under 32 bytes (few lines or long ones: every 2-D
+case of CASES), else in place on column tiles (ROUTES, which also run the
+unmasked kernel of 16 points a lane in both precisions)."""
+import numpy as np
 import pytest
 
+from oracle import schemes
 from paper_2007_03041_gb300 import molt as M
+from tests.gpu_util import assert_grid_parity, need_gpu, state_dtype, to_dev, tol_for
+from tests.test_gpu_advdiff import _field
 from tests.test_gpu_advdiff import test_advdiff_steps_match_oracle as run_case
 
 pytestmark = pytest.mark.gpu
@@ -33,3 +38,55 @@ CASES = [
 @pytest.mark.parametrize("case", CASES, ids=["x".join(map(str, c[0])) for c in CASES])
 def test_fused_axis_edges(case):
     run_case(case)
+
+
+# numpy shape, prec, weights, npts, whether y runs on the transposed state
+ROUTES = [
+    ((70, 2600), F32, WZ, 5, False),       # column tiles, 4 points a lane, masked
+    ((300, 2600), F32, LIN, 6, False),     # 16 points a lane, masked
+    ((512, 2600), F32, WZ, 5, False),      # 16 points a lane, exact
+    ((512, 2600), F32, LIN, 6, False),
+    ((1024, 2440), F32, WZ, 5, False),     # two warps a line
+    ((64, 1300), F64, WZ, 5, False),
+    ((1024, 1300), F64, WZ, 5, False),     # exact, two warps a line
+    ((1024, 1300), F64, LIN, 6, False),
+    ((1300, 1024), F64, WZ, 5, True),      # x exact, y transposed
+    ((128, 128), F32, WZ, 5, True),        # short lines, but few of them
+    ((11, 20, 35), F32, WZ, 5, None),      # 3-D: column tiles along y and z
+    ((10, 33, 18), F64, WZ, 5, None),
+    ((9, 64, 128), F64, LIN, 6, None),
+]
+
+
+@pytest.mark.parametrize("case", ROUTES, ids=["x".join(map(str, c[0])) + "-%d-%d" % c[1:3] for c in ROUTES])
+def test_fused_axis_routes(case):
+    need_gpu()
+    shape, prec, weights, npts, transposed = case
+    nd = len(shape)
+    vel = (0.7, -0.4, 0.25)[:nd]
+    hs = [2 * np.pi / n for n in shape]
+    c, kappa, beta = 1.6, 0.01, 0.6
+    dt = 0.5 * min(hs) / c
+    u0 = _field(shape, 60 + nd)
+    if prec == F32:
+        u0 = u0.astype(np.float32).astype(np.float64)
+    d = M.make_desc(tuple(reversed(shape)), lo=[0.0] * nd, hi=[2 * np.pi] * nd, P=1, quad_points=npts, weights=weights,
+                    beta=beta, pde=M.PDE_ADVDIFF, c=c, diffusivity=kappa, dt=dt, prec=prec, velocity=vel, flux=B,
+                    integrator=M.INT_EULER)
+    ctx = M.molt_create(d)
+    try:
+        M.molt_set_option(ctx, M.OPT_PROFILE, 1)
+        u = to_dev(u0, state_dtype(prec))
+        M.molt_step(ctx, u, None, nsteps=2, t=[0.0])
+        got = u.double().cpu().numpy()
+        axes = M.molt_profile_read(ctx, M.KERNEL_ACC_ADD)[1]
+        turns = M.molt_profile_read(ctx, M.KERNEL_TRANSPOSE)[1]
+        flux = M.molt_profile_read(ctx, M.KERNEL_FLUX)[1]
+    finally:
+        M.molt_destroy(ctx)
+    assert (axes, turns, flux) == (2 * nd, 2 if transposed else 0, 0)
+    want = u0
+    for _ in range(2):
+        want = schemes.advdiff_step(want, hs, dt, schemes.FLUX_BURGERS, vel[::-1], c, kappa, beta, npts, 1, False,
+                                    "wenoz" if weights == WZ else "linear")
+    assert_grid_parity(got, want, tol_for(prec), what=str(case))
