@@ -1553,28 +1553,28 @@ __global__ void advdiff_update_kernel(const TC* __restrict__ acc, const TS* un, 
 
 // The last axis's sums on the transposed grid (st, x-major) with the update:
 // dst = a0 u^n + a1 (u_s + (acc + st^T)), through 64 x 64 tiles.
-template <typename T>
-__global__ void advdiff_update_t_kernel(const T* __restrict__ acc, const T* __restrict__ st, const T* un, const T* us,
-                                        T* dst, double a0, double a1, long long ny, long long nx, int* status) {
-  __shared__ T tile[64][65];
+__global__ void advdiff_update_t_kernel(const float* __restrict__ acc, const float* __restrict__ st, const float* un,
+                                        const float* us, float* dst, double a0, double a1, long long ny,
+                                        long long nx, int* status) {
+  __shared__ float tile[64][65];
   const long long x0 = (long long)blockIdx.x * 64, y0 = (long long)blockIdx.y * 64;
-  T v[16];
+  float v[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
     const long long x = x0 + threadIdx.y + 8 * (k >> 1), y = y0 + threadIdx.x + 32 * (k & 1);
-    v[k] = (x < nx && y < ny) ? st[x * ny + y] : T(0);
+    v[k] = (x < nx && y < ny) ? st[x * ny + y] : 0.f;
   }
 #pragma unroll
   for (int k = 0; k < 16; ++k) tile[threadIdx.y + 8 * (k >> 1)][threadIdx.x + 32 * (k & 1)] = v[k];
   __syncthreads();
-  T w[16], z[16];
+  float w[16], z[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
     const int j = threadIdx.y + 8 * (k >> 1), i = threadIdx.x + 32 * (k & 1);
     const long long x = x0 + i, y = y0 + j;
     if (x < nx && y < ny) {
       v[k] = acc[y * nx + x] + tile[i][j];
-      w[k] = a0 != 0.0 ? un[y * nx + x] : T(0);
+      w[k] = a0 != 0.0 ? un[y * nx + x] : 0.f;
       z[k] = us[y * nx + x];
     }
   }
@@ -1583,12 +1583,29 @@ __global__ void advdiff_update_t_kernel(const T* __restrict__ acc, const T* __re
   for (int k = 0; k < 16; ++k) {
     const long long x = x0 + threadIdx.x + 32 * (k & 1), y = y0 + threadIdx.y + 8 * (k >> 1);
     if (x < nx && y < ny) {
-      const T r = fma(T(a0), w[k], T(a1) * (z[k] + v[k]));
+      const float r = fmaf(float(a0), w[k], float(a1) * (z[k] + v[k]));
       dst[y * nx + x] = r;
       bad |= nonfinite(r);
     }
   }
   if (bad) atomicOr(status, ST_NONFINITE);
+}
+
+// Whether the y axis of a 2-D stage runs on the transposed state (two more
+// launches): FP32, over 2^18 points, and column tiles (W lines) whose rows fill
+// less than half of a 32-byte sector, or less than one where y lines have 2048
+// points or more.  Euler steps, WENO-Z / linear weights, us in place against
+// transposed (nx x ny): 128^2 16.9/16.7 25.4/25.3, 64 x 2048 27/22 31/28, 512^2
+// 33.2/26.1 33.7/29.5; over 2^18 points with rows of 4 and 8 bytes 600 x 1024
+// 44.0/40.1 38.1/31.5, 700^2 35.9/30.8 37.9/33.6, 1024^2 44.6/37.5 41.8/33.7,
+// 64 x 8192 58/51 45/38, 4096^2 508/412 408/317; with rows of 16 bytes 1500 x
+// 1024 50.0/38.9 61.3/49.7, 2000 x 1100 80/60 85/66, 2048^2 111/83 104/80.  FP64,
+// bound by its pipe: 128^2 83/36 95/48, 1024^2 1035/230 1046/240, 4096^2
+// 14114/3049 13935/3065.
+bool transposed_y(const Problem& p, int W) {
+  const int row = W * int(state_bytes(p.d));
+  return !is_f64_sweep(p.d) && p.total > (1LL << 18) &&
+         (row < kStridedRowBytes / 2 || (row < kStridedRowBytes && p.n[1] >= 2048));
 }
 
 // The fused axis kernel takes stages with one term per sum on uniform axes
@@ -1642,10 +1659,9 @@ molt_status advdiff_stage_fused(molt_ctx* c, Problem& p, const void* un, const v
   for (int ax = 0; ax < p.d.ndim; ++ax) {
     const bool last = ax + 1 == p.d.ndim;
     if (last && p.d.ndim == 2) {
-      // long y lines: a tile's rows of them would not fill a 32-byte sector
       Plan pl;
       if ((st = plan_axis(c, p, ax, MODE_R, 1, beta / (cb * dt), &pl)) != MOLT_OK) return st;
-      if (size_t(pl.a.W) * el < 32) {
+      if (transposed_y(p, pl.a.W)) {
         const long long nx = p.n[0], ny = p.n[1];
         const Problem pt = transposed(p);
         if ((st = transpose(c, p, us, p.gp, ny, nx, el)) != MOLT_OK) return st;
@@ -1653,14 +1669,9 @@ molt_status advdiff_stage_fused(molt_ctx* c, Problem& p, const void* un, const v
         molt_ctx::Rec rec;
         record_begin(c, &rec, MOLT_KERNEL_UPDATE);
         const dim3 grid(unsigned((nx + 63) / 64), unsigned((ny + 63) / 64)), block(32, 8);
-        if (f64)
-          advdiff_update_t_kernel<double><<<grid, block, 0, c->stream>>>(
-              static_cast<const double*>(p.acc), static_cast<const double*>(p.gm), static_cast<const double*>(un),
-              static_cast<const double*>(us), static_cast<double*>(dst), a0, a1, ny, nx, c->status_dev);
-        else
-          advdiff_update_t_kernel<float><<<grid, block, 0, c->stream>>>(
-              static_cast<const float*>(p.acc), static_cast<const float*>(p.gm), static_cast<const float*>(un),
-              static_cast<const float*>(us), static_cast<float*>(dst), a0, a1, ny, nx, c->status_dev);
+        advdiff_update_t_kernel<<<grid, block, 0, c->stream>>>(
+            static_cast<const float*>(p.acc), static_cast<const float*>(p.gm), static_cast<const float*>(un),
+            static_cast<const float*>(us), static_cast<float*>(dst), a0, a1, ny, nx, c->status_dev);
         record_end(c, &rec);
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "advection-diffusion update");
         continue;

@@ -1,9 +1,9 @@
 """The fused advection-diffusion axis kernel against the oracle at the edges
 of its shapes: lines around lane, warp and tile ends, one to three axes, no
-diffusion, both integrators.  In 2-D the y axis runs on the transposed state
-where a tile's rows would be under 32 bytes (few lines or long ones: every 2-D
-case of CASES), else in place on column tiles (ROUTES, which also run the
-unmasked kernel of 16 points a lane in both precisions)."""
+diffusion, both integrators.  In 2-D the y axis runs on column tiles in place,
+that of larger FP32 grids whose tiles have narrow rows on the transposed state:
+ROUTES has both sides of that rule, and the unmasked kernel of 16 points a lane
+in both precisions."""
 import numpy as np
 import pytest
 
@@ -50,8 +50,14 @@ ROUTES = [
     ((64, 1300), F64, WZ, 5, False),
     ((1024, 1300), F64, WZ, 5, False),     # exact, two warps a line
     ((1024, 1300), F64, LIN, 6, False),
-    ((1300, 1024), F64, WZ, 5, True),      # x exact, y transposed
-    ((128, 128), F32, WZ, 5, True),        # short lines, but few of them
+    ((1300, 1024), F64, WZ, 5, False),     # x exact
+    ((128, 128), F32, WZ, 5, False),       # rows of 4 bytes, small
+    ((512, 512), F32, WZ, 5, False),       # rows of 4 bytes, 2^18 points
+    ((512, 515), F32, WZ, 5, True),        # just over
+    ((1024, 700), F32, LIN, 6, True),      # rows of 8 bytes; the transposed lines exact
+    ((1024, 1500), F32, WZ, 5, False),     # rows of 16 bytes
+    ((2048, 1500), F32, LIN, 6, True),     # the same, long lines
+    ((8192, 129), F32, WZ, 5, True),       # the longest lines
     ((11, 20, 35), F32, WZ, 5, None),      # 3-D: column tiles along y and z
     ((10, 33, 18), F64, WZ, 5, None),
     ((9, 64, 128), F64, LIN, 6, None),
