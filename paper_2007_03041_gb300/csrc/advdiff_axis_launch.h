@@ -8,9 +8,13 @@ namespace molt {
 
 template <typename T, bool WENO, int EPI, bool RAGGED, int E>
 cudaError_t launch_advdiff_kernel(const AdvArgs& A, int grid, int block, size_t smem, cudaStream_t s) {
-  const cudaError_t e = cudaFuncSetAttribute(&advdiff_axis_kernel<T, WENO, EPI, RAGGED, E>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemTileBudget));
-  if (e != cudaSuccess) return e;
+  static bool configured = false;
+  if (!configured) {
+    const cudaError_t e = cudaFuncSetAttribute(&advdiff_axis_kernel<T, WENO, EPI, RAGGED, E>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemTileBudget));
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
   advdiff_axis_kernel<T, WENO, EPI, RAGGED, E><<<grid, block, smem, s>>>(A);
   return cudaGetLastError();
 }
