@@ -61,8 +61,12 @@ typedef enum { MOLT_BC_PERIODIC = 0, MOLT_BC_DIRICHLET = 1 } molt_bc;
 typedef enum { MOLT_OP_L = 0, MOLT_OP_R = 1, MOLT_OP_0 = 2 } molt_op;
 typedef enum {
   MOLT_PREC_F64 = 0,            /* FP64 state, FP64 sweeps                         */
-  MOLT_PREC_F32_F64UPDATE = 1,  /* FP64 state, FP32 sweeps, FP64 A/B and update    */
-  MOLT_PREC_F32 = 2             /* FP32 state and sweeps, FP64 A/B                 */
+  MOLT_PREC_F32_F64UPDATE = 1,  /* FP64 state, FP32 sweeps, FP64 update            */
+  MOLT_PREC_F32 = 2             /* FP32 state and sweeps                           */
+  /* FP32 sweeps: the factors of the boundary constants A and B come in FP64 from
+   * the host; their products with the line totals run in FP64 (x lines and
+   * 32-line tiles of 16..512 points with the linear rule) or in pairs of FP32
+   * numbers (48 bits; all other lines), and enter the FP32 scan rounded once.  */
 } molt_prec;
 typedef enum { MOLT_PDE_HEAT = 0, MOLT_PDE_WAVE = 1, MOLT_PDE_HJ = 2, MOLT_PDE_ADVDIFF = 3 } molt_pde;
 /* Flux of the advection-diffusion problem u_t + sum_d d_d g_d(u) = kappa Lap u

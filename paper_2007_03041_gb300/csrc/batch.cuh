@@ -8,8 +8,9 @@
 // own tile shape (points per lane E, warps per line, lines per tile), chosen
 // per size class by the host-side autotuner.  Every wait is bounded: a grid
 // barrier that does not complete within the wait limit records ST_TIMEOUT and
-// the kernel returns.  Data written earlier in the same launch is read through
-// L2 only.
+// the kernel returns.  Data written earlier in the same launch is read after a
+// grid barrier, whose fences order it: the update and the accumulators through
+// L2, the sweeps' lines by cp.async (through L1, which the fences invalidate).
 #pragma once
 
 #include "sweep.cuh"
@@ -149,8 +150,9 @@ __device__ __forceinline__ int find_problem(const BatchParams& p, long long item
 }
 
 // Compiled for two CTAs per SM (64 registers; more spills than at 128, but
-// the second resident CTA covers the phases' memory latency: 64 problems,
-// 7.09 -> 6.81 ms per RK3 step).
+// the second resident CTA covers the phases' memory latency: 64 problems, two
+// steps, 1 / 2 / 3 CTAs per SM 14.1 / 11.4 / 15.0 ms, before the update's
+// smaller chunks; 10.4 ms now).
 #ifndef MOLT_BATCH_MIN_BLOCKS
 #define MOLT_BATCH_MIN_BLOCKS 2
 #endif

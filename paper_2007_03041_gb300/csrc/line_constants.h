@@ -73,16 +73,19 @@ inline void fit_residual_f32(SweepArgs& a, double q, double p, bool has_f1) {
 // are those of that ratio, so that the periodic image sum and the Dirichlet
 // solve close the recurrences the kernel actually runs.  Every form takes
 // differences of v, so D of a constant is exactly zero at any rounding.
-//   b[]     K_R(x_i) = sum_m b_m d_{i+m}, m = -2..2 (weights summing to 1 - q)
+//   b[]     K_R(x_i) = sum_m b_m d_{i+m}, m = -2..2 (the weights of J sum to
+//     1 - q, the taps on its differences to (1 - q) / nu)
 //   f0, f1, kap   the residual form of D_0: with N(z) = (1-q/z)(1-qz) -
 //     [J(z)(1-qz) + J(1/z)(1-q/z)]/2 = delta^2 (a0 + a1 (z+1/z) + a2 (z^2+1/z^2))
 //     and x = delta^2 = z - 2 + 1/z, M(x) = M0 + M1 x + M2 x^2 is divided by
 //     (1-q)^2 - q x: M = (Q0 + Q1 x)((1-q)^2 - q x) + rho, and
 //     U + V = -(1+q) delta^2 v / ((1-q)^2 - q x) gives kap = -rho/(1+q),
-//     f0 = Q0 - 2 Q1, f1 = Q1.  Q0 and Q1 are small (below 0.03 up to nu = 1.2)
-//     and grow like e^{3 nu}; past kResidualMax their cancellation against
-//     kap (U + V) would show in the last digits, and the K filters run.
+//     f0 = Q0 - 2 Q1, f1 = Q1.  Q0 and Q1 are below 0.03 up to nu = 1.2; those of
+//     the 5- and 6-point rules grow like e^{3 nu}, and past kResidualMax (nu = 1.66
+//     and 2.08), where their cancellation against kap (U + V) would show in the
+//     last digits, the K filters run.  The 3-point rule's stay below 0.04.
 constexpr double kResidualMax = 0.125;
+// linear: the sweep reads the FP32 residual form (not with WENO-Z weights).
 inline void set_line_constants(SweepArgs& a, const QuadTable& qt, int N, int E, bool f32_sweeps, bool linear = true) {
   const double nu = qt.nu, qx = qt.q;
   const double* c = qt.c;

@@ -106,8 +106,9 @@ int phys_len(int e) {
   return ee + (ee >> 4);
 }
 
-// Kernel arguments of the sum_{p<=P} D_0^p sweep along `ax` (same tile rules
-// as molt_step's planner).  Returns false if the line does not fit.
+// Kernel arguments of the sum_{p<=P} D_0^p sweep along `ax`, in tiles of 16
+// points a lane and up to 512 threads (molt_step's planner also takes 8 and 4
+// points a lane and smaller tiles).  Returns false if the line does not fit.
 bool plan(const molt_desc& d, int ax, double alpha, int* status, SweepArgs* a, int* grid, int* block,
           size_t* smem) {
   std::memset(a, 0, sizeof(*a));

@@ -1,5 +1,5 @@
 // FP32 sweeps on FP64 state: the sweeps read the FP32 copy of the state, the
-// boundary solve and the state update run in FP64.
+// state update runs in FP64, the boundary constants in pairs of FP32 numbers.
 #include "sweep_launch.h"
 
 namespace molt {

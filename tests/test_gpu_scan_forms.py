@@ -1,6 +1,7 @@
 """The scan kernel's forms of D against the oracle, where they can go wrong:
 D_0 with linear weights on both sides of the rule that picks the residual
-form or the K filters (nu about 1.7 for the 6-point rule), one-sided sweeps
+form or the K filters (nu = 1.66 for the 5-point rule, 2.08 for the 6-point
+one; the 3-point rule stays with the residual form), one-sided sweeps
 (the L side runs the line mirrored), and lines around the edges of lanes,
 warps and tiles, where the scans' carries change hands."""
 import numpy as np
