@@ -60,8 +60,10 @@ WORKLOAD = {
 BYTES_PER_DOF = {"x": 8, "yz": 12, "last_update": 36, "update": 32, "update_x": 36}
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per DOF per launch
 # from one ncu capture of each kernel on the 512^3 step itself (one-pass
-# metrics); a kernel changed since its capture has no entry
+# metrics; xline_wave_kernel: on 512 x 512 x 128); a kernel changed since its
+# capture has no entry
 TRAFFIC_PER_DOF = {"wave_update_kernel (FP64 leapfrog update)": 31.65,
+                   "xline_wave_kernel (FP64 leapfrog update + next step's x sweep)": 34.3,
                    "lanes_sweep_kernel ACC_ADD (y lines)": 11.61}
 
 
@@ -522,9 +524,9 @@ def run_ours(args):
 # the measured form over it, the relative L2 difference of the final states).
 CONFIGS = {
     # heat 256^2: FP64 thread-instructions per DOF and step from one ncu
-    # capture (6 sweeps x 77.3 + 3 stage updates x 4.0); the state stays in L2
+    # capture (6 sweeps x 38.5 + 3 stage updates x 4.0); the state stays in L2
     "heat256": dict(metric="DOF updates/sec (2-D heat, 256^2, P=3, FP64, SSP-RK3) on GB300",
-                    bytes_per_dof=168, bound="fp64", dtype="f64", flush_l2=True, fp64_inst_per_dof=476.0,
+                    bytes_per_dof=168, bound="fp64", dtype="f64", flush_l2=True, fp64_inst_per_dof=243.0,
                     dram_per_dof=None),
     "batch64": dict(metric="DOF updates/sec (64 batched 2-D heat problems, sides 128..2048, P=3) on GB300",
                     bytes_per_dof=156, bound="hbm", dtype="f32",
@@ -539,11 +541,11 @@ CONFIGS = {
     # the paper's own test problems (Sec. 5.1) on its 5277^2 grid: P = 1,
     # 6-point linear quadrature, forward Euler, FP64
     "paper_ex1_advection": dict(metric="DOF updates/sec (Sec. 5.1 Example 1, 2-D linear advection, 5277^2, FP64) on GB300",
-                                bytes_per_dof=40, bound="fp64", dtype="f64", fp64_inst_per_dof=54.2,
-                                dram_per_dof=41.0),
+                                bytes_per_dof=40, bound="fp64", dtype="f64", fp64_inst_per_dof=48.9,
+                                dram_per_dof=65.4),
     "paper_ex2_diffusion": dict(metric="DOF updates/sec (Sec. 5.1 Example 2, 2-D diffusion, 5277^2, FP64) on GB300",
-                                bytes_per_dof=40, bound="fp64", dtype="f64", fp64_inst_per_dof=45.6,
-                                dram_per_dof=48.0),
+                                bytes_per_dof=40, bound="fp64", dtype="f64", fp64_inst_per_dof=32.8,
+                                dram_per_dof=50.5),
     # Sec. 2.5 flux-split advection-diffusion: 2-D viscous Burgers, FP32,
     # WENO-Z, forward Euler with P = 1; per step one fused pass per axis (u in,
     # sums out), y on the transposed state, and the transposing update
@@ -551,11 +553,11 @@ CONFIGS = {
                                 # x axis 8, transpose 8, y axis 8, update (sums of both, state in and out) 16
                                 bytes_per_dof=40, bound="hbm", dtype="f32", flush_l2=True),
     "paper_ex3_hj": dict(metric="DOF updates/sec (Sec. 5.1 Example 3, 2-D Hamilton-Jacobi with source, 5277^2, FP64) on GB300",
-                         bytes_per_dof=80, bound="fp64", dtype="f64", fp64_inst_per_dof=65.2, dram_per_dof=104.4),
+                         bytes_per_dof=80, bound="fp64", dtype="f64", fp64_inst_per_dof=58.5, dram_per_dof=79.4),
 }
 # FP64-bound lines: FP64 thread-instructions (DFMA + DADD + DMUL) and DRAM bytes
-# per DOF per step from one ncu capture of the step's sweeps at 4096^2 (both
-# scale with the points); peak = the nominal 1.25 TFLOP/s FP64 rate as thread-
+# per DOF per step from one ncu capture of every launch of a step at the size
+# of the line; peak = the nominal 1.25 TFLOP/s FP64 rate as thread-
 # instructions: 2 per SM per cycle, 304 over the GPU, at the 2070 MHz maximum
 # SM clock
 FP64_PEAK_GINST = 304 * 2.070
@@ -791,10 +793,10 @@ def _hj_first_steps_error(n, seed, nsteps):
 
 
 # FP32-issue bound of the Hamilton-Jacobi WENO-Z steps: thread instructions
-# per DOF and step of the sweeps (x pass 204, y pass on the transposed state
-# 232, from one ncu capture at 4096^2) against 128 thread instructions per SM
+# per DOF and step (x pass 165, y pass on the transposed state 189, two
+# transposes 26 each, from one ncu capture at 4096^2) against 128 thread instructions per SM
 # per cycle (4 schedulers x 32 lanes) x 152 SMs x 2070 MHz
-HJ_INST_PER_DOF = 436.0
+HJ_INST_PER_DOF = 406.0
 ISSUE_PEAK_GINST = 128 * 152 * 2.070
 
 

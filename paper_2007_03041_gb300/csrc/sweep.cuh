@@ -960,7 +960,8 @@ __device__ __forceinline__ void line_scans(const LineConst& L, const LineLane<T,
 // three constants (the 3-point rule has f1 = 0).  Per point: 11 operations
 // (9 with the 3-point rule) where the two 6-tap integrals, folds, fix-ups and
 // D = v - (I_R + I_L)/2 took 20.  f0, f1 of the 5- and 6-point rules grow like
-// e^{3 nu}: a.d0 chooses this form while they stay small (set_line_constants), else the K filters.
+// e^{3 nu}: a.d0 chooses this form while they stay small (set_line_constants),
+// else the K filters.
 //
 // JQ_LINEAR1 / JQ_WENOZ1 (MODE_R or MODE_L alone): the one side that is
 // asked for, the L side as the R scan of the mirrored line.
@@ -969,7 +970,7 @@ __device__ __forceinline__ void line_scans(const LineConst& L, const LineLane<T,
 // all have the multiplier q^E, so a warp scan moves one value per lane, and a
 // line of several warps scans its warps' totals 16 lanes at a time (R in
 // lanes 0-15, L in lanes 16-31), each warp for itself: one line_sync per
-// application of D and one per write-back, no barrier for lines owned by one
+// application of D and one per write-back, no barrier for a line owned by one
 // warp.
 // GEN: MODE_RL supports every HamKind (else |grad u|^2/2 only).
 template <typename T, int JQ, bool RAGGED, int E = kE, bool GEN = false>
