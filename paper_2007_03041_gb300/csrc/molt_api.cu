@@ -1553,28 +1553,28 @@ __global__ void advdiff_update_kernel(const TC* __restrict__ acc, const TS* un, 
 
 // The last axis's sums on the transposed grid (st, x-major) with the update:
 // dst = a0 u^n + a1 (u_s + (acc + st^T)), through 64 x 64 tiles.
-__global__ void advdiff_update_t_kernel(const float* __restrict__ acc, const float* __restrict__ st, const float* un,
-                                        const float* us, float* dst, double a0, double a1, long long ny,
-                                        long long nx, int* status) {
-  __shared__ float tile[64][65];
+template <typename T>
+__global__ void advdiff_update_t_kernel(const T* __restrict__ acc, const T* __restrict__ st, const T* un, const T* us,
+                                        T* dst, double a0, double a1, long long ny, long long nx, int* status) {
+  __shared__ T tile[64][65];
   const long long x0 = (long long)blockIdx.x * 64, y0 = (long long)blockIdx.y * 64;
-  float v[16];
+  T v[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
     const long long x = x0 + threadIdx.y + 8 * (k >> 1), y = y0 + threadIdx.x + 32 * (k & 1);
-    v[k] = (x < nx && y < ny) ? st[x * ny + y] : 0.f;
+    v[k] = (x < nx && y < ny) ? st[x * ny + y] : T(0);
   }
 #pragma unroll
   for (int k = 0; k < 16; ++k) tile[threadIdx.y + 8 * (k >> 1)][threadIdx.x + 32 * (k & 1)] = v[k];
   __syncthreads();
-  float w[16], z[16];
+  T w[16], z[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
     const int j = threadIdx.y + 8 * (k >> 1), i = threadIdx.x + 32 * (k & 1);
     const long long x = x0 + i, y = y0 + j;
     if (x < nx && y < ny) {
       v[k] = acc[y * nx + x] + tile[i][j];
-      w[k] = a0 != 0.0 ? un[y * nx + x] : 0.f;
+      w[k] = a0 != 0.0 ? un[y * nx + x] : T(0);
       z[k] = us[y * nx + x];
     }
   }
@@ -1583,7 +1583,7 @@ __global__ void advdiff_update_t_kernel(const float* __restrict__ acc, const flo
   for (int k = 0; k < 16; ++k) {
     const long long x = x0 + threadIdx.x + 32 * (k & 1), y = y0 + threadIdx.y + 8 * (k >> 1);
     if (x < nx && y < ny) {
-      const float r = fmaf(float(a0), w[k], float(a1) * (z[k] + v[k]));
+      const T r = fma(T(a0), w[k], T(a1) * (z[k] + v[k]));
       dst[y * nx + x] = r;
       bad |= nonfinite(r);
     }
@@ -1592,20 +1592,22 @@ __global__ void advdiff_update_t_kernel(const float* __restrict__ acc, const flo
 }
 
 // Whether the y axis of a 2-D stage runs on the transposed state (two more
-// launches): FP32, over 2^18 points, and column tiles (W lines) whose rows fill
-// less than half of a 32-byte sector, or less than one where y lines have 2048
-// points or more.  Euler steps, WENO-Z / linear weights, us in place against
-// transposed (nx x ny): 128^2 16.9/16.7 25.4/25.3, 64 x 2048 27/22 31/28, 512^2
-// 33.2/26.1 33.7/29.5; over 2^18 points with rows of 4 and 8 bytes 600 x 1024
-// 44.0/40.1 38.1/31.5, 700^2 35.9/30.8 37.9/33.6, 1024^2 44.6/37.5 41.8/33.7,
-// 64 x 8192 58/51 45/38, 4096^2 508/412 408/317; with rows of 16 bytes 1500 x
-// 1024 50.0/38.9 61.3/49.7, 2000 x 1100 80/60 85/66, 2048^2 111/83 104/80.  FP64,
-// bound by its pipe: 128^2 83/36 95/48, 1024^2 1035/230 1046/240, 4096^2
-// 14114/3049 13935/3065.
+// launches): over 2^18 points, and column tiles (W lines) whose rows fill less
+// than a 32-byte sector where y lines have 2048 points or more, or less than
+// half of one in FP32.  Euler steps, WENO-Z / linear weights, us in place against
+// transposed (nx x ny).  FP32: 128^2 16.9/16.7 25.4/25.3, 64 x 2048 27/22 31/28,
+// 512^2 33.2/26.1 33.7/29.5; over 2^18 points with rows of 4 and 8 bytes 600 x
+// 1024 44.0/40.1 38.1/31.5, 700^2 35.9/30.8 37.9/33.6, 1024^2 44.6/37.5
+// 41.8/33.7, 64 x 8192 58/51 45/38, 4096^2 508/412 408/317; with rows of 16 bytes
+// 1500 x 1024 50.0/38.9 61.3/49.7, 2000 x 1100 80/60 85/66, 2048^2 111/83 104/80.
+// FP64, bound by its pipe: 128^2 83/36 95/48, 300 x 1024 406/105 413/113, 1024^2
+// 1035/230 1046/240, 700 x 1536 1190/291 1201/301, 300 x 2048 786/195 796/202, 600 x
+// 2500 1570/414 1582/398, 64 x 8192 1039/277 1030/267, 1000 x 3000 2851/661
+// 2671/629, 1024 x 4096 3858/886 3626/851, 4096^2 14114/3049 13935/3065.
 bool transposed_y(const Problem& p, int W) {
   const int row = W * int(state_bytes(p.d));
-  return !is_f64_sweep(p.d) && p.total > (1LL << 18) &&
-         (row < kStridedRowBytes / 2 || (row < kStridedRowBytes && p.n[1] >= 2048));
+  return p.total > (1LL << 18) && ((row < kStridedRowBytes && p.n[1] >= 2048) ||
+                                   (!is_f64_sweep(p.d) && row < kStridedRowBytes / 2));
 }
 
 // The fused axis kernel takes stages with one term per sum on uniform axes
@@ -1669,9 +1671,14 @@ molt_status advdiff_stage_fused(molt_ctx* c, Problem& p, const void* un, const v
         molt_ctx::Rec rec;
         record_begin(c, &rec, MOLT_KERNEL_UPDATE);
         const dim3 grid(unsigned((nx + 63) / 64), unsigned((ny + 63) / 64)), block(32, 8);
-        advdiff_update_t_kernel<<<grid, block, 0, c->stream>>>(
-            static_cast<const float*>(p.acc), static_cast<const float*>(p.gm), static_cast<const float*>(un),
-            static_cast<const float*>(us), static_cast<float*>(dst), a0, a1, ny, nx, c->status_dev);
+        if (f64)
+          advdiff_update_t_kernel<double><<<grid, block, 0, c->stream>>>(
+              static_cast<const double*>(p.acc), static_cast<const double*>(p.gm), static_cast<const double*>(un),
+              static_cast<const double*>(us), static_cast<double*>(dst), a0, a1, ny, nx, c->status_dev);
+        else
+          advdiff_update_t_kernel<float><<<grid, block, 0, c->stream>>>(
+              static_cast<const float*>(p.acc), static_cast<const float*>(p.gm), static_cast<const float*>(un),
+              static_cast<const float*>(us), static_cast<float*>(dst), a0, a1, ny, nx, c->status_dev);
         record_end(c, &rec);
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "advection-diffusion update");
         continue;

@@ -1,7 +1,7 @@
 """The fused advection-diffusion axis kernel against the oracle at the edges
 of its shapes: lines around lane, warp and tile ends, one to three axes, no
 diffusion, both integrators.  In 2-D the y axis runs on column tiles in place,
-that of larger FP32 grids whose tiles have narrow rows on the transposed state:
+that of larger grids whose tiles have narrow rows on the transposed state:
 ROUTES has both sides of that rule, and the unmasked kernel of 16 points a lane
 in both precisions."""
 import numpy as np
@@ -58,6 +58,8 @@ ROUTES = [
     ((1024, 1500), F32, WZ, 5, False),     # rows of 16 bytes
     ((2048, 1500), F32, LIN, 6, True),     # the same, long lines
     ((8192, 129), F32, WZ, 5, True),       # the longest lines
+    ((2048, 150), F64, LIN, 6, True),      # FP64: long lines only
+    ((2047, 150), F64, WZ, 5, False),
     ((11, 20, 35), F32, WZ, 5, None),      # 3-D: column tiles along y and z
     ((10, 33, 18), F64, WZ, 5, None),
     ((9, 64, 128), F64, LIN, 6, None),
