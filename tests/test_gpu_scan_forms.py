@@ -48,6 +48,24 @@ def test_wenoz_line_edges(prec, bc, op):
         check(got, want, prec, 2, 0, n)
 
 
+@pytest.mark.parametrize("prec", [M.PREC_F64, M.PREC_F32])
+@pytest.mark.parametrize("n,W", [(1000, 4), (1024, 4), (1100, 2), (1536, 2), (2048, 2)])
+def test_tiles_of_several_lines_of_several_warps(prec, n, W):
+    """Enough lines that a CTA holds 2 or 4 lines of 2 to 4 warps, whose
+    barriers it shares or keeps apart; the last tile is partly empty."""
+    lines = 1301
+    plan = M.molt_plan_sweep(M.make_desc((n, lines), prec=prec), 0, M.OP_0, 2, 0.3 * n)
+    assert (plan["points_per_lane"], plan["lines_per_cta"]) == (16, W) and plan["warps_per_line"] > 1
+    for k, bc in enumerate((M.BC_PERIODIC, M.BC_DIRICHLET)):
+        got, want = run_apply((lines, n), 0, M.OP_0, 2, 0.3, bc, 6, prec, seed=n + k)
+        check(got, want, prec, 2, 0, (n, "rows"))
+        got, want = run_apply((n, lines), 1, (M.OP_R, M.OP_L)[k], 2, 0.3, bc, 6, prec, seed=n + k)
+        check(got, want, prec, 2, 1, (n, "columns"))
+    if prec == M.PREC_F32:
+        got, want = run_apply((lines, n), 0, M.OP_0, 1, 2.0 / 3.0, M.BC_PERIODIC, 5, prec, weights=M.W_WENOZ, seed=n)
+        check(got, want, prec, 2, 0, (n, "WENO-Z rows"))
+
+
 @pytest.mark.parametrize("npts", [3, 5, 6])
 @pytest.mark.parametrize("n", [500, 512])
 def test_symbol_of_D0_in_fp32(n, npts):
